@@ -300,6 +300,7 @@ struct Pair {
     int fdepth, mdepth;
     int mdtype;  // stored moving type: 0 u8, 1 u16
     long long nvf, nvm;
+    long long nsampled = 0;     // sampled fixed voxels (random sampling only)
     DevBuf fbins, mov, movp;    // hard path (movp: x-paired moving volume)
     cudaArray_t arr = nullptr;  // the pairs as a 3D array, read through tex
     cudaTextureObject_t tex = 0;
@@ -356,8 +357,11 @@ struct mi_ctx {
     // per-q FP64 tables, keyed by the float bits of q
     std::map<uint32_t, std::unique_ptr<DevBuf>> tables;
     // call scratch
-    DevBuf d_aff, d_items, d_mi, d_h, d_cnt, d_hist, d_flags, d_ticket, d_dump, d_cols, d_part;
-    HostBuf h_aff, h_items, h_out, h_read;
+    // (d_in: affines, work items and slots of a call, staged in h_in or v_in; d_work: the zeroed workspace of a
+    // launch: ticket, slot counters, slot histograms; d_part: partial entropy sums)
+    DevBuf d_aff, d_in, d_mi, d_h, d_cnt, d_flags, d_work, d_part, d_dump;
+    HostBuf h_in, h_read;
+    std::vector<char> v_in;  // the same staging where no graph replays it
     // Parzen: the pairs' descriptors (device array), per-call pair indices and row offsets, scratch
     DevBuf p_pairs, p_pair_of, p_row_start;
     int p_bmax = 0, p_nxmax = 0;
@@ -452,6 +456,8 @@ int effective_depth(const mi_volume *v) {
     return v->bit_depth == 0 ? full : v->bit_depth;
 }
 
+size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+
 size_t dtype_size(int dt) { return dt == MI_U8 ? 1 : (dt == MI_U16 ? 2 : 4); }
 
 // Copy a caller volume (host or device) into a fresh device buffer.
@@ -484,6 +490,7 @@ mi_status build_samples(mi_ctx *ctx, Pair &P, const uint8_t *fb, cudaStream_t s)
         acc += cnt[(size_t)r];
     }
     ptr[(size_t)R] = (uint32_t)acc;
+    P.nsampled = (long long)acc;
     MI_CU(P.srow.ensure(((size_t)R + 1) * 4), "allocating sample rows");
     MI_CU(P.scol.ensure(std::max<size_t>((size_t)acc * 2, 2)), "allocating sample columns");
     MI_CU(P.sbin.ensure(std::max<size_t>((size_t)acc, 1)), "allocating sample bins");
@@ -911,7 +918,6 @@ mi_status create_common(mi_ctx **out, const mi_volume *fixed, const mi_volume *m
             return st;
         }
         MI_CU(ctx->d_flags.ensure(2 * sizeof(int)), "allocating flags");
-        MI_CU(ctx->d_ticket.ensure(2 * sizeof(int)), "allocating the ticket");  // ticket, sweep phase
     }
     *out = ctx.release();
     return MI_OK;
@@ -963,6 +969,10 @@ mi_status make_qset(mi_ctx *ctx, const float *qv, int nq, QSet &Q) {
     Q.bits = ctx->opt.log_bits ? 1 : 0;
     for (int i = 0; i < nq; ++i) {
         Q.q[i] = qv[i];
+        const double q = (double)qv[i];
+        Q.c2[i] = q * (q - 1.0) / 2.0;
+        Q.c3[i] = q * (q - 1.0) * (q - 2.0) / 6.0;
+        Q.inv_q1[i] = q == 1.0 ? 0.0 : 1.0 / (q - 1.0);
         if (ctx->opt.kernel == MI_HARD) {
             auto it = ctx->tables.find(fbits(qv[i]));
             if (it == ctx->tables.end()) {
@@ -1061,65 +1071,102 @@ std::vector<Choice> candidates(mi_ctx *ctx, int bins, long long nvox_max) {
     return c;
 }
 
-// ---------------------------------------------------------------------------
-// Plain path: many CTAs per transform, global histograms, then the entropy kernel
-// ---------------------------------------------------------------------------
+// The plain path's variant (it is not autotuned): the first of these kinds that fits, 1024 threads.  A few
+// transforms wait for the moving volume's first use, where the gather atlas is half the quads' bytes; from
+// kPlainQuads on its reuse weighs more and the quads' fewer instructions win.  A lone transform's parts are
+// a dozen rows a warp, whose ends the stream walk packs; more take two rows a step.  128 bins, 256 x 256 x
+// 160, us: one transform 72 (gather, stream), 74 (two rows), above 79 (quads); 8: 288 gather, 300 quads;
+// 24: 705 and 690; 81: 2201 and 2035.
+constexpr int kPlainQuads = 24, kPlainRows = 4;
 
-mi_status run_plain(mi_ctx *ctx, int pair, const int32_t *d_aff, int n, const QSet &Q, const Outputs &O,
-                    const Choice &ch, uint32_t *keep_hist) {
-    const Pair &P = *ctx->pairs[pair];
-    const PairDev hp = host_pairdev(P);
-    const PairDev *dp = ctx->d_pairs.as<PairDev>() + pair;
-    const size_t B2 = (size_t)P.bins * P.bins;
-    int chunk = (int)std::max<size_t>(1, (64u << 20) / (B2 * 4));
-    chunk = std::min(chunk, 4096);
-    MI_CU(cudaEventRecord(ctx->ev0, ctx->stream), "event");
-    ctx->last_launches = 0;
-    for (int t0 = 0; t0 < n; t0 += chunk) {
-        const int m = std::min(chunk, n - t0);
-        uint32_t *hist = keep_hist ? keep_hist + (size_t)t0 * B2 : nullptr;
-        if (!hist) {
-            MI_CU(ctx->d_hist.ensure((size_t)m * B2 * 4), "allocating histograms");
-            hist = ctx->d_hist.as<uint32_t>();
-        }
-        // CTAs per transform: fill the GPU, but keep at least 8 row batches of 32 rows per CTA
-        const long long rows = (long long)P.nf[1] * P.nf[2];
-        const int per_sm =
-            std::max(1, batched_ctas_per_sm(ch.variant, P.bins, ch.threads, P.rows_words, P.nm[2]));
-        long long ctas = ((long long)ctx->sms * per_sm + m - 1) / m;
-        ctas = std::min<long long>(ctas, std::max<long long>(1, rows / (32 * 8)));
-        MI_CU(launch_plain_hist(dp, hp, d_aff + (size_t)t0 * 12, m, hist, ch.variant, ch.threads, (int)std::max(1LL, ctas),
-                                ch.tile, O.flags, ctx->stream),
-              "plain histogram kernel");
-        if (O.mi || O.h || O.count) {
-            Outputs Oc = O;
-            if (Oc.mi) Oc.mi += (size_t)t0 * Q.nq;
-            if (Oc.h) Oc.h += (size_t)t0 * Q.nq * 3;
-            if (Oc.count) Oc.count += t0;
-            Oc.dump = nullptr;
-            if (m < ctx->sms) {
-                // few transforms: the reduction of each histogram is split over several CTAs
-                MI_CU(ctx->d_cols.ensure((size_t)m * P.bins * 4), "allocating column sums");
-                MI_CU(ctx->d_part.ensure((size_t)m * entropy_parts(P.bins) * (1 + 2 * kMaxQ) * 8),
-                      "allocating partial sums");
-                MI_CU(launch_entropy_split(hist, m, P.bins, Q, Oc, ctx->d_cols.as<uint32_t>(), ctx->d_part.as<double>(),
-                                           ctx->stream),
-                      "entropy kernels");
-                ctx->last_launches += 2;
-            } else {
-                MI_CU(launch_entropy(hist, m, P.bins, Q, Oc, ctx->stream), "entropy kernel");
-                ctx->last_launches += 1;
-            }
-        }
-        ctx->last_launches += 1;
+Choice plain_choice(mi_ctx *ctx, const std::vector<Choice> &cands, int n) {
+    const int gather[] = {HV_U32_GATHER, HV_ROWS_GATHER, HV_U16_GATHER, HV_U32_QUAD, HV_ROWS_QUAD, HV_U16_QUAD,
+                          HV_U32, HV_U16};
+    const int quads[] = {HV_U32_QUAD, HV_ROWS_QUAD, HV_U16_QUAD, HV_U32, HV_U16};
+    const bool many = n >= kPlainQuads;
+    const int lpr = n >= kPlainRows ? 4 : 0;
+    for (const int *v = many ? quads : gather, *end = many ? std::end(quads) : std::end(gather); v != end; ++v) {
+        if (hv_kind(*v) == HV_U32 && ctx->max_bins > 181) continue;
+        for (const Choice &c : cands)
+            if (c.variant == *v && (c.threads == 1024 || ctx->opt.block_threads) &&
+                (hv_fetch(*v) < FM_QUAD || ctx->opt.tile_rows || c.tile.lpr_log2 == lpr))
+                return c;
     }
-    MI_CU(cudaEventRecord(ctx->ev1, ctx->stream), "event");
-    return MI_OK;
+    return cands.front();
 }
 
+// How the plain path's choices are kept: by the rule's ranges of the transform count.
+int plain_bucket(int n) { return n >= kPlainQuads ? 2 : n >= kPlainRows ? 1 : 0; }
+
 // ---------------------------------------------------------------------------
-// Batched path: persistent kernel over a work queue, replayed as a CUDA graph
+// Work items of a call
 // ---------------------------------------------------------------------------
+
+struct HardPlan {
+    std::vector<Item> items;  // in ticket order
+    std::vector<Slot> slots;  // transforms whose histogram is summed in global memory
+};
+
+enum PlanMode {
+    kPlanWhole,  // one item per transform, reduced in place
+    kPlanTail,   // as few split transforms as balance the CTAs, the others whole
+    kPlanSlots   // every transform through a slot (the plain path), split to fill the GPU
+};
+
+// Appends the items of transforms t0 .. t0 + m - 1.  CTAs take items in order, each as it finishes its
+// last one, so with whole transforms alone a call ends on its last wave: 400 transforms on 304 resident
+// CTAs took the time of 608 and 81 transforms at two CTAs each on 152 that of 152 at one.  So the
+// transforms are taken largest first and each is cut into as many parts as keep a part below half of the
+// CTAs' mean share of what is left: all but the last ~2 P of many equal transforms stay whole
+// (P = CTAs resident at once).  A part costs its CTA the clearing and flushing of a histogram, about
+// bins^2 / 8 + 2000 voxels' time, so parts stay eight times that; a call too small for such parts
+// (below 32 of them a CTA) is cut once into equal parts, one for every CTA.
+// Against whole transforms (batched) and equal CTA counts per transform (plain), kernel times: 81 transforms on
+// 256 x 256 x 160 at 128 bins 4320 -> 1945 us, 400 sampled ones 3875 -> 2710, 768 on twelve pairs of 96^3 to
+// 320 x 320 x 200 16490 -> 13400.
+void plan_items(const mi_ctx *ctx, const std::vector<int> &pair_of, int t0, int m, const Choice &ch, PlanMode mode,
+                HardPlan &plan) {
+    const int P = std::max(1, ch.ctas), nwarps = ch.threads / 32;
+    auto cost = [&](int pair) {
+        const Pair &p = *ctx->pairs[pair];
+        return (double)(p.srow.p ? std::max(1LL, p.nsampled) : p.nvf);
+    };
+    auto overhead = [&](int pair) { return (double)ctx->pairs[pair]->bins * ctx->pairs[pair]->bins / 8.0 + 2000.0; };
+    std::vector<int> order(m);
+    for (int i = 0; i < m; ++i) order[i] = t0 + i;
+    if (!pair_of.empty())
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int a, int b) { return ctx->pairs[pair_of[a]]->nvf > ctx->pairs[pair_of[b]]->nvf; });
+    double left = 0.0, over = 0.0;
+    for (int t : order) {
+        const int pair = pair_of.empty() ? 0 : pair_of[t];
+        left += cost(pair);
+        over = std::max(over, overhead(pair));
+    }
+    const double total = left;
+    const bool once = m <= P && total < 32.0 * over * P;
+    const size_t slot0 = plan.slots.size();
+    for (int t : order) {
+        const int pair = pair_of.empty() ? 0 : pair_of[t];
+        const Pair &p = *ctx->pairs[pair];
+        const double c = cost(pair);
+        double parts = 1.0;
+        if (mode != kPlanWhole) {
+            parts = once ? floor(c * P / total) : std::min(ceil(2.0 * c * P / left), floor(c / (8.0 * overhead(pair))));
+            const long long blocks = ((long long)p.nf[1] * p.nf[2] + nwarps - 1) / nwarps;
+            parts = std::max(1.0, std::min({parts, (double)P, (double)blocks, 65535.0}));
+        }
+        left -= c;
+        const int k = (int)parts;
+        int slot = -1;
+        if (k > 1 || mode == kPlanSlots) {
+            slot = (int)(plan.slots.size() - slot0);
+            plan.slots.push_back(Slot{t, p.bins});
+        }
+        for (int i = 0; i < k; ++i)
+            plan.items.push_back(Item{pair, t, (unsigned short)i, (unsigned short)k, slot});
+    }
+}
 
 // Event record that also fires when replayed from a captured graph (external
 // event node while the stream is capturing, a plain record otherwise).
@@ -1131,15 +1178,14 @@ cudaError_t record_event(cudaEvent_t ev, cudaStream_t s) {
                                                : cudaEventRecord(ev, s);
 }
 
-mi_status launch_batched_once(mi_ctx *ctx, int nitems, const QSet &Q, const Outputs &O, const Choice &ch,
-                              bool record = false) {
-    MI_CU(cudaMemsetAsync(ctx->d_ticket.p, 0, 2 * sizeof(int), ctx->stream), "resetting the work queue");
-    if (record) MI_CU(record_event(ctx->ev0, ctx->stream), "event");
-    MI_CU(launch_batched(ctx->d_pairs.as<PairDev>(), ctx->d_aff.as<int32_t>(), ctx->d_items.as<Item>(), nitems,
-                         ctx->d_ticket.as<int>(), ctx->max_bins, ctx->max_rows_words, ctx->max_zplanes, ch.variant,
-                         ch.threads, ch.ctas, ch.tile, Q, O, ctx->stream),
+// One launch of the hard-path kernel over whole items (the autotuner's unit).
+mi_status launch_whole(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, const QSet &Q,
+                       const Outputs &O, const Choice &ch) {
+    MI_CU(cudaMemsetAsync(ctx->d_work.p, 0, 2 * sizeof(int), ctx->stream), "resetting the work queue");
+    MI_CU(launch_batched(ctx->d_pairs.as<PairDev>(), d_aff, d_items, nitems, ctx->d_work.as<int>(), ctx->max_bins,
+                         ctx->max_rows_words, ctx->max_zplanes, ch.variant, ch.threads, ch.ctas, ch.tile, Q, O, nullptr,
+                         0, ctx->stream),
           "batched kernel");
-    if (record) MI_CU(record_event(ctx->ev1, ctx->stream), "event");
     return MI_OK;
 }
 
@@ -1224,8 +1270,8 @@ void cache_store(const std::string &path, const std::string &key, const Choice &
 // Autotune: time every candidate on the first items of this call (up to three
 // waves, so that effects that build up across waves, such as CTAs drifting to
 // different parts of the volumes, show in the timing).
-mi_status autotune(mi_ctx *ctx, int nitems, const QSet &Q, const Outputs &O, Choice &best,
-                   const std::vector<Choice> &cands) {
+mi_status autotune(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, const QSet &Q, const Outputs &O,
+                   Choice &best, const std::vector<Choice> &cands) {
     if (cands.empty()) return ctx->fail(MI_EUNSUPPORTED, "no histogram variant fits this bin count and volume size");
     if (cands.size() == 1 || !ctx->opt.autotune) {
         best = cands.front();
@@ -1245,7 +1291,7 @@ mi_status autotune(mi_ctx *ctx, int nitems, const QSet &Q, const Outputs &O, Cho
     auto time_per_item = [&](const Choice &c, int items, float &ms) -> mi_status {
         Choice cc = c;
         cudaEventRecord(e0, ctx->stream);
-        mi_status st = launch_batched_once(ctx, items, Q, Ot, cc);
+        mi_status st = launch_whole(ctx, d_aff, d_items, items, Q, Ot, cc);
         if (st != MI_OK) return st;
         cudaEventRecord(e1, ctx->stream);
         cudaError_t e = cudaEventSynchronize(e1);
@@ -1258,7 +1304,7 @@ mi_status autotune(mi_ctx *ctx, int nitems, const QSet &Q, const Outputs &O, Cho
     mi_status st = MI_OK;
     for (size_t i = 0; i < cands.size() && st == MI_OK; ++i) {
         Choice cc = cands[i];
-        if ((st = launch_batched_once(ctx, std::min(nitems, 8), Q, Ot, cc)) != MI_OK) break;  // warm-up
+        if ((st = launch_whole(ctx, d_aff, d_items, std::min(nitems, 8), Q, Ot, cc)) != MI_OK) break;  // warm-up
         float ms = 0;
         if ((st = time_per_item(cands[i], std::min(nitems, cands[i].ctas), ms)) == MI_OK) first.push_back({ms, i});
     }
@@ -1277,42 +1323,6 @@ mi_status autotune(mi_ctx *ctx, int nitems, const QSet &Q, const Outputs &O, Cho
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return st;
-}
-
-mi_status run_batched(mi_ctx *ctx, int nitems, const QSet &Q, const Outputs &O, const Choice &ch, bool use_graph,
-                      const std::string &key, const void *h_aff_src, size_t aff_bytes, const void *h_items_src,
-                      size_t item_bytes) {
-    // inputs go through pinned staging so that a captured graph can replay the copies
-    MI_CU(ctx->h_aff.ensure(aff_bytes), "pinned staging");
-    MI_CU(ctx->h_items.ensure(item_bytes), "pinned staging");
-    memcpy(ctx->h_aff.p, h_aff_src, aff_bytes);
-    memcpy(ctx->h_items.p, h_items_src, item_bytes);
-    if (!use_graph) {
-        MI_CU(cudaMemcpyAsync(ctx->d_aff.p, ctx->h_aff.p, aff_bytes, cudaMemcpyHostToDevice, ctx->stream), "H2D");
-        MI_CU(cudaMemcpyAsync(ctx->d_items.p, ctx->h_items.p, item_bytes, cudaMemcpyHostToDevice, ctx->stream), "H2D");
-        return launch_batched_once(ctx, nitems, Q, O, ch, true);
-    }
-    auto it = ctx->graphs.find(key);
-    if (it == ctx->graphs.end()) {
-        // set kernel attributes outside of capture
-        batched_ctas_per_sm(ch.variant, ctx->max_bins, ch.threads, ctx->max_rows_words, ctx->max_zplanes);
-        cudaGraph_t g;
-        MI_CU(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeRelaxed), "begin capture");
-        cudaMemcpyAsync(ctx->d_aff.p, ctx->h_aff.p, aff_bytes, cudaMemcpyHostToDevice, ctx->stream);
-        cudaMemcpyAsync(ctx->d_items.p, ctx->h_items.p, item_bytes, cudaMemcpyHostToDevice, ctx->stream);
-        mi_status st = launch_batched_once(ctx, nitems, Q, O, ch, true);
-        cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
-        if (st != MI_OK) return st;
-        if (e != cudaSuccess) return ctx->cuda_fail(e, "end capture");
-        auto ge = std::make_unique<GraphEntry>();
-        e = cudaGraphInstantiate(&ge->exec, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return ctx->cuda_fail(e, "instantiating the graph");
-        if (ctx->graphs.size() > 32) ctx->graphs.clear();
-        it = ctx->graphs.emplace(key, std::move(ge)).first;
-    }
-    MI_CU(cudaGraphLaunch(it->second->exec, ctx->stream), "graph launch");
-    return MI_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1337,7 +1347,6 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     MI_CU(ctx->d_mi.ensure((size_t)n * nq * 8), "allocating outputs");
     MI_CU(ctx->d_h.ensure((size_t)n * nq * 3 * 8), "allocating outputs");
     MI_CU(ctx->d_cnt.ensure((size_t)n * 8), "allocating outputs");
-    MI_CU(ctx->d_aff.ensure((size_t)n * 12 * 4), "allocating affines");
     MI_CU(cudaMemsetAsync(ctx->d_flags.p, 0, 2 * sizeof(int), ctx->stream), "resetting flags");
     Outputs O;
     O.mi = ctx->d_mi.as<double>();
@@ -1349,98 +1358,150 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     int path = R.path;
     if (path == MI_PATH_AUTO) path = (multi || n >= ctx->sms) ? MI_PATH_BATCHED : MI_PATH_PLAIN;
     if (multi && path == MI_PATH_PLAIN) return ctx->fail(MI_EINVAL, "multi-pair contexts use the batched path");
+    const bool plain = path == MI_PATH_PLAIN;
     long long nvox_max = 0;
     for (auto &p : ctx->pairs) nvox_max = std::max(nvox_max, p->nvf);
     std::vector<Choice> cands = candidates(ctx, ctx->max_bins, nvox_max);
     if (cands.empty()) return ctx->fail(MI_EUNSUPPORTED, "no histogram variant fits this bin count and volume size");
-    if (path == MI_PATH_PLAIN) {
-        const int32_t *d_aff = R.d_q16;
-        if (!d_aff) {
-            MI_CU(cudaMemcpyAsync(ctx->d_aff.p, R.q16.data(), (size_t)n * 48, cudaMemcpyHostToDevice, ctx->stream), "H2D");
-            d_aff = ctx->d_aff.as<int32_t>();
-        }
-        auto key = std::make_tuple((int)MI_PATH_PLAIN, 0, 0);
-        Choice ch;
-        auto it = ctx->tuned.find(key);
-        if (it != ctx->tuned.end()) {
-            ch = it->second;
-        } else {
-            // heuristic (the plain form is not autotuned): the first of these kinds that fits, with
-            // 1024 threads and the stream walk where the fetch allows it
-            const int order[] = {HV_U32_GATHER, HV_ROWS_GATHER, HV_U16_GATHER, HV_U32_QUAD, HV_ROWS_QUAD,
-                                 HV_U16_QUAD, HV_U32, HV_U16};
-            ch = cands.front();
-            bool found = false;
-            for (int v : order) {
-                if (v == HV_U32_GATHER || v == HV_U32_QUAD || v == HV_U32)
-                    if (ctx->max_bins > 181) continue;
-                for (const Choice &c : cands)
-                    if (c.variant == v && c.threads == 1024 && (c.tile.lpr_log2 == 0 || hv_fetch(v) < FM_QUAD)) {
-                        ch = c;
-                        found = true;
-                        break;
-                    }
-                if (found) break;
-            }
-            ctx->tuned[key] = ch;
-        }
-        st = run_plain(ctx, 0, d_aff, n, Q, O, ch, R.dump);
-        if (st != MI_OK) return st;
-        ctx->timed = true;
+    const int bucket = plain ? plain_bucket(n) : n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0);
+    auto key = std::make_tuple(path, plain ? 0 : -1, bucket);
+    Choice ch;
+    auto it = ctx->tuned.find(key);
+    if (it != ctx->tuned.end()) {
+        ch = it->second;
+    } else if (plain) {
+        ch = plain_choice(ctx, cands, n);
+        ctx->tuned[key] = ch;
     } else {
-        // work items sorted by cost (voxels of the pair), largest first
-        std::vector<Item> items(n);
-        for (int t = 0; t < n; ++t) items[t] = Item{R.pair_of.empty() ? 0 : R.pair_of[t], t};
-        if (multi)
-            std::stable_sort(items.begin(), items.end(), [&](const Item &a, const Item &b) {
-                return ctx->pairs[a.pair]->nvf > ctx->pairs[b.pair]->nvf;
-            });
-        MI_CU(ctx->d_items.ensure((size_t)n * sizeof(Item)), "allocating items");
-        std::vector<int32_t> q16h;
-        const int32_t *h_aff = R.q16.data();
-        if (R.d_q16) {
-            q16h.resize((size_t)n * 12);
-            if ((st = read_from_device(ctx, q16h.data(), R.d_q16, (size_t)n * 48)) != MI_OK) return st;
-            h_aff = q16h.data();
+        const std::string cpath = ctx->opt.autotune && cands.size() > 1 ? cache_path() : std::string();
+        const std::string ckey = cpath.empty() ? std::string() : tune_key(ctx, bucket, nq);
+        if (cpath.empty() || !cache_lookup(cpath, ckey, cands, ch)) {
+            // tuning needs the affines and whole items on the device
+            HardPlan whole;
+            plan_items(ctx, R.pair_of, 0, n, cands.front(), kPlanWhole, whole);
+            const size_t aff_bytes = align256((size_t)n * 48), item_bytes = (size_t)n * sizeof(Item);
+            MI_CU(ctx->d_in.ensure(aff_bytes + item_bytes), "allocating the call's inputs");
+            MI_CU(ctx->d_work.ensure(256), "allocating the ticket");
+            MI_CU(cudaMemcpyAsync(ctx->d_in.p, R.d_q16 ? R.d_q16 : R.q16.data(), (size_t)n * 48, cudaMemcpyDefault,
+                                  ctx->stream),
+                  "affines");
+            const Item *d_items = (const Item *)(ctx->d_in.as<char>() + aff_bytes);
+            MI_CU(cudaMemcpyAsync((void *)d_items, whole.items.data(), item_bytes, cudaMemcpyHostToDevice, ctx->stream),
+                  "H2D");
+            st = autotune(ctx, ctx->d_in.as<int32_t>(), d_items, n, Q, O, ch, cands);
+            if (st != MI_OK) return st;
+            MI_CU(cudaMemsetAsync(ctx->d_flags.p, 0, 2 * sizeof(int), ctx->stream), "resetting flags");
+            if (!cpath.empty()) cache_store(cpath, ckey, ch);
         }
-        const int bucket = n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0);
-        auto key = std::make_tuple((int)MI_PATH_BATCHED, -1, bucket);
-        Choice ch;
-        auto it = ctx->tuned.find(key);
-        if (it != ctx->tuned.end()) {
-            ch = it->second;
-        } else {
-            const std::string cpath = ctx->opt.autotune && cands.size() > 1 ? cache_path() : std::string();
-            const std::string ckey = cpath.empty() ? std::string() : tune_key(ctx, bucket, nq);
-            if (cpath.empty() || !cache_lookup(cpath, ckey, cands, ch)) {
-                // tuning needs the inputs on the device
-                MI_CU(cudaMemcpyAsync(ctx->d_aff.p, h_aff, (size_t)n * 48, cudaMemcpyHostToDevice, ctx->stream),
-                      "H2D");
-                MI_CU(cudaMemcpyAsync(ctx->d_items.p, items.data(), (size_t)n * sizeof(Item), cudaMemcpyHostToDevice,
-                                      ctx->stream),
-                      "H2D");
-                st = autotune(ctx, n, Q, O, ch, cands);
-                if (st != MI_OK) return st;
-                MI_CU(cudaMemsetAsync(ctx->d_flags.p, 0, 2 * sizeof(int), ctx->stream), "resetting flags");
-                if (!cpath.empty()) cache_store(cpath, ckey, ch);
-            }
-            ctx->tuned[key] = ch;
+        ctx->tuned[key] = ch;
+    }
+
+    // The plain path sums every histogram in global memory, in chunks of at most 64 MB of them; the
+    // batched path reduces whole transforms in place and splits the last ones, unless the caller asked
+    // for the batched path of a single pair by name or wants the histograms themselves.
+    const size_t B2 = (size_t)ctx->max_bins * ctx->max_bins;
+    const PlanMode mode = plain ? kPlanSlots
+                          : !R.dump && (multi || R.path == MI_PATH_AUTO) ? kPlanTail : kPlanWhole;
+    const int chunk = plain ? (int)std::min<size_t>(4096, std::max<size_t>(1, (64u << 20) / (B2 * 4))) : n;
+    struct Range {
+        int t0, m;
+        size_t item0, nitems, slot0, nslots;
+    };
+    std::vector<Range> ranges;
+    HardPlan plan;
+    size_t max_slots = 0;
+    for (int t0 = 0; t0 < n; t0 += chunk) {
+        Range r{t0, std::min(chunk, n - t0), plan.items.size(), 0, plan.slots.size(), 0};
+        plan_items(ctx, R.pair_of, t0, r.m, ch, mode, plan);
+        r.nitems = plan.items.size() - r.item0;
+        r.nslots = plan.slots.size() - r.slot0;
+        max_slots = std::max(max_slots, r.nslots);
+        ranges.push_back(r);
+    }
+    const size_t aff_bytes = align256((size_t)n * 48), items_at = aff_bytes,
+                 slots_at = items_at + align256(plan.items.size() * sizeof(Item)),
+                 in_bytes = slots_at + plan.slots.size() * sizeof(Slot);
+    const size_t done_at = 256, hist_at = done_at + align256(max_slots * 4);
+    const bool own_hist = !(plain && R.dump);
+    const size_t work_bytes = hist_at + (own_hist ? max_slots * B2 * 4 : 0);
+    MI_CU(ctx->d_in.ensure(in_bytes), "allocating the call's inputs");
+    MI_CU(ctx->d_work.ensure(work_bytes), "allocating the workspace");
+    if (max_slots)
+        MI_CU(ctx->d_part.ensure(entropy_part_bytes((ctx->max_bins + 7) / 8, (int)max_slots)), "allocating partial sums");
+    cudaStream_t s = ctx->stream;
+    // A batched call is replayed as a CUDA graph, so its inputs go through pinned staging.  The plain path
+    // takes a few launches a call: capturing and instantiating would cost a first call more than it saves.
+    const bool use_graph = !plain && ctx->opt.use_graphs && !R.dump && s != nullptr;
+    char *staged;
+    if (use_graph) {
+        MI_CU(ctx->h_in.ensure(in_bytes), "pinned staging");
+        staged = ctx->h_in.as<char>();
+    } else {
+        ctx->v_in.resize(in_bytes);
+        staged = ctx->v_in.data();
+    }
+    if (!R.d_q16) memcpy(staged, R.q16.data(), (size_t)n * 48);
+    memcpy(staged + items_at, plan.items.data(), plan.items.size() * sizeof(Item));
+    if (!plan.slots.empty()) memcpy(staged + slots_at, plan.slots.data(), plan.slots.size() * sizeof(Slot));
+    if (R.d_q16)
+        MI_CU(cudaMemcpyAsync(ctx->d_in.p, R.d_q16, (size_t)n * 48, cudaMemcpyDeviceToDevice, s), "copying the affines");
+    auto enqueue = [&]() -> mi_status {
+        const size_t from = R.d_q16 ? items_at : 0;
+        char *in = ctx->d_in.as<char>(), *work = ctx->d_work.as<char>();
+        MI_CU(cudaMemcpyAsync(in + from, staged + from, in_bytes - from, cudaMemcpyHostToDevice, s), "H2D");
+        MI_CU(record_event(ctx->ev0, s), "event");
+        for (const Range &r : ranges) {
+            uint32_t *hist = own_hist ? (uint32_t *)(work + hist_at) : R.dump + (size_t)r.t0 * B2;
+            MI_CU(cudaMemsetAsync(work, 0, hist_at + (own_hist ? r.nslots * B2 * 4 : 0), s), "clearing the workspace");
+            if (!own_hist) MI_CU(cudaMemsetAsync(hist, 0, r.nslots * B2 * 4, s), "clearing histograms");
+            MI_CU(launch_batched(ctx->d_pairs.as<PairDev>(), (const int32_t *)in, (const Item *)(in + items_at) + r.item0,
+                                 (int)r.nitems, (int *)work, ctx->max_bins, ctx->max_rows_words, ctx->max_zplanes,
+                                 ch.variant, ch.threads, ch.ctas, ch.tile, Q, O, hist, (long long)B2, s),
+                  "histogram kernel");
+            if (r.nslots)
+                MI_CU(launch_entropy_slots(hist, (long long)B2, (const Slot *)(in + slots_at) + r.slot0, (int)r.nslots,
+                                           entropy_parts(ctx->max_bins, (int)r.nslots, ctx->sms), Q,
+                                           (unsigned *)(work + done_at), ctx->d_part.as<double>(), O, s),
+                      "entropy kernel");
         }
-        const bool use_graph = ctx->opt.use_graphs && !R.dump && ctx->stream != nullptr;
-        // staging buffers are sized before the key is formed: a graph replays copies from their addresses
-        MI_CU(ctx->h_aff.ensure((size_t)n * 48), "pinned staging");
-        MI_CU(ctx->h_items.ensure((size_t)n * sizeof(Item)), "pinned staging");
-        char kb[512];
-        int off = snprintf(kb, sizeof kb, "b:%d:%d:%d:%d:%d:%d:%d:%p:%p:%p:%p:%p:%p:%p:%d:%d", n, nq, ch.variant,
-                           ch.threads, ch.ctas, ch.tile.lpr_log2, ch.tile.slabs, ctx->d_aff.p, ctx->d_items.p,
-                           ctx->d_mi.p, ctx->d_h.p, ctx->d_cnt.p, ctx->h_aff.p, ctx->h_items.p, Q.form, Q.bits);
+        MI_CU(record_event(ctx->ev1, s), "event");
+        return MI_OK;
+    };
+    if (!use_graph) {
+        if ((st = enqueue()) != MI_OK) return st;
+    } else {
+        char kb[640];
+        int off = snprintf(kb, sizeof kb, "%d:%d:%d:%d:%d:%d:%d:%zu:%zu:%d:%p:%p:%p:%p:%p:%p:%p:%d:%d", n, nq, ch.variant,
+                           ch.threads, ch.ctas, ch.tile.lpr_log2, ch.tile.slabs, plan.items.size(), plan.slots.size(),
+                           R.d_q16 ? 1 : 0, ctx->d_in.p, ctx->d_work.p, ctx->d_part.p, ctx->d_mi.p, ctx->d_h.p,
+                           ctx->d_cnt.p, ctx->h_in.p, Q.form, Q.bits);
         for (int i = 0; i < nq && off < (int)sizeof kb - 40; ++i)
             off += snprintf(kb + off, sizeof kb - off, ":%08x:%p", fbits(Q.q[i]), (const void *)Q.tab[i]);
-        st = run_batched(ctx, n, Q, O, ch, use_graph, kb, h_aff, (size_t)n * 48, items.data(), (size_t)n * sizeof(Item));
-        if (st != MI_OK) return st;
-        ctx->timed = true;
-        ctx->last_launches = 1;
+        auto it = ctx->graphs.find(kb);
+        if (it == ctx->graphs.end()) {
+            // set kernel attributes outside of capture
+            batched_ctas_per_sm(ch.variant, ctx->max_bins, ch.threads, ctx->max_rows_words, ctx->max_zplanes);
+            cudaGraph_t g;
+            MI_CU(cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed), "begin capture");
+            st = enqueue();
+            cudaError_t e = cudaStreamEndCapture(s, &g);
+            if (st != MI_OK) {
+                if (e == cudaSuccess) cudaGraphDestroy(g);
+                return st;
+            }
+            if (e != cudaSuccess) return ctx->cuda_fail(e, "end capture");
+            auto ge = std::make_unique<GraphEntry>();
+            e = cudaGraphInstantiate(&ge->exec, g, 0);
+            cudaGraphDestroy(g);
+            if (e != cudaSuccess) return ctx->cuda_fail(e, "instantiating the graph");
+            if (ctx->graphs.size() > 32) ctx->graphs.clear();
+            it = ctx->graphs.emplace(kb, std::move(ge)).first;
+        }
+        MI_CU(cudaGraphLaunch(it->second->exec, s), "graph launch");
     }
+    ctx->timed = true;
+    ctx->last_launches = 0;
+    for (const Range &r : ranges) ctx->last_launches += r.nslots ? 2 : 1;
     if ((st = deliver(ctx, out_mi, ctx->d_mi.p, (size_t)n * nq * 8)) != MI_OK) return st;
     if ((st = deliver(ctx, out_h, ctx->d_h.p, (size_t)n * nq * 3 * 8)) != MI_OK) return st;
     if ((st = deliver(ctx, out_count, ctx->d_cnt.p, (size_t)n * 8)) != MI_OK) return st;
@@ -1903,7 +1964,7 @@ mi_status mi_last_kernel_ms(mi_ctx *ctx, float *ms, int *launches) {
 static const Choice *selected_choice(mi_ctx *ctx, int n) {
     const int path = ctx->opt.path == MI_PATH_AUTO ? ((ctx->pairs.size() > 1 || n >= ctx->sms) ? MI_PATH_BATCHED : MI_PATH_PLAIN)
                                                    : ctx->opt.path;
-    const int bucket = path == MI_PATH_BATCHED ? (n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0)) : 0;
+    const int bucket = path == MI_PATH_BATCHED ? (n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0)) : plain_bucket(n);
     auto it = ctx->tuned.find(std::make_tuple(path, path == MI_PATH_BATCHED ? -1 : 0, bucket));
     return it == ctx->tuned.end() ? nullptr : &it->second;
 }

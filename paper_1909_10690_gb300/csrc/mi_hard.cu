@@ -10,12 +10,12 @@
 //
 // Kernels:
 //   k_bin_fixed       fixed volume -> uint8 bins, once per context
-//   k_hist<...>       plain form: many CTAs per transform, privatised shared
-//                     histograms flushed to a global histogram per transform
-//   k_entropy         plain form: one CTA per transform reduces the global histogram
-//   k_batched<...>    batched form: persistent CTAs pull (pair, transform)
-//                     items from an atomic ticket; one CTA builds the whole
-//                     histogram of an item in shared memory and reduces it in place
+//   k_batched<...>    persistent CTAs pull work items from an atomic ticket.  An
+//                     item is a whole (pair, transform), whose histogram one CTA
+//                     builds in shared memory and reduces in place, or one of
+//                     several interleaved parts of it, whose histogram is added
+//                     to the transform's slot in global memory
+//   k_entropy_slots   reduces the slots' histograms, several CTAs per slot
 //   k_resample        v(T(x)) on the fixed grid
 //
 // Row clipping: along a fixed row (j, k) the moving index is linear in i, so
@@ -480,19 +480,15 @@ struct HistRows {
     }
 };
 
-// Global 32-bit histogram, row-major bins x bins (plain path's entropy reduction).
-struct HistGlobal {
-    const uint32_t *h;
-    int B;
-    __device__ __forceinline__ uint32_t count(int bf, int bm) const { return __ldg(h + bf * B + bm); }
-};
-
 // Shared-memory layout of a CTA: [histogram words][ovf keys][ovf counts][bitmap] [rows][cols] [FP64 scratch].
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct SmemLayout {
-    size_t hist, okey, ocnt, bmap, rinfo, rows, cols, red, zoff, total;
+    size_t hist, okey, ocnt, bmap, rinfo, rows, cols, red, zoff, small, total;
+    bool has_small;  // the count table of reduce_entropies fits
 };
+constexpr size_t kMaxCtaSmem = 227 * 1024;
+constexpr int kReduceWords = 1024;
 
 // zmax: planes of the largest moving volume (the gather variants keep one float2 offset per plane).
 __host__ __device__ inline SmemLayout smem_layout(int variant, int bins, int threads, int rows_words, int zmax) {
@@ -524,6 +520,9 @@ __host__ __device__ inline SmemLayout smem_layout(int variant, int bins, int thr
     o += (size_t)(3 * 32 + 3 * kMaxQ + 1) * 8;
     L.zoff = o;
     if (hv_fetch(variant) == FM_GATHER) o += (size_t)zmax * 8;
+    L.small = o;
+    L.has_small = o + kReduceWords * 4 <= kMaxCtaSmem;
+    if (L.has_small) o += kReduceWords * 4;
     L.total = o;
     (void)threads;
     return L;
@@ -883,16 +882,69 @@ __device__ __forceinline__ void load_zoff(const PairDev &P, float2 *s_zoff) {
 // Entropy reduction of one histogram by one CTA (Eq. 1, Eq. 2, Tsallis)
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ double term(uint32_t v, int iq, const QSet &Q) {
-    if (v < (uint32_t)kTab) return __ldg(Q.tab[iq] + v);
-    const double d = (double)v;
-    return Q.q[iq] == 1.0f ? d * log(d) : pow(d, (double)Q.q[iq]);
+// Entropy terms of a count v < 2^31: v ln v (q == 1) or v^q, from the count-indexed table; beyond it, with m
+// the leading 16 bits of v, v = 2^e m (1 + x), 0 <= x < 2^-15, from the table's entries of m and 2^e and
+// the series of ln(1 + x) or (1 + x)^q, whose terms after the cubic are below 2^-54 of the result for
+// q <= 7 (larger q: pow).  FP64 units are few (two lanes a clock an SM, so a warp's instruction takes 16
+// clocks whatever its active lanes), and a log or a pow is some 50 or 250 instructions; the series takes
+// eight for x, shared by every q, and five per q.
+__device__ __noinline__ double pow_term(double v, double q) { return pow(v, q); }
+
+struct Split {  // v = 2^e m (1 + x); e < 0: v is below the table's end
+    int e;
+    uint32_t m;
+    double x;
+};
+
+__device__ __forceinline__ Split split_count(uint32_t v) {
+    Split s;
+    s.e = v < (uint32_t)kTab ? -1 : 16 - __clz((int)v);
+    if (s.e < 0) {
+        s.m = v;
+        s.x = 0.0;
+        return s;
+    }
+    s.m = v >> s.e;
+    const double dm = (double)s.m;
+    double y = (double)__frcp_rn((float)s.m);  // 1 / m to 2^-24, then 2^-47: x keeps 2^-62
+    y = fma(fma(-dm, y, 1.0), y, y);
+    s.x = (double)(v - (s.m << s.e)) * y * __hiloint2double((1023 - s.e) << 20, 0);
+    return s;
 }
+
+__device__ __forceinline__ double split_term(uint32_t v, const Split &s, int iq, const QSet &Q) {
+    const double *__restrict__ tab = Q.tab[iq];
+    const double tm = __ldg(tab + s.m);
+    if (s.e < 0) return tm;
+    const float qf = Q.q[iq];
+    const double x = s.x;
+    if (qf == 1.0f) {
+        const double l = x * fma(-x, fma(-x, 1.0 / 3.0, 0.5), 1.0);
+        return fma((double)v, fma((double)s.e, 0.69314718055994530942, l), fma(x, tm, tm) * (double)(1u << s.e));
+    }
+    if (qf > 7.0f) return pow_term((double)v, (double)qf);
+    const double t = tm * __ldg(tab + (1u << s.e));
+    return fma(t, x * fma(x, fma(x, Q.c3[iq], Q.c2[iq]), (double)qf), t);
+}
+
+__device__ __forceinline__ double term(uint32_t v, int iq, const QSet &Q) { return split_term(v, split_count(v), iq, Q); }
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
+}
+
+// Warp-wide FP64 sums of four values: lane l gets the sum of a[l & 3].  Half of the values change lanes in
+// each of the first two steps, so six additions are issued instead of twenty (16 clocks each).
+__device__ __forceinline__ double warp_sum4(const double (&a)[4]) {
+    const bool odd = threadIdx.x & 1, upper = threadIdx.x & 2;
+    const double b0 = (odd ? a[1] : a[0]) + __shfl_xor_sync(kFull, odd ? a[0] : a[1], 1);
+    const double b1 = (odd ? a[3] : a[2]) + __shfl_xor_sync(kFull, odd ? a[2] : a[3], 1);
+    double c = (upper ? b1 : b0) + __shfl_xor_sync(kFull, upper ? b0 : b1, 2);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) c += __shfl_xor_sync(kFull, c, o);
+    return c;
 }
 
 // Block-wide FP64 sum of three values; every thread gets the results.
@@ -916,252 +968,322 @@ __device__ __forceinline__ void block_sum3(double &a, double &b, double &c, doub
     }
 }
 
-// Entropies and MI of transform t from the overlap count N and, per q, the sums over the fixed
-// marginal, the moving marginal and the joint cells (res[3 q + 0..2]) of c ln c (q == 1) or c^q:
-// H = ln N - S / N (Eq. 1), S_q = (1 - N^-q S) / (q - 1), MI = H_F + H_M - H_FM (Eq. 2) plus
-// (1 - q) S_q(F) S_q(M) in the pseudo-additive form.  One thread.
-__device__ void write_mi(double N, const double *res, const QSet &Q, long long t, const Outputs &O) {
-    const int nq = Q.nq;
-    if (O.count) O.count[t] = (long long)N;
-    if (N <= 0.0 && O.flags) atomicOr(&O.flags[0], 1);
-    for (int iq = 0; iq < nq; ++iq) {
-        const float qf = Q.q[iq];
-        const double SF = res[3 * iq + 0], SM = res[3 * iq + 1], SJ = res[3 * iq + 2];
-        double hf, hm, hj;
-        if (N <= 0.0) {
-            hf = hm = hj = __longlong_as_double(0x7ff8000000000000ll);
-        } else if (qf == 1.0f) {
-            const double lnN = log(N);
-            hf = lnN - SF / N;
-            hm = lnN - SM / N;
-            hj = lnN - SJ / N;
-            if (Q.bits) {
-                const double l2 = log(2.0);
-                hf /= l2;
-                hm /= l2;
-                hj /= l2;
-            }
-        } else {
-            const double q = (double)qf, Nq = pow(N, -q);
-            hf = (1.0 - Nq * SF) / (q - 1.0);
-            hm = (1.0 - Nq * SM) / (q - 1.0);
-            hj = (1.0 - Nq * SJ) / (q - 1.0);
-        }
-        double I = hf + hm - hj;
-        if (qf != 1.0f && Q.form == 1) I += (1.0 - (double)qf) * hf * hm;
-        if (O.mi) O.mi[t * nq + iq] = I;
-        if (O.h) {
-            O.h[(t * nq + iq) * 3 + 0] = hf;
-            O.h[(t * nq + iq) * 3 + 1] = hm;
-            O.h[(t * nq + iq) * 3 + 2] = hj;
+// Entropies and MI of transform t from the overlap count N and, per q, the sums S over the fixed marginal,
+// the moving marginal and the joint cells of c ln c (q == 1) or c^q: H = (N ln N - S) / N (Eq. 1),
+// S_q = (1 - S / N^q) / (q - 1), MI = H_F + H_M - H_FM (Eq. 2) plus (1 - q) S_q(F) S_q(M) in the
+// pseudo-additive form.  N ln N and N^q are the term of a cell that holds every voxel.  One warp: lane
+// 3 iq + w brings sum w of q iq (so every division is issued once).
+__device__ void write_mi(uint32_t N, double S, const QSet &Q, long long t, const Outputs &O) {
+    const int lane = threadIdx.x & 31, nq = Q.nq;
+    if (lane == 0) {
+        if (O.count) O.count[t] = (long long)N;
+        if (N == 0 && O.flags) atomicOr(&O.flags[0], 1);
+    }
+    const int iq = min(lane / 3, nq - 1);
+    const float qf = Q.q[iq];
+    double h;
+    if (N == 0) {
+        h = __longlong_as_double(0x7ff8000000000000ll);
+    } else {
+        const double full = term(N, iq, Q);
+        const bool shannon = qf == 1.0f;
+        double unit = shannon ? (double)N : full;
+        if (shannon && Q.bits) unit *= 0.69314718055994530942;
+        const double r = (shannon ? full - S : S) / unit;
+        h = shannon ? r : (1.0 - r) * Q.inv_q1[iq];
+    }
+    const double hm = __shfl_down_sync(kFull, h, 1), hj = __shfl_down_sync(kFull, h, 2);
+    if (lane < 3 * nq) {
+        if (O.h) O.h[t * nq * 3 + lane] = h;
+        if (lane % 3 == 0 && O.mi) {
+            double I = h + hm - hj;
+            if (qf != 1.0f && Q.form == 1) I += (1.0 - (double)qf) * h * hm;
+            O.mi[t * nq + iq] = I;
         }
     }
 }
 
-// Entropies of one histogram by one CTA.  Pass 1: marginals (row sums by
-// warps, column sums by shared atomics) and N.  Then one pass per q over the
-// non-zero cells and the marginals, with one FP64 accumulator triple live at a
-// time: sum c ln c (q == 1) or sum c^q (count-indexed tables for c < kTab).
+// Entropies of one histogram by one CTA, in one pass over the cells: marginals (row sums by warps,
+// column sums by shared atomics) and the joint terms of every q.  FP64 bounds it, so additions are saved
+// and FP64 instructions issued with full warps: most cells hold small counts, which are only counted
+// (small[c] = number of cells that hold c < kSmallCounts, an integer atomic) and enter the sums as one
+// product per count; counts below the table's end are looked up on the way; the few beyond it are listed
+// and taken side by side at the end.  One addition per cell and q, in a pass
+// per q, with every thread adding every warp's partial sums and log / pow beyond the table, was 4 % of the
+// batched kernel at 256 bins and four q (with the split tail, 4096 transforms of 256^3: 168.3 -> 163.6 ms a call).
+constexpr int kSmallCounts = 768;
+constexpr int kBigCounts = 255;
+
+// The shared words of a reduction (kReduceWords): cells per small count, then the listed counts.
+struct CountTable {
+    uint32_t *small;  // null: no room, every term is taken on the way
+    __device__ __forceinline__ uint32_t *nbig() const { return small + kSmallCounts; }
+    __device__ __forceinline__ uint32_t *big() const { return small + kSmallCounts + 1; }
+    __device__ void zero() {
+        if (small)
+            for (int c = threadIdx.x; c <= kSmallCounts; c += blockDim.x) small[c] = 0;
+    }
+    // True if the table took the count; else the caller adds its terms.
+    __device__ __forceinline__ bool take(uint32_t v) {
+        if (!small) return false;
+        if (v < (uint32_t)kSmallCounts) {
+            atomicAdd(&small[v], 1u);
+            return true;
+        }
+        if (v < (uint32_t)kTab) return false;
+        const uint32_t i = atomicAdd(nbig(), 1u);
+        if (i >= (uint32_t)kBigCounts) return false;
+        big()[i] = v;
+        return true;
+    }
+    // The same answer for a pass after the first (which lists large counts if there is room for all).
+    __device__ __forceinline__ bool taken_before(uint32_t v) const {
+        return small && (v < (uint32_t)kSmallCounts || (v >= (uint32_t)kTab && *nbig() <= (uint32_t)kBigCounts));
+    }
+    // This thread's share of the table's terms of q0 .. q0 + 3.
+    __device__ __forceinline__ void add_terms(double (&a)[4], int q0, const QSet &Q) const {
+        if (!small) return;
+#pragma unroll 3
+        for (int c = threadIdx.x; c < kSmallCounts; c += blockDim.x) {
+            const uint32_t m = small[c];
+            double tv[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tv[k] = m && q0 + k < Q.nq ? __ldg(Q.tab[q0 + k] + c) : 0.0;
+            if (m) {
+                const double dm = (double)m;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a[k] = fma(dm, tv[k], a[k]);
+            }
+        }
+        // when the list overflowed, the passes after the first take every large count on the way
+        const int n = (int)*nbig() <= kBigCounts ? (int)*nbig() : (q0 == 0 ? kBigCounts : 0);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) add_count(a, big()[i], q0, Q);
+    }
+    __device__ __forceinline__ static void add_count(double (&a)[4], uint32_t v, int q0, const QSet &Q) {
+        const Split s = split_count(v);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (q0 + k < Q.nq) a[k] += split_term(v, s, q0 + k, Q);
+    }
+};
+static_assert(kSmallCounts + 1 + kBigCounts == kReduceWords, "the table fills its shared words");
+
 template <class Hist>
 __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *s_rows, uint32_t *s_cols,
-                                 double *s_red, long long t, const Outputs &O) {
+                                 double *s_red, CountTable C, long long t, const Outputs &O) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int nq = Q.nq;
-    double *s_res = s_red + 3 * 32;  // 3 nq + 1 results after the per-warp scratch
+    double *s_res = s_red + 3 * 32;  // 3 nq results after the per-warp scratch
     for (int c = tid; c < B; c += blockDim.x) s_cols[c] = 0;
+    C.zero();
     __syncthreads();
-    for (int r = warp; r < B; r += nwarps) {
-        uint32_t rsum = 0;
-        for (int c = lane; c < B; c += 32) {
-            const uint32_t v = H.count(r, c);
-            if (v) {
-                rsum += v;
-                atomicAdd(&s_cols[c], v);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rsum += __shfl_xor_sync(kFull, rsum, o);
-        if (lane == 0) s_rows[r] = rsum;
-    }
-    __syncthreads();
-    {
-        double n0 = 0.0, z1 = 0.0, z2 = 0.0;
-        for (int r = tid; r < B; r += blockDim.x) n0 += (double)s_rows[r];
-        block_sum3(n0, z1, z2, s_red);
-        if (tid == 0) s_res[3 * kMaxQ] = n0;
-    }
-    for (int iq = 0; iq < nq; ++iq) {
-        double aj = 0.0, af = 0.0, am = 0.0;
-        for (int r = warp; r < B; r += nwarps)
+    // four q per pass over the cells: the accumulators of more would spill
+    for (int q0 = 0; q0 < nq; q0 += 4) {
+        double aj[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int r = warp; r < B; r += nwarps) {
+            uint32_t rsum = 0;
             for (int c = lane; c < B; c += 32) {
                 const uint32_t v = H.count(r, c);
-                if (v) aj += term(v, iq, Q);
+                if (v == 0) continue;
+                bool taken;
+                if (q0 == 0) {
+                    rsum += v;
+                    atomicAdd(&s_cols[c], v);
+                    taken = C.take(v);
+                } else {
+                    taken = C.taken_before(v);
+                }
+                if (!taken) CountTable::add_count(aj, v, q0, Q);
             }
-        for (int r = tid; r < B; r += blockDim.x) {
-            const uint32_t vf = s_rows[r], vm = s_cols[r];
-            if (vf) af += term(vf, iq, Q);
-            if (vm) am += term(vm, iq, Q);
+            if (q0 == 0) {
+                rsum = __reduce_add_sync(kFull, rsum);
+                if (lane == 0) s_rows[r] = rsum;
+            }
         }
-        block_sum3(af, am, aj, s_red);
-        if (tid == 0) {
-            s_res[3 * iq + 0] = af;
-            s_res[3 * iq + 1] = am;
-            s_res[3 * iq + 2] = aj;
+        __syncthreads();
+        C.add_terms(aj, q0, Q);
+        // joint sums: the upper 16 warps' into the lower 16; marginals: up to 64 entries a warp, warps
+        // 0..3 the rows and 4..7 the columns; then warp 0 takes lane = 4 j + k for q0 + k
+        double *s_joint = s_red, *s_marg = s_red + 64;
+        double j = warp_sum4(aj);
+        if (warp >= 16 && lane < 4) s_joint[4 * (warp - 16) + lane] = j;
+        __syncthreads();
+        if (warp < 16 && lane < 4) s_joint[4 * warp + lane] = j + (warp + 16 < nwarps ? s_joint[4 * warp + lane] : 0.0);
+        if (warp < 8) {
+            const uint32_t *m = warp < 4 ? s_rows : s_cols;
+            double am[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int x = (warp & 3) * 32 + lane; x < B; x += 128)
+                if (m[x]) CountTable::add_count(am, m[x], q0, Q);
+            const double v = warp_sum4(am);
+            if (lane < 4) s_marg[4 * warp + lane] = v;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const int k = lane & 3, i = lane >> 2;
+            double v = s_joint[4 * i + k] + s_joint[4 * (i + 8) + k], mg = s_marg[4 * i + k];
+#pragma unroll
+            for (int o = 4; o < 16; o <<= 1) {
+                v += __shfl_xor_sync(kFull, v, o);
+                mg += __shfl_xor_sync(kFull, mg, o);
+            }
+            v += __shfl_xor_sync(kFull, v, 16);
+            if (q0 + k < nq) {
+                if (i == 0) s_res[3 * (q0 + k) + 0] = mg;
+                if (i == 4) s_res[3 * (q0 + k) + 1] = mg;
+                if (i == 0) s_res[3 * (q0 + k) + 2] = v;
+            }
         }
     }
     __syncthreads();
-    if (tid == 0) write_mi(s_res[3 * kMaxQ], s_res, Q, t, O);
+    if (warp == 0) {
+        uint32_t N = 0;  // fewer than 2^31 voxels
+        for (int r = lane; r < B; r += 32) N += s_rows[r];
+        N = __reduce_add_sync(kFull, N);
+        write_mi(N, lane < 3 * nq ? s_res[lane] : 0.0, Q, t, O);
+    }
     __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
-// Plain form
+// Entropies of the histograms in global memory (transforms whose work was split over CTAs)
 // ---------------------------------------------------------------------------
 
-template <typename PairT, int HV, int FM>
-__global__ void __launch_bounds__(1024, 1)
-    k_hist(const PairDev *__restrict__ pairs, const int32_t *__restrict__ aff, uint32_t *__restrict__ ghist,
-           int *flags, Tile tile) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const PairDev P = pairs[0];
-    const int t = blockIdx.y;
-    const int B = P.bins;
-    const SmemLayout L = smem_layout(HV, B, blockDim.x, P.rows_words, P.nm[2]);
-    __shared__ int q[12];
-    if (threadIdx.x < 12) q[threadIdx.x] = aff[(size_t)t * 12 + threadIdx.x];
-    float2 *s_zoff = (float2 *)(smem + L.zoff);
-    load_zoff<FM>(P, s_zoff);
-    auto H = make_hist<HV>(smem, L, B, flags, P.rows_words);
-    H.load_info(P.rowinfo);
-    H.zero();
-    __syncthreads();
-    const int nwarps = blockDim.x >> 5, lane = threadIdx.x & 31;
-    walk_rows<PairT, FM>(P, q, s_zoff, blockIdx.x, gridDim.x, ((long long)P.nf[1] * P.nf[2] + nwarps - 1) / nwarps,
-                         tile.lpr_log2, H);
-    __syncthreads();
-    uint32_t *gh = ghist + (size_t)t * B * B;
-    for (int r = threadIdx.x >> 5; r < B; r += nwarps)
-        for (int c = lane; c < B; c += 32) {
-            const uint32_t v = H.count(r, c);
-            if (v) atomicAdd(gh + r * B + c, v);
-        }
+// Grid (parts, slots): CTA (p, i) takes rows p, p + parts, ... of slot i's histogram (their cells' joint
+// terms and their sums, the fixed marginal) and a contiguous share of its columns (the moving marginal).
+// part[(i parts + p) kPartStride]: per q the sums of the fixed, moving and joint terms and, last, the
+// count; the CTA that finishes a slot last (a counter in `done`, zeroed by the caller) adds the parts in a
+// fixed order and writes the results.
+// What bounds it: for one slot the latency of dependent FP64 instructions (64 clocks and more each on the
+// SM's few FP64 lanes), so loads are issued together, sums are trees, marginal entries take a lane each
+// beside one another and no step is left to one CTA but the last sum; for many slots the FP64 issue (16
+// clocks a warp), so a CTA with many cells counts the small counts first (CountTable).
+// Two launches (parts, then one CTA per transform), log / pow beyond the table and sums by one thread took
+// 81 us for one transform at 256 bins and four q and 332 us for 81 at 128 bins and six; this takes 23 and 53.
+constexpr int kPartStride = 3 * kMaxQ + 1;
+constexpr int kEntThreads = 256;
+
+__device__ __forceinline__ double tree8(const double *v, int stride) {
+    return ((v[0] + v[stride]) + (v[2 * stride] + v[3 * stride])) +
+           ((v[4 * stride] + v[5 * stride]) + (v[6 * stride] + v[7 * stride]));
 }
 
-// Shared memory of k_entropy: [rows B u32][cols B u32][FP64 scratch, 16-byte aligned].
-__host__ __device__ inline size_t entropy_red_offset(int B) { return align_up((size_t)B * 8, 16); }
-__host__ __device__ inline size_t entropy_smem_bytes(int B, int threads) {
-    return entropy_red_offset(B) + (size_t)(3 * 32 + 3 * kMaxQ + 1) * 8;
-}
-
-__global__ void __launch_bounds__(1024, 1)
-    k_entropy(const uint32_t *__restrict__ ghist, int B, QSet Q, Outputs O) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const long long t = blockIdx.x;
-    HistGlobal H{ghist + (size_t)t * B * B, B};
-    reduce_entropies(H, B, Q, (uint32_t *)smem, (uint32_t *)(smem + (size_t)B * 4),
-                     (double *)(smem + entropy_red_offset(B)), t, O);
-}
-
-// The same reduction split over `parts` CTAs per transform, for calls with few transforms (the plain
-// form's one-transform calls), where one CTA per transform would leave the GPU idle.  CTA (p, t) takes
-// rows p, p + parts, ... of histogram t: their sums (the fixed marginal) and terms, the joint terms of
-// their cells and their part of the column sums (the moving marginal, into cols[t], zeroed by the
-// caller).  part[(t parts + p) (1 + 2 kMaxQ)]: the count, then per q the joint and fixed-marginal sums.
-constexpr int kPartStride = 1 + 2 * kMaxQ;
-
-__global__ void __launch_bounds__(256)
-    k_entropy_part(const uint32_t *__restrict__ ghist, int B, QSet Q, uint32_t *__restrict__ cols,
-                   double *__restrict__ part, int parts) {
-    __shared__ uint32_t s_cols[256];
-    __shared__ double s_red[3 * 32];
-    const int t = blockIdx.y, p = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    const uint32_t *h = ghist + (size_t)t * B * B;
-    for (int c = tid; c < B; c += blockDim.x) s_cols[c] = 0;
+__global__ void __launch_bounds__(kEntThreads)
+    k_entropy_slots(const uint32_t *__restrict__ hist, long long hist_stride, const Slot *__restrict__ slots,
+                    const __grid_constant__ QSet Q, unsigned int *__restrict__ done, double *__restrict__ part,
+                    const __grid_constant__ Outputs O) {
+    constexpr int nwarps = kEntThreads / 32;
+    static_assert(nwarps == 8 && kPartStride <= 32, "trees over eight warps, a lane per sum");
+    __shared__ uint32_t s_rows[256], s_cols[256], s_words[kReduceWords];
+    __shared__ double s_joint[nwarps][kMaxQ], s_marg[nwarps][kMaxQ], s_part[nwarps][32];
+    __shared__ uint32_t s_n[nwarps];
+    __shared__ bool s_last;
+    const int slot = blockIdx.y, p = blockIdx.x, parts = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int t = slots[slot].t, B = slots[slot].bins, nq = Q.nq;
+    const uint32_t *h = hist + (size_t)slot * hist_stride;
+    const bool few = B * B <= 2048 * parts;  // few cells: looked up on the way
+    CountTable C{few ? nullptr : s_words};
+    const int c0 = (int)((long long)B * p / parts), ncols = (int)((long long)B * (p + 1) / parts) - c0;
+    const int nrows = (B - p + parts - 1) / parts;
+    s_cols[tid] = 0;
+    C.zero();
     __syncthreads();
-    double n = 0.0, aj[kMaxQ], af[kMaxQ];
+    for (int q0 = 0; q0 < nq; q0 += 4) {
+        double aj[4] = {0.0, 0.0, 0.0, 0.0};
+        if (q0 == 0 && parts > 1)  // the column share; with one part the row pass meets every column
+            for (int x = tid; x < B * ncols; x += kEntThreads) {
+                const uint32_t v = __ldcg(h + (size_t)(x / ncols) * B + c0 + x % ncols);
+                if (v) atomicAdd(&s_cols[x % ncols], v);
+            }
+        for (int i = warp; i < nrows; i += nwarps) {
+            const uint32_t *row = h + (size_t)(p + parts * i) * B;
+            uint32_t v[8], rsum = 0;
 #pragma unroll
-    for (int iq = 0; iq < kMaxQ; ++iq) aj[iq] = af[iq] = 0.0;
-    for (int r = p + parts * warp; r < B; r += parts * nwarps) {
-        uint32_t rsum = 0;
-        for (int c = lane; c < B; c += 32) {
-            const uint32_t v = __ldg(h + (size_t)r * B + c);
-            if (v) {
-                rsum += v;
-                atomicAdd(&s_cols[c], v);
+            for (int k = 0; k < 8; ++k) v[k] = lane + 32 * k < B ? __ldcg(row + lane + 32 * k) : 0u;
 #pragma unroll
-                for (int iq = 0; iq < kMaxQ; ++iq)
-                    if (iq < Q.nq) aj[iq] += term(v, iq, Q);
+            for (int k = 0; k < 8; ++k) {
+                if (v[k] == 0) continue;
+                bool taken;
+                if (q0 == 0) {
+                    rsum += v[k];
+                    if (parts == 1) atomicAdd(&s_cols[lane + 32 * k], v[k]);
+                    taken = C.take(v[k]);
+                } else {
+                    taken = C.taken_before(v[k]);
+                }
+                if (!taken) CountTable::add_count(aj, v[k], q0, Q);
+            }
+            if (q0 == 0) {
+                rsum = __reduce_add_sync(kFull, rsum);
+                if (lane == 0) s_rows[i] = rsum;
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rsum += __shfl_xor_sync(kFull, rsum, o);
-        if (lane == 0 && rsum) {
-            n += (double)rsum;
-#pragma unroll
-            for (int iq = 0; iq < kMaxQ; ++iq)
-                if (iq < Q.nq) af[iq] += term(rsum, iq, Q);
+        __syncthreads();
+        // marginal entries: warps 0..3 the rows, 4..7 the columns
+        const uint32_t *line = warp < 4 ? s_rows : s_cols;
+        const int nline = warp < 4 ? nrows : ncols;
+        double m = 0.0;
+        if ((warp & 3) * 32 < nline) {
+            double am[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int i = tid & 127; i < nline; i += 128)
+                if (line[i]) CountTable::add_count(am, line[i], q0, Q);
+            m = warp_sum4(am);
+        }
+        C.add_terms(aj, q0, Q);
+        const double j = warp_sum4(aj);
+        if (lane < 4) {
+            s_joint[warp][q0 + lane] = j;
+            s_marg[warp][q0 + lane] = m;
         }
     }
+    uint32_t n = 0;  // fewer than 2^31 voxels
+    for (int i = tid; i < nrows; i += kEntThreads) n += s_rows[i];
+    n = __reduce_add_sync(kFull, n);
+    if (lane == 0) s_n[warp] = n;
     __syncthreads();
-    for (int c = tid; c < B; c += blockDim.x)
-        if (s_cols[c]) atomicAdd(cols + (size_t)t * B + c, s_cols[c]);
-    double *out = part + ((size_t)t * parts + p) * kPartStride;
-    double z = 0.0;
-    block_sum3(n, z, z, s_red);
-    if (tid == 0) out[0] = n;
-    for (int iq = 0; iq < Q.nq; ++iq) {
-        double a = aj[iq], b = af[iq];
-        z = 0.0;
-        block_sum3(a, b, z, s_red);
-        if (tid == 0) {
-            out[1 + 2 * iq] = a;
-            out[2 + 2 * iq] = b;
+    // lane 3 iq + w of warp 0: this CTA's sum w of q iq (fixed, moving, joint); lane 3 nq: its count
+    double S = 0.0;
+    uint32_t N = 0;
+    if (warp == 0) {
+        const int iq = lane / 3, w = lane % 3;
+        for (int k = 0; k < nwarps; ++k) N += s_n[k];
+        if (lane < 3 * nq) {
+            const double *g = &s_marg[w == 1 ? 4 : 0][iq];
+            S = w == 2 ? tree8(&s_joint[0][iq], kMaxQ) : (g[0] + g[kMaxQ]) + (g[2 * kMaxQ] + g[3 * kMaxQ]);
         }
     }
-}
-
-// Finishes the split reduction: the moving-marginal terms from cols[t], the parts' sums, then MI.
-__global__ void __launch_bounds__(256)
-    k_entropy_final(const uint32_t *__restrict__ cols, const double *__restrict__ part, int parts, int B, QSet Q,
-                    Outputs O) {
-    __shared__ double s_red[3 * 32];
-    __shared__ double s_res[3 * kMaxQ + 1];
-    const int t = blockIdx.x, tid = threadIdx.x;
-    for (int iq = 0; iq < Q.nq; ++iq) {
-        double am = 0.0, z0 = 0.0, z1 = 0.0;
-        for (int c = tid; c < B; c += blockDim.x) {
-            const uint32_t v = cols[(size_t)t * B + c];
-            if (v) am += term(v, iq, Q);
+    if (parts > 1) {
+        double *out = part + (size_t)slot * parts * kPartStride;
+        if (warp == 0 && lane <= 3 * nq) out[(size_t)p * kPartStride + lane] = lane < 3 * nq ? S : (double)N;
+        __threadfence();  // this CTA's part is visible before it counts as finished
+        __syncthreads();
+        if (tid == 0) s_last = atomicAdd(done + slot, 1u) == (unsigned)parts - 1u;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        double a = 0.0;
+        if (lane <= 3 * nq) {
+#pragma unroll 4
+            for (int k = warp; k < parts; k += nwarps) a += __ldcg(out + (size_t)k * kPartStride + lane);
         }
-        block_sum3(am, z0, z1, s_red);
-        if (tid == 0) {
-            double sj = 0.0, sf = 0.0;
-            for (int p = 0; p < parts; ++p) {
-                const double *in = part + ((size_t)t * parts + p) * kPartStride;
-                sj += in[1 + 2 * iq];
-                sf += in[2 + 2 * iq];
-            }
-            s_res[3 * iq + 0] = sf;
-            s_res[3 * iq + 1] = am;
-            s_res[3 * iq + 2] = sj;
-        }
+        s_part[warp][lane] = a;
+        __syncthreads();
+        S = tree8(&s_part[0][lane], 32);
+        N = (uint32_t)__shfl_sync(kFull, S, 3 * nq);
     }
-    if (tid == 0) {
-        double N = 0.0;
-        for (int p = 0; p < parts; ++p) N += part[((size_t)t * parts + p) * kPartStride];
-        write_mi(N, s_res, Q, t, O);
-    }
+    if (warp == 0) write_mi(N, S, Q, t, O);
 }
 
 // ---------------------------------------------------------------------------
-// Batched form: persistent CTAs, one (pair, transform) item per CTA at a time
+// Persistent CTAs, one work item (a whole transform, or one part of one) per CTA at a time
 // ---------------------------------------------------------------------------
 
 template <int HV, int FM>
 __global__ void __launch_bounds__(1024, 1)
     k_batched(const PairDev *__restrict__ pairs, const int32_t *__restrict__ aff, const Item *__restrict__ items,
-              int nitems, int *ticket, int max_bins, int rows_words, int zmax, Tile tile, QSet Q, Outputs O) {
+              int nitems, int *ticket, int max_bins, int rows_words, int zmax, Tile tile,
+              const __grid_constant__ QSet Q, const __grid_constant__ Outputs O,
+              uint32_t *__restrict__ slot_hist, long long slot_stride) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_item, s_slab;
     __shared__ int q[12];
@@ -1189,6 +1311,23 @@ __global__ void __launch_bounds__(1024, 1)
         // started by any CTA, so CTAs working on different transforms keep to neighbouring slabs
         // of the volumes and their working set stays in L2.  No CTA waits for another.
         const long long NB = ((long long)P.nf[1] * P.nf[2] + nwarps - 1) / nwarps;
+        if (I.slot >= 0) {
+            // one part of a transform: row blocks part, part + parts, ... (interleaved, so every part
+            // meets the same share of the overlap), added to the transform's slot
+            if (FM == FM_QUAD || FM == FM_GATHER || P.mdtype == 1)
+                walk_rows<uint32_t, FM>(P, q, s_zoff, I.part, I.parts, NB, tile.lpr_log2, H);
+            else
+                walk_rows<uint16_t, FM>(P, q, s_zoff, I.part, I.parts, NB, tile.lpr_log2, H);
+            __syncthreads();
+            uint32_t *gh = slot_hist + (size_t)I.slot * slot_stride;
+            for (int r = threadIdx.x >> 5; r < B; r += nwarps)
+                for (int c = threadIdx.x & 31; c < B; c += 32) {
+                    const uint32_t v = H.count(r, c);
+                    if (v) atomicAdd(gh + r * B + c, v);
+                }
+            __syncthreads();
+            continue;
+        }
         const long long SB = (NB + slabs - 1) / slabs;
         unsigned left = (1u << slabs) - 1u;
         while (left) {
@@ -1219,7 +1358,7 @@ __global__ void __launch_bounds__(1024, 1)
                 for (int c = threadIdx.x & 31; c < B; c += 32) dh[r * B + c] = H.count(r, c);
         }
         reduce_entropies(H, P.bins, Q, (uint32_t *)(smem + L.rows), (uint32_t *)(smem + L.cols),
-                         (double *)(smem + L.red), I.t, O);
+                         (double *)(smem + L.red), CountTable{L.has_small ? (uint32_t *)(smem + L.small) : nullptr}, I.t, O);
     }
 }
 
@@ -1413,63 +1552,20 @@ cudaError_t launch_table(double *tab, float q, cudaStream_t s) {
     X(HV_U16_GATHER, HV_U16, FM_GATHER)
 #define MI_VARIANTS(X) MI_VARIANTS_PAIRED(X) MI_VARIANTS_TEXEL(X)
 
-template <typename MT>
-static const void *plain_fn_of(int variant) {
-    switch (variant) {
-#define MI_PLAIN_CASE(V, K, F) \
-    case V: return (const void *)k_hist<MT, K, F>;
-        MI_VARIANTS_PAIRED(MI_PLAIN_CASE)
-#undef MI_PLAIN_CASE
-        default: return nullptr;
-    }
-}
-
-static const void *plain_fn(int variant, int mdtype) {
-    switch (variant) {
-#define MI_PLAIN_CASE(V, K, F) \
-    case V: return (const void *)k_hist<uint32_t, K, F>;
-        MI_VARIANTS_TEXEL(MI_PLAIN_CASE)
-#undef MI_PLAIN_CASE
-        default: return mdtype == 0 ? plain_fn_of<uint16_t>(variant) : plain_fn_of<uint32_t>(variant);
-    }
-}
-
-cudaError_t launch_plain_hist(const PairDev *d_pair, const PairDev &h_pair, const int32_t *d_aff, int n,
-                              uint32_t *d_hist, int variant, int threads, int ctas, Tile tile, int *d_flags,
-                              cudaStream_t s) {
-    const size_t B2 = (size_t)h_pair.bins * h_pair.bins;
-    cudaError_t e = cudaMemsetAsync(d_hist, 0, (size_t)n * B2 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
-    const size_t smem = smem_layout(variant, h_pair.bins, threads, h_pair.rows_words, h_pair.nm[2]).total;
-    const void *fn = plain_fn(variant, h_pair.mdtype);
-    if (!fn) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
-    void *args[] = {(void *)&d_pair, (void *)&d_aff, (void *)&d_hist, (void *)&d_flags, (void *)&tile};
-    return cudaLaunchKernel(fn, dim3(ctas, n), dim3(threads), args, smem, s);
-}
-
-cudaError_t launch_entropy(const uint32_t *d_hist, int n, int bins, const QSet &Q, const Outputs &O, cudaStream_t s) {
-    const int threads = 1024;
-    const size_t smem = entropy_smem_bytes(bins, threads);
-    cudaError_t e = set_smem(k_entropy, smem);
-    if (e != cudaSuccess) return e;
-    k_entropy<<<n, threads, smem, s>>>(d_hist, bins, Q, O);
+cudaError_t launch_entropy_slots(const uint32_t *d_hist, long long hist_stride, const Slot *d_slots, int nslots,
+                                 int parts, const QSet &Q, unsigned int *d_done, double *d_part, const Outputs &O,
+                                 cudaStream_t s) {
+    k_entropy_slots<<<dim3(parts, nslots), kEntThreads, 0, s>>>(d_hist, hist_stride, d_slots, Q, d_done, d_part, O);
     return cudaGetLastError();
 }
 
-int entropy_parts(int bins) { return bins >= 256 ? 32 : (bins / 8 > 1 ? bins / 8 : 1); }
-
-cudaError_t launch_entropy_split(const uint32_t *d_hist, int n, int bins, const QSet &Q, const Outputs &O,
-                                 uint32_t *d_cols, double *d_part, cudaStream_t s) {
-    const int parts = entropy_parts(bins);
-    cudaError_t e = cudaMemsetAsync(d_cols, 0, (size_t)n * bins * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
-    k_entropy_part<<<dim3(parts, n), 256, 0, s>>>(d_hist, bins, Q, d_cols, d_part, parts);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_entropy_final<<<n, 256, 0, s>>>(d_cols, d_part, parts, bins, Q, O);
-    return cudaGetLastError();
+// Parts per slot: about two CTAs an SM over all slots (more would only repeat the reductions, whose FP64
+// additions bound a launch over many slots), each of at least eight rows (one per warp).
+int entropy_parts(int max_bins, int nslots, int sms) {
+    const int most = (max_bins + 7) / 8, want = (2 * sms + nslots - 1) / nslots;
+    return want < most ? want : most;
 }
+size_t entropy_part_bytes(int parts, int nslots) { return (size_t)parts * nslots * kPartStride * sizeof(double); }
 
 static const void *batched_fn(int variant) {
     switch (variant) {
@@ -1493,15 +1589,17 @@ int batched_ctas_per_sm(int variant, int max_bins, int threads, int rows_words, 
 
 cudaError_t launch_batched(const PairDev *d_pairs, const int32_t *d_aff, const Item *d_items, int nitems,
                            int *d_ticket, int max_bins, int rows_words, int zmax, int variant, int threads, int ctas,
-                           Tile tile, const QSet &Q, const Outputs &O, cudaStream_t s) {
+                           Tile tile, const QSet &Q, const Outputs &O, uint32_t *slot_hist, long long slot_stride,
+                           cudaStream_t s) {
     const size_t smem = smem_layout(variant, max_bins, threads, rows_words, zmax).total;
     const void *fn = batched_fn(variant);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&d_pairs, (void *)&d_aff, (void *)&d_items, (void *)&nitems, (void *)&d_ticket,
-                    (void *)&max_bins, (void *)&rows_words, (void *)&zmax, (void *)&tile, (void *)&Q, (void *)&O};
-    return cudaLaunchKernel(fn, dim3(ctas), dim3(threads), args, smem, s);
+                    (void *)&max_bins, (void *)&rows_words, (void *)&zmax, (void *)&tile, (void *)&Q, (void *)&O,
+                    (void *)&slot_hist, (void *)&slot_stride};
+    return cudaLaunchKernel(fn, dim3(ctas < nitems ? ctas : nitems), dim3(threads), args, smem, s);
 }
 
 cudaError_t launch_resample(const PairDev *d_pair, const PairDev &h_pair, const int32_t *d_aff, void *out,

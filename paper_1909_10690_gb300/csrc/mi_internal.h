@@ -43,6 +43,8 @@ struct QSet {
     int pad;
     float q[kMaxQ];
     const double *tab[kMaxQ];
+    double c2[kMaxQ], c3[kMaxQ];  // q (q - 1) / 2 and q (q - 1) (q - 2) / 6
+    double inv_q1[kMaxQ];         // 1 / (q - 1) (0 for q == 1)
 };
 
 // Per-transform outputs (device pointers; any may be null).
@@ -54,10 +56,18 @@ struct Outputs {
     int *flags;          // [0] empty overlap seen, [1] drain table overflow
 };
 
-// Work item of the batched kernel.
+// Work item of the hard-path kernel: a whole transform, reduced in place by its CTA (slot < 0), or the
+// row blocks part, part + parts, ... of one, added to histogram `slot` in global memory.
 struct Item {
     int pair;
     int t;   // transform index (row of the affine array and of the outputs)
+    unsigned short part, parts;
+    int slot;
+};
+// A histogram in global memory: the transform it belongs to and its bin count.
+struct Slot {
+    int t;
+    int bins;
 };
 
 // Histogram variants (match the public MI_HV_* values).  0..3: counter kinds
@@ -124,21 +134,19 @@ cudaError_t launch_make_zpairs(const void *mov, int dtype, const int nm[3], int 
 cudaError_t launch_bin_fixed(const void *data, int dtype, int depth, long long n, int bins, uint8_t *out,
                              cudaStream_t s);
 cudaError_t launch_table(double *tab, float q, cudaStream_t s);
-// Plain path: n transforms, grid (ctas, n); histograms in global memory (n x bins^2 u32, zeroed here).
-cudaError_t launch_plain_hist(const PairDev *d_pair, const PairDev &h_pair, const int32_t *d_aff, int n,
-                              uint32_t *d_hist, int variant, int threads, int ctas, Tile tile, int *d_flags,
-                              cudaStream_t s);
-cudaError_t launch_entropy(const uint32_t *d_hist, int n, int bins, const QSet &Q, const Outputs &O,
-                           cudaStream_t s);
-// The same reduction split over entropy_parts(bins) CTAs per transform (for few transforms).
-// Scratch: d_cols n x bins u32 (zeroed here), d_part n x entropy_parts(bins) x (1 + 2 kMaxQ) FP64.
-int entropy_parts(int bins);
-cudaError_t launch_entropy_split(const uint32_t *d_hist, int n, int bins, const QSet &Q, const Outputs &O,
-                                 uint32_t *d_cols, double *d_part, cudaStream_t s);
-// Batched path: persistent CTAs pull items from *d_ticket (reset by the caller).
+// The hard-path kernel: persistent CTAs pull items from *d_ticket (reset by the caller); the parts of split
+// transforms are added to slot_hist + slot * slot_stride (bins^2 u32 each, zeroed by the caller).
 cudaError_t launch_batched(const PairDev *d_pairs, const int32_t *d_aff, const Item *d_items, int nitems,
                            int *d_ticket, int max_bins, int rows_words, int zmax, int variant, int threads, int ctas,
-                           Tile tile, const QSet &Q, const Outputs &O, cudaStream_t s);
+                           Tile tile, const QSet &Q, const Outputs &O, uint32_t *slot_hist, long long slot_stride,
+                           cudaStream_t s);
+// Entropies and MI of the slots' histograms, `parts` CTAs per slot (entropy_parts).  Scratch: d_done (one
+// per slot, zeroed by the caller) and d_part (entropy_part_bytes).
+int entropy_parts(int max_bins, int nslots, int sms);
+size_t entropy_part_bytes(int parts, int nslots);
+cudaError_t launch_entropy_slots(const uint32_t *d_hist, long long hist_stride, const Slot *d_slots, int nslots,
+                                 int parts, const QSet &Q, unsigned int *d_done, double *d_part, const Outputs &O,
+                                 cudaStream_t s);
 int batched_ctas_per_sm(int variant, int max_bins, int threads, int rows_words, int zmax);
 cudaError_t launch_resample(const PairDev *d_pair, const PairDev &h_pair, const int32_t *d_aff, void *out,
                             cudaStream_t s);
