@@ -386,7 +386,7 @@ mi_status mi_last_kernel_ms(mi_ctx *ctx, float *ms, int *launches);
  *    MI_NOALLOC_MAX_MOVING_VOXELS.  Larger sizes return MI_EINVAL.
  *  - out_mi: nq doubles, host or device memory.  stream: a cudaStream_t
  *    (NULL = legacy default stream); the call synchronises it.
- *  - Intermediates live in one static device array of about 257 KiB that every
+ *  - Intermediates live in one static device array of about 280 KiB that every
  *    GPU loading the library holds until the process exits.  The call clears
  *    the histogram part before use; the array keeps the last call's contents.
  *    All calls share it, so calls that overlap on the GPU (several streams or

@@ -968,11 +968,7 @@ mi_status make_qset(mi_ctx *ctx, const float *qv, int nq, QSet &Q) {
     Q.form = ctx->opt.tsallis_form;
     Q.bits = ctx->opt.log_bits ? 1 : 0;
     for (int i = 0; i < nq; ++i) {
-        Q.q[i] = qv[i];
-        const double q = (double)qv[i];
-        Q.c2[i] = q * (q - 1.0) / 2.0;
-        Q.c3[i] = q * (q - 1.0) * (q - 2.0) / 6.0;
-        Q.inv_q1[i] = q == 1.0 ? 0.0 : 1.0 / (q - 1.0);
+        set_q(Q, i, qv[i]);
         if (ctx->opt.kernel == MI_HARD) {
             auto it = ctx->tables.find(fbits(qv[i]));
             if (it == ctx->tables.end()) {
@@ -2003,6 +1999,17 @@ mi_status mi_selected_config(mi_ctx *ctx, int n, int out[5]) {
 // Helpers for the allocation-free entry point in mi_noalloc.cu
 // ---------------------------------------------------------------------------
 namespace mi {
+
+void set_q(QSet &Q, int i, float qv) {
+    const double q = (double)qv;
+    Q.q[i] = qv;
+    double c = q;
+    for (int k = 2; k <= kSeries; ++k) {
+        c *= (q - (double)(k - 1)) / (double)k;
+        Q.binom[i][k - 2] = c;
+    }
+    Q.inv_q1[i] = qv == 1.0f ? 0.0 : 1.0 / (q - 1.0);
+}
 
 bool host_affine_q16(const float prm[9], const int nf[3], const float sf[3], const int nm[3], const float sm[3],
                      int32_t q16[12]) {

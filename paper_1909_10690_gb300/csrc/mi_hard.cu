@@ -24,6 +24,7 @@
 // so the per-voxel arithmetic is exact in 32 bits.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "mi_internal.h"
@@ -882,12 +883,13 @@ __device__ __forceinline__ void load_zoff(const PairDev &P, float2 *s_zoff) {
 // Entropy reduction of one histogram by one CTA (Eq. 1, Eq. 2, Tsallis)
 // ---------------------------------------------------------------------------
 
-// Entropy terms of a count v < 2^31: v ln v (q == 1) or v^q, from the count-indexed table; beyond it, with m
-// the leading 16 bits of v, v = 2^e m (1 + x), 0 <= x < 2^-15, from the table's entries of m and 2^e and
-// the series of ln(1 + x) or (1 + x)^q, whose terms after the cubic are below 2^-54 of the result for
-// q <= 7 (larger q: pow).  FP64 units are few (two lanes a clock an SM, so a warp's instruction takes 16
-// clocks whatever its active lanes), and a log or a pow is some 50 or 250 instructions; the series takes
-// eight for x, shared by every q, and five per q.
+// Entropy terms of a count v < 2^31: v ln v (q == 1) or v^q, from the count-indexed table of 2^TB entries;
+// beyond it, with m the leading TB bits of v, v = 2^e m (1 + x), 0 <= x < 2^(1 - TB), from the table's
+// entries of m and 2^e and the series of ln(1 + x) or (1 + x)^q: three terms for a context's 65536 entries
+// (TB 16), eight for the 256 an evaluation without a context builds itself (TB 8), whose rest is below
+// 2^-54 of the result for q <= 7 (larger q: pow).  FP64 units are few (two lanes a clock an SM, so a
+// warp's instruction takes 16 clocks whatever its active lanes), and a log or a pow is some 50 or 250
+// instructions; the series takes eight for x, shared by every q, and five (ten) per q.
 __device__ __noinline__ double pow_term(double v, double q) { return pow(v, q); }
 
 struct Split {  // v = 2^e m (1 + x); e < 0: v is below the table's end
@@ -896,9 +898,10 @@ struct Split {  // v = 2^e m (1 + x); e < 0: v is below the table's end
     double x;
 };
 
+template <int TB>
 __device__ __forceinline__ Split split_count(uint32_t v) {
     Split s;
-    s.e = v < (uint32_t)kTab ? -1 : 16 - __clz((int)v);
+    s.e = v < (1u << TB) ? -1 : 32 - TB - __clz((int)v);
     if (s.e < 0) {
         s.m = v;
         s.x = 0.0;
@@ -906,33 +909,40 @@ __device__ __forceinline__ Split split_count(uint32_t v) {
     }
     s.m = v >> s.e;
     const double dm = (double)s.m;
-    double y = (double)__frcp_rn((float)s.m);  // 1 / m to 2^-24, then 2^-47: x keeps 2^-62
+    double y = (double)__frcp_rn((float)s.m);  // 1 / m to 2^-24, then 2^-47, then (for x < 2^-7) 2^-53
     y = fma(fma(-dm, y, 1.0), y, y);
+    if (TB < 16) y = fma(fma(-dm, y, 1.0), y, y);
     s.x = (double)(v - (s.m << s.e)) * y * __hiloint2double((1023 - s.e) << 20, 0);
     return s;
 }
 
+template <int TB>
 __device__ __forceinline__ double split_term(uint32_t v, const Split &s, int iq, const QSet &Q) {
+    constexpr int terms = TB == 16 ? 3 : kSeries;
+    static_assert(TB == 16 || TB == 8, "terms are chosen for these tables");
     const double *__restrict__ tab = Q.tab[iq];
     const double tm = __ldg(tab + s.m);
     if (s.e < 0) return tm;
     const float qf = Q.q[iq];
     const double x = s.x;
     if (qf == 1.0f) {
-        const double l = x * fma(-x, fma(-x, 1.0 / 3.0, 0.5), 1.0);
-        return fma((double)v, fma((double)s.e, 0.69314718055994530942, l), fma(x, tm, tm) * (double)(1u << s.e));
+        double l = 1.0 / terms;
+#pragma unroll
+        for (int k = terms - 1; k >= 1; --k) l = fma(-x, l, 1.0 / k);
+        return fma((double)v, fma((double)s.e, 0.69314718055994530942, x * l), fma(x, tm, tm) * (double)(1u << s.e));
     }
     if (qf > 7.0f) return pow_term((double)v, (double)qf);
-    const double t = tm * __ldg(tab + (1u << s.e));
-    return fma(t, x * fma(x, fma(x, Q.c3[iq], Q.c2[iq]), (double)qf), t);
+    double p = Q.binom[iq][terms - 2];
+#pragma unroll
+    for (int k = terms - 1; k >= 2; --k) p = fma(x, p, Q.binom[iq][k - 2]);
+    p = x * fma(x, p, (double)qf);
+    const double t = tm * __ldg(tab + (s.e < TB ? 1u << s.e : (1u << TB) + s.e - TB));
+    return fma(t, p, t);
 }
 
-__device__ __forceinline__ double term(uint32_t v, int iq, const QSet &Q) { return split_term(v, split_count(v), iq, Q); }
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
+template <int TB>
+__device__ __forceinline__ double term(uint32_t v, int iq, const QSet &Q) {
+    return split_term<TB>(v, split_count<TB>(v), iq, Q);
 }
 
 // Warp-wide FP64 sums of four values: lane l gets the sum of a[l & 3].  Half of the values change lanes in
@@ -947,32 +957,12 @@ __device__ __forceinline__ double warp_sum4(const double (&a)[4]) {
     return c;
 }
 
-// Block-wide FP64 sum of three values; every thread gets the results.
-__device__ __forceinline__ void block_sum3(double &a, double &b, double &c, double *s_red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    a = warp_sum(a);
-    b = warp_sum(b);
-    c = warp_sum(c);
-    __syncthreads();
-    if (lane == 0) {
-        s_red[3 * warp + 0] = a;
-        s_red[3 * warp + 1] = b;
-        s_red[3 * warp + 2] = c;
-    }
-    __syncthreads();
-    a = b = c = 0.0;
-    for (int w = 0; w < nwarps; ++w) {
-        a += s_red[3 * w + 0];
-        b += s_red[3 * w + 1];
-        c += s_red[3 * w + 2];
-    }
-}
-
 // Entropies and MI of transform t from the overlap count N and, per q, the sums S over the fixed marginal,
 // the moving marginal and the joint cells of c ln c (q == 1) or c^q: H = (N ln N - S) / N (Eq. 1),
 // S_q = (1 - S / N^q) / (q - 1), MI = H_F + H_M - H_FM (Eq. 2) plus (1 - q) S_q(F) S_q(M) in the
 // pseudo-additive form.  N ln N and N^q are the term of a cell that holds every voxel.  One warp: lane
 // 3 iq + w brings sum w of q iq (so every division is issued once).
+template <int TB>
 __device__ void write_mi(uint32_t N, double S, const QSet &Q, long long t, const Outputs &O) {
     const int lane = threadIdx.x & 31, nq = Q.nq;
     if (lane == 0) {
@@ -985,7 +975,7 @@ __device__ void write_mi(uint32_t N, double S, const QSet &Q, long long t, const
     if (N == 0) {
         h = __longlong_as_double(0x7ff8000000000000ll);
     } else {
-        const double full = term(N, iq, Q);
+        const double full = term<TB>(N, iq, Q);
         const bool shannon = qf == 1.0f;
         double unit = shannon ? (double)N : full;
         if (shannon && Q.bits) unit *= 0.69314718055994530942;
@@ -1015,7 +1005,9 @@ constexpr int kSmallCounts = 768;
 constexpr int kBigCounts = 255;
 
 // The shared words of a reduction (kReduceWords): cells per small count, then the listed counts.
+template <int TB>
 struct CountTable {
+    static constexpr uint32_t kBig = 1u << 16;  // counts listed (with TB 16 those beyond the table)
     uint32_t *small;  // null: no room, every term is taken on the way
     __device__ __forceinline__ uint32_t *nbig() const { return small + kSmallCounts; }
     __device__ __forceinline__ uint32_t *big() const { return small + kSmallCounts + 1; }
@@ -1030,7 +1022,7 @@ struct CountTable {
             atomicAdd(&small[v], 1u);
             return true;
         }
-        if (v < (uint32_t)kTab) return false;
+        if (v < kBig) return false;
         const uint32_t i = atomicAdd(nbig(), 1u);
         if (i >= (uint32_t)kBigCounts) return false;
         big()[i] = v;
@@ -1038,7 +1030,7 @@ struct CountTable {
     }
     // The same answer for a pass after the first (which lists large counts if there is room for all).
     __device__ __forceinline__ bool taken_before(uint32_t v) const {
-        return small && (v < (uint32_t)kSmallCounts || (v >= (uint32_t)kTab && *nbig() <= (uint32_t)kBigCounts));
+        return small && (v < (uint32_t)kSmallCounts || (v >= kBig && *nbig() <= (uint32_t)kBigCounts));
     }
     // This thread's share of the table's terms of q0 .. q0 + 3.
     __device__ __forceinline__ void add_terms(double (&a)[4], int q0, const QSet &Q) const {
@@ -1048,7 +1040,7 @@ struct CountTable {
             const uint32_t m = small[c];
             double tv[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tv[k] = m && q0 + k < Q.nq ? __ldg(Q.tab[q0 + k] + c) : 0.0;
+            for (int k = 0; k < 4; ++k) tv[k] = m && q0 + k < Q.nq ? term<TB>((uint32_t)c, q0 + k, Q) : 0.0;
             if (m) {
                 const double dm = (double)m;
 #pragma unroll
@@ -1060,17 +1052,17 @@ struct CountTable {
         for (int i = threadIdx.x; i < n; i += blockDim.x) add_count(a, big()[i], q0, Q);
     }
     __device__ __forceinline__ static void add_count(double (&a)[4], uint32_t v, int q0, const QSet &Q) {
-        const Split s = split_count(v);
+        const Split s = split_count<TB>(v);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (q0 + k < Q.nq) a[k] += split_term(v, s, q0 + k, Q);
+            if (q0 + k < Q.nq) a[k] += split_term<TB>(v, s, q0 + k, Q);
     }
 };
 static_assert(kSmallCounts + 1 + kBigCounts == kReduceWords, "the table fills its shared words");
 
 template <class Hist>
 __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *s_rows, uint32_t *s_cols,
-                                 double *s_red, CountTable C, long long t, const Outputs &O) {
+                                 double *s_red, CountTable<16> C, long long t, const Outputs &O) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int nq = Q.nq;
     double *s_res = s_red + 3 * 32;  // 3 nq results after the per-warp scratch
@@ -1093,7 +1085,7 @@ __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *
                 } else {
                     taken = C.taken_before(v);
                 }
-                if (!taken) CountTable::add_count(aj, v, q0, Q);
+                if (!taken) CountTable<16>::add_count(aj, v, q0, Q);
             }
             if (q0 == 0) {
                 rsum = __reduce_add_sync(kFull, rsum);
@@ -1113,7 +1105,7 @@ __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *
             const uint32_t *m = warp < 4 ? s_rows : s_cols;
             double am[4] = {0.0, 0.0, 0.0, 0.0};
             for (int x = (warp & 3) * 32 + lane; x < B; x += 128)
-                if (m[x]) CountTable::add_count(am, m[x], q0, Q);
+                if (m[x]) CountTable<16>::add_count(am, m[x], q0, Q);
             const double v = warp_sum4(am);
             if (lane < 4) s_marg[4 * warp + lane] = v;
         }
@@ -1139,7 +1131,7 @@ __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *
         uint32_t N = 0;  // fewer than 2^31 voxels
         for (int r = lane; r < B; r += 32) N += s_rows[r];
         N = __reduce_add_sync(kFull, N);
-        write_mi(N, lane < 3 * nq ? s_res[lane] : 0.0, Q, t, O);
+        write_mi<16>(N, lane < 3 * nq ? s_res[lane] : 0.0, Q, t, O);
     }
     __syncthreads();
 }
@@ -1167,8 +1159,10 @@ __device__ __forceinline__ double tree8(const double *v, int stride) {
            ((v[4 * stride] + v[5 * stride]) + (v[6 * stride] + v[7 * stride]));
 }
 
-__global__ void __launch_bounds__(kEntThreads)
-    k_entropy_slots(const uint32_t *__restrict__ hist, long long hist_stride, const Slot *__restrict__ slots,
+// TB: bits of the tables in Q.  slots null: one histogram, `single`.
+template <int TB>
+__global__ void __launch_bounds__(kEntThreads, 4)
+    k_entropy_slots(const uint32_t *__restrict__ hist, long long hist_stride, const Slot *__restrict__ slots, Slot single,
                     const __grid_constant__ QSet Q, unsigned int *__restrict__ done, double *__restrict__ part,
                     const __grid_constant__ Outputs O) {
     constexpr int nwarps = kEntThreads / 32;
@@ -1179,10 +1173,11 @@ __global__ void __launch_bounds__(kEntThreads)
     __shared__ bool s_last;
     const int slot = blockIdx.y, p = blockIdx.x, parts = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int t = slots[slot].t, B = slots[slot].bins, nq = Q.nq;
+    const Slot S0 = slots ? slots[slot] : single;
+    const int t = S0.t, B = S0.bins, nq = Q.nq;
     const uint32_t *h = hist + (size_t)slot * hist_stride;
     const bool few = B * B <= 2048 * parts;  // few cells: looked up on the way
-    CountTable C{few ? nullptr : s_words};
+    CountTable<TB> C{few ? nullptr : s_words};
     const int c0 = (int)((long long)B * p / parts), ncols = (int)((long long)B * (p + 1) / parts) - c0;
     const int nrows = (B - p + parts - 1) / parts;
     s_cols[tid] = 0;
@@ -1211,7 +1206,7 @@ __global__ void __launch_bounds__(kEntThreads)
                 } else {
                     taken = C.taken_before(v[k]);
                 }
-                if (!taken) CountTable::add_count(aj, v[k], q0, Q);
+                if (!taken) CountTable<TB>::add_count(aj, v[k], q0, Q);
             }
             if (q0 == 0) {
                 rsum = __reduce_add_sync(kFull, rsum);
@@ -1226,7 +1221,7 @@ __global__ void __launch_bounds__(kEntThreads)
         if ((warp & 3) * 32 < nline) {
             double am[4] = {0.0, 0.0, 0.0, 0.0};
             for (int i = tid & 127; i < nline; i += 128)
-                if (line[i]) CountTable::add_count(am, line[i], q0, Q);
+                if (line[i]) CountTable<TB>::add_count(am, line[i], q0, Q);
             m = warp_sum4(am);
         }
         C.add_terms(aj, q0, Q);
@@ -1271,7 +1266,7 @@ __global__ void __launch_bounds__(kEntThreads)
         S = tree8(&s_part[0][lane], 32);
         N = (uint32_t)__shfl_sync(kFull, S, 3 * nq);
     }
-    if (warp == 0) write_mi(N, S, Q, t, O);
+    if (warp == 0) write_mi<TB>(N, S, Q, t, O);
 }
 
 // ---------------------------------------------------------------------------
@@ -1358,7 +1353,7 @@ __global__ void __launch_bounds__(1024, 1)
                 for (int c = threadIdx.x & 31; c < B; c += 32) dh[r * B + c] = H.count(r, c);
         }
         reduce_entropies(H, P.bins, Q, (uint32_t *)(smem + L.rows), (uint32_t *)(smem + L.cols),
-                         (double *)(smem + L.red), CountTable{L.has_small ? (uint32_t *)(smem + L.small) : nullptr}, I.t, O);
+                         (double *)(smem + L.red), CountTable<16>{L.has_small ? (uint32_t *)(smem + L.small) : nullptr}, I.t, O);
     }
 }
 
@@ -1555,7 +1550,8 @@ cudaError_t launch_table(double *tab, float q, cudaStream_t s) {
 cudaError_t launch_entropy_slots(const uint32_t *d_hist, long long hist_stride, const Slot *d_slots, int nslots,
                                  int parts, const QSet &Q, unsigned int *d_done, double *d_part, const Outputs &O,
                                  cudaStream_t s) {
-    k_entropy_slots<<<dim3(parts, nslots), kEntThreads, 0, s>>>(d_hist, hist_stride, d_slots, Q, d_done, d_part, O);
+    k_entropy_slots<16><<<dim3(parts, nslots), kEntThreads, 0, s>>>(d_hist, hist_stride, d_slots, Slot{}, Q, d_done,
+                                                                    d_part, O);
     return cudaGetLastError();
 }
 
@@ -1618,9 +1614,9 @@ cudaError_t set_drain_cap(int cap) { return cudaMemcpyToSymbol(g_drain_cap, &cap
 
 // ===========================================================================
 // Allocation-free variant of the plain path (entry point in mi_noalloc.cu):
-// the fixed volume is binned on the fly from its raw values, the histogram
-// lives in caller-provided scratch (a static device array), and the entropy
-// terms are evaluated directly in FP64 instead of from count-indexed tables.
+// the fixed volume is binned on the fly from its raw values, and the
+// histogram, the entropy tables (256 entries a q) and the partial sums live
+// in caller-provided scratch (a static device array).
 // ===========================================================================
 
 namespace mi {
@@ -1658,167 +1654,88 @@ __device__ __forceinline__ int sample_hard_raw(const MovT *__restrict__ mov, int
     return lerp8(g0, g1, fz);
 }
 
+// Warp w of all takes rows w, w + warps, ...; 32 of them are clipped at once (lane l: its l-th).
 template <typename FixT, typename MovT, class Hist>
-__device__ void accumulate_rows_raw(const RawPair &P, const int *q, long long first_batch, long long batch_stride,
-                                    Hist &H) {
+__device__ void accumulate_rows_raw(const RawPair &P, const int *q, Hist &H) {
     const int lane = threadIdx.x & 31;
     const int nf0 = P.nf[0], nf1 = P.nf[1];
     const long long R = (long long)nf1 * P.nf[2];
+    const long long first = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                    warps = ((long long)gridDim.x * blockDim.x) >> 5;
     const int n0 = P.nm[0], n1 = P.nm[1], n2 = P.nm[2];
     const int st0 = q[0], st1 = q[4], st2 = q[8];
     const int bins = P.bins, mdepth = P.mdepth, fdepth = P.fdepth;
     const uint32_t fvmax = (uint32_t)((1ull << fdepth) - 1ull);
+    const int vmax = (int)((1u << mdepth) - 1u);
     const MovT *__restrict__ mov = (const MovT *)P.mov;
-    for (long long rb = first_batch * 32; rb < R; rb += batch_stride * 32) {
+    for (long long rb = first; rb < R; rb += 32 * warps) {
         RowClip mine;
         mine.lo = 0;
         mine.hi = -1;
         mine.u0 = mine.u1 = mine.u2 = 0;
-        const long long r = rb + lane;
-        if (r < R) mine = clip_row(q, (int)(r % nf1), (int)(r / nf1), nf0, P.nm);
+        const long long rl = rb + lane * warps;
+        if (rl < R) mine = clip_row(q, (int)(rl % nf1), (int)(rl / nf1), nf0, P.nm);
         for (int s = 0; s < 32; ++s) {
+            const long long r = rb + s * warps;
+            if (r >= R) break;  // warp-uniform
             const int lo = __shfl_sync(kFull, mine.lo, s), hi = __shfl_sync(kFull, mine.hi, s);
             if (lo > hi) continue;
             const int U0 = __shfl_sync(kFull, mine.u0, s), U1 = __shfl_sync(kFull, mine.u1, s),
                       U2 = __shfl_sync(kFull, mine.u2, s);
-            const FixT *__restrict__ frow = (const FixT *)P.fix + (size_t)(rb + s) * nf0;
-            for (int i0 = lo; i0 <= hi; i0 += 32) {
-                const int i = i0 + lane;
-                const bool valid = i <= hi;
-                int bf = 0, bm = 0;
-                if (valid) {
-                    const int d = i - lo;
-                    // volumes are read in place; each value is clamped to its bit depth as it is read
-                    const int v = sample_hard_raw<MovT>(mov, n0, n1, n2, U0 + st0 * d, U1 + st1 * d, U2 + st2 * d,
-                                                        (int)((1u << mdepth) - 1u));
-                    bm = (v * bins) >> mdepth;
-                    uint32_t fv = (uint32_t)__ldg(frow + i);
-                    fv = fv > fvmax ? fvmax : fv;
-                    bf = (int)((fv * (uint32_t)bins) >> fdepth);
-                }
-                H.add(bf, bm, valid);
+            const FixT *__restrict__ frow = (const FixT *)P.fix + (size_t)r * nf0;
+#pragma unroll 2
+            for (int i = lo + lane; i <= hi; i += 32) {
+                const int d = i - lo;
+                // volumes are read in place; each value is clamped to its bit depth as it is read
+                const int v = sample_hard_raw<MovT>(mov, n0, n1, n2, U0 + st0 * d, U1 + st1 * d, U2 + st2 * d, vmax);
+                uint32_t fv = (uint32_t)__ldg(frow + i);
+                fv = fv > fvmax ? fvmax : fv;
+                H.add((int)((fv * (uint32_t)bins) >> fdepth), (v * bins) >> mdepth, true);
             }
         }
     }
 }
 
-template <typename FixT, typename MovT>
-__global__ void __launch_bounds__(1024, 1) k_hist_raw(RawPair P, Q12 A, uint32_t *__restrict__ ghist, int *flags) {
+// 32-bit counters up to kRawU32Bins bins, drained 16-bit ones above (where the 32-bit ones leave the L1
+// too little for the volumes, then do not fit).  What bounds it is the latency of the eight scattered
+// loads a voxel, so every warp of every SM takes rows: with batches of 32 rows a warp, a 192 x 192 x 128
+// volume's 24576 rows occupied 768 of the 4864 warps and the kernel took 148 us; now 33.
+// The first lanes of each CTA build the entropy tables on the way.
+constexpr int kRawU32Bins = 160;
+
+template <typename FixT, typename MovT, int HV>
+__global__ void __launch_bounds__(1024, 1)
+    k_hist_raw(RawPair P, Q12 A, const __grid_constant__ QSet Q, NoallocScratch *__restrict__ D) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = P.bins;
-    const SmemLayout L = smem_layout(HV_U16_MATCH, B, blockDim.x, 0, 0);
+    const SmemLayout L = smem_layout(HV, B, blockDim.x, 0, 0);
     __shared__ int q[12];
     if (threadIdx.x < 12) q[threadIdx.x] = A.q[threadIdx.x];
-    auto H = make_hist<HV_U16_MATCH>(smem, L, B, flags);
+    auto H = make_hist<HV>(smem, L, B, D->flags);
     H.zero();
+    // entry c < 256: c ln c or c^q; entry 256 + i: that of 2^(8 + i)
+    constexpr int entries = 256 + 16;
+    for (int x = threadIdx.x * gridDim.x + blockIdx.x; x < entries * Q.nq; x += blockDim.x * gridDim.x) {
+        const int iq = x / entries, c = x % entries;
+        const double d = c < 256 ? (double)c : (double)(1u << (c - 248));
+        D->tab[iq][c] = c == 0 ? 0.0 : Q.q[iq] == 1.0f ? d * log(d) : pow(d, (double)Q.q[iq]);
+    }
     __syncthreads();
     const int nwarps = blockDim.x >> 5;
-    accumulate_rows_raw<FixT, MovT>(P, q, (long long)blockIdx.x * nwarps + (threadIdx.x >> 5),
-                                    (long long)gridDim.x * nwarps, H);
+    accumulate_rows_raw<FixT, MovT>(P, q, H);
     __syncthreads();
     for (int r = threadIdx.x >> 5; r < B; r += nwarps)
         for (int c = threadIdx.x & 31; c < B; c += 32) {
             const uint32_t v = H.count(r, c);
-            if (v) atomicAdd(ghist + r * B + c, v);
+            if (v) atomicAdd(D->hist + r * B + c, v);
         }
-}
-
-// Entropy term of one count, evaluated directly in FP64: c ln c or c^q.
-__device__ __forceinline__ double term_direct(uint32_t v, float qf) {
-    const double d = (double)v;
-    return qf == 1.0f ? d * log(d) : pow(d, (double)qf);
-}
-
-// One CTA: marginals, FP64 sums per q and MI from a global histogram.
-// out: nq MI values, then nq x 3 entropies, then the overlap count (as a double).
-__global__ void __launch_bounds__(1024, 1)
-    k_entropy_direct(const uint32_t *__restrict__ ghist, int B, QSet Q, double *__restrict__ out, int *flags) {
-    __shared__ uint32_t s_rows[256], s_cols[256];
-    __shared__ double s_red[3 * 32];
-    __shared__ double s_res[3 * kMaxQ + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    for (int c = tid; c < B; c += blockDim.x) s_cols[c] = 0;
-    __syncthreads();
-    for (int r = warp; r < B; r += nwarps) {
-        uint32_t rsum = 0;
-        for (int c = lane; c < B; c += 32) {
-            const uint32_t v = __ldg(ghist + r * B + c);
-            if (v) {
-                rsum += v;
-                atomicAdd(&s_cols[c], v);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rsum += __shfl_xor_sync(kFull, rsum, o);
-        if (lane == 0) s_rows[r] = rsum;
-    }
-    __syncthreads();
-    {
-        double n0 = 0.0, z1 = 0.0, z2 = 0.0;
-        for (int r = tid; r < B; r += blockDim.x) n0 += (double)s_rows[r];
-        block_sum3(n0, z1, z2, s_red);
-        if (tid == 0) s_res[3 * kMaxQ] = n0;
-    }
-    for (int iq = 0; iq < Q.nq; ++iq) {
-        double aj = 0.0, af = 0.0, am = 0.0;
-        for (int c = tid; c < B * B; c += blockDim.x) {
-            const uint32_t v = __ldg(ghist + c);
-            if (v) aj += term_direct(v, Q.q[iq]);
-        }
-        for (int r = tid; r < B; r += blockDim.x) {
-            if (s_rows[r]) af += term_direct(s_rows[r], Q.q[iq]);
-            if (s_cols[r]) am += term_direct(s_cols[r], Q.q[iq]);
-        }
-        block_sum3(af, am, aj, s_red);
-        if (tid == 0) {
-            s_res[3 * iq + 0] = af;
-            s_res[3 * iq + 1] = am;
-            s_res[3 * iq + 2] = aj;
-        }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const double N = s_res[3 * kMaxQ];
-        out[4 * Q.nq] = N;
-        if (N <= 0.0) atomicOr(&flags[0], 1);
-        for (int iq = 0; iq < Q.nq; ++iq) {
-            const float qf = Q.q[iq];
-            const double SF = s_res[3 * iq + 0], SM = s_res[3 * iq + 1], SJ = s_res[3 * iq + 2];
-            double hf, hm, hj;
-            if (N <= 0.0) {
-                hf = hm = hj = __longlong_as_double(0x7ff8000000000000ll);
-            } else if (qf == 1.0f) {
-                const double lnN = log(N);
-                hf = lnN - SF / N;
-                hm = lnN - SM / N;
-                hj = lnN - SJ / N;
-                if (Q.bits) {
-                    const double l2 = log(2.0);
-                    hf /= l2;
-                    hm /= l2;
-                    hj /= l2;
-                }
-            } else {
-                const double qd = (double)qf, Nq = pow(N, -qd);
-                hf = (1.0 - Nq * SF) / (qd - 1.0);
-                hm = (1.0 - Nq * SM) / (qd - 1.0);
-                hj = (1.0 - Nq * SJ) / (qd - 1.0);
-            }
-            double I = hf + hm - hj;
-            if (qf != 1.0f && Q.form == 1) I += (1.0 - (double)qf) * hf * hm;
-            out[iq] = I;
-            out[Q.nq + 3 * iq + 0] = hf;
-            out[Q.nq + 3 * iq + 1] = hm;
-            out[Q.nq + 3 * iq + 2] = hj;
-        }
-    }
 }
 
 }  // namespace
 
 cudaError_t launch_noalloc_eval(const void *fix, int fdtype, int fdepth, const void *mov, int mdtype, int mdepth,
-                                const int nf[3], const int nm[3], int bins, const int32_t q16[12], const QSet &Q,
-                                uint32_t *hist, int *flags, double *out, int ctas, cudaStream_t s) {
+                                const int nf[3], const int nm[3], int bins, const int32_t q16[12], QSet Q,
+                                NoallocScratch *d, int sms, cudaStream_t s) {
     RawPair P;
     P.fix = fix;
     P.mov = mov;
@@ -1831,23 +1748,39 @@ cudaError_t launch_noalloc_eval(const void *fix, int fdtype, int fdepth, const v
     P.mdepth = mdepth;
     Q12 A;
     for (int e = 0; e < 12; ++e) A.q[e] = q16[e];
+    for (int i = 0; i < Q.nq; ++i) Q.tab[i] = d->tab[i];
     const int threads = 1024;
-    const size_t smem = smem_layout(HV_U16_MATCH, bins, threads, 0, 0).total;
-    cudaError_t e = cudaMemsetAsync(hist, 0, (size_t)bins * bins * sizeof(uint32_t), s);
+    const long long rows = (long long)nf[1] * nf[2], all = (rows + 31) / 32;  // a row a warp at least
+    const int ctas = (int)(all < sms ? all : sms);
+    const bool u32 = bins <= kRawU32Bins;
+    const size_t smem = smem_layout(u32 ? HV_U32 : HV_U16, bins, threads, 0, 0).total;
+    cudaError_t e = cudaMemsetAsync(d, 0, offsetof(NoallocScratch, hist) + (size_t)bins * bins * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(flags, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
-#define MI_RAW(FT, MT)                                                                     \
+#define MI_RAW_H(FT, MT, HV)                                                                \
     do {                                                                                   \
-        if ((e = set_smem(k_hist_raw<FT, MT>, smem)) != cudaSuccess) return e;            \
-        k_hist_raw<FT, MT><<<ctas, threads, smem, s>>>(P, A, hist, flags);                 \
+        if ((e = set_smem(k_hist_raw<FT, MT, HV>, smem)) != cudaSuccess) return e;         \
+        k_hist_raw<FT, MT, HV><<<ctas, threads, smem, s>>>(P, A, Q, d);                    \
+    } while (0)
+#define MI_RAW(FT, MT)                  \
+    do {                                \
+        if (u32) MI_RAW_H(FT, MT, HV_U32); \
+        else MI_RAW_H(FT, MT, HV_U16);  \
     } while (0)
     if (fdtype == 0 && mdtype == 0) MI_RAW(uint8_t, uint8_t);
     else if (fdtype == 0) MI_RAW(uint8_t, uint16_t);
     else if (mdtype == 0) MI_RAW(uint16_t, uint8_t);
     else MI_RAW(uint16_t, uint16_t);
 #undef MI_RAW
+#undef MI_RAW_H
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_entropy_direct<<<1, 1024, 0, s>>>(hist, bins, Q, out, flags);
+    Outputs O;
+    O.mi = d->mi;
+    O.h = nullptr;
+    O.count = nullptr;
+    O.dump = nullptr;
+    O.flags = d->flags;
+    k_entropy_slots<8><<<dim3(entropy_parts(bins, 1, sms), 1), kEntThreads, 0, s>>>(d->hist, 0, nullptr, Slot{0, bins}, Q,
+                                                                                    &d->done, d->part, O);
     return cudaGetLastError();
 }
 

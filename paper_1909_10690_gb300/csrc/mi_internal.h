@@ -9,6 +9,7 @@ namespace mi {
 
 constexpr int kMaxQ = 8;
 constexpr int kTab = 65536;        // count-indexed FP64 tables cover counts < kTab
+constexpr int kSeries = 8;         // terms of (1 + x)^q kept at most
 constexpr int kDrainT = 1 << 14;   // 16-bit counters are drained once they reach 2^14
 constexpr int kOvfSlots = 4096;    // drain table entries (each entry holds >= kDrainT counts)
 
@@ -35,7 +36,8 @@ struct PairDev {
 };
 
 // q values of one call with their count-indexed FP64 tables
-// tab[i][c] = c ln c (q == 1) or c^q (q != 1), c < kTab.
+// tab[i][c] = c ln c (q == 1) or c^q (q != 1), c < kTab (or, without a context, c < 256 and then the
+// entries of 2^8 .. 2^23).
 struct QSet {
     int nq;
     int form;   // 0 additive, 1 pseudo-additive Tsallis MI
@@ -43,7 +45,7 @@ struct QSet {
     int pad;
     float q[kMaxQ];
     const double *tab[kMaxQ];
-    double c2[kMaxQ], c3[kMaxQ];  // q (q - 1) / 2 and q (q - 1) (q - 2) / 6
+    double binom[kMaxQ][kSeries - 1];  // C(q, k), k = 2 .. kSeries
     double inv_q1[kMaxQ];         // 1 / (q - 1) (0 for q == 1)
 };
 
@@ -221,13 +223,25 @@ cudaError_t launch_parzen_adjoint(const ParzenLaunch &L, const ParzenAffine *d_a
                                   int ctas, const float *d_w, const unsigned long long *d_count, double *d_mom,
                                   double *d_grad, cudaStream_t s);
 
+// The host-side part of a QSet: q and what the kernels derive from it (not the tables).
+void set_q(QSet &Q, int i, float qv);
+
 // ---- allocation-free evaluation (mi_noalloc.cu) ---------------------------
-// Plain-path variant that bins the fixed volume on the fly and keeps its
-// histogram (bins^2 u32), flags (2 int) and results (4 nq + 1 doubles) in
-// caller-provided device memory.
+// Device memory of one evaluation: what the kernels add to (cleared by the launcher), then their results
+// and tables.
+struct NoallocScratch {
+    int flags[2];        // [0] empty overlap, [1] drain failure
+    unsigned int done;   // finished parts of the entropy kernel
+    int pad;
+    uint32_t hist[256 * 256];
+    double mi[kMaxQ];    // directly after what is cleared
+    double part[25 * 32];
+    double tab[kMaxQ][256 + 16];
+};
+// Plain-path variant that bins the fixed volume on the fly and keeps everything in *d (device memory).
 cudaError_t launch_noalloc_eval(const void *fix, int fdtype, int fdepth, const void *mov, int mdtype, int mdepth,
-                                const int nf[3], const int nm[3], int bins, const int32_t q16[12], const QSet &Q,
-                                uint32_t *hist, int *flags, double *out, int ctas, cudaStream_t s);
+                                const int nf[3], const int nm[3], int bins, const int32_t q16[12], QSet Q,
+                                NoallocScratch *d, int sms, cudaStream_t s);
 // The context path's parameter -> 16.16 affine builder (false if an entry does not fit).
 bool host_affine_q16(const float prm[9], const int nf[3], const float sf[3], const int nm[3], const float sm[3],
                      int32_t q16[12]);

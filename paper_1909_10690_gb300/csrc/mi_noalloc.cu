@@ -23,18 +23,12 @@
 
 namespace {
 
-// Scratch layout: histogram (256 x 256 u32), then flags (2 int, padded to
-// 256 bytes), then results (4 nq + 1 <= 33 doubles, padded).
-constexpr size_t kHistBytes = (size_t)MI_NOALLOC_MAX_BINS * MI_NOALLOC_MAX_BINS * sizeof(uint32_t);
-constexpr size_t kFlagsOffset = kHistBytes;
-constexpr size_t kOutOffset = kHistBytes + 256;
-constexpr size_t kScratchBytes = kOutOffset + 512;
-
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
+static_assert(MI_NOALLOC_MAX_BINS == 256 && MI_MAX_Q == mi::kMaxQ, "the static scratch is sized for these");
+static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(mi::NoallocScratch)];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
-unsigned char *g_scratch_addr[kMaxDevices] = {};
+mi::NoallocScratch *g_scratch_addr[kMaxDevices] = {};
 int g_sms[kMaxDevices] = {};
 
 mi_status fail(mi_status st, const char *msg) {
@@ -120,7 +114,7 @@ extern "C" mi_status mi_eval_noalloc(const mi_volume *fixed, const mi_volume *mo
         const float v = q[i];
         if (!(v > 0.0f) || !isfinite(v) || (v != 1.0f && fabsf(v - 1.0f) < 1e-6f))
             return fail(MI_EINVAL, "q values must be finite, > 0 and not within 1e-6 of 1 (use 1 for Shannon)");
-        Q.q[i] = v;
+        mi::set_q(Q, i, v);
     }
     for (int i = 0; i < 9; ++i)
         if (!isfinite(transform[i])) return fail(MI_EINVAL, "transform is not finite");
@@ -128,7 +122,7 @@ extern "C" mi_status mi_eval_noalloc(const mi_volume *fixed, const mi_volume *mo
     if (!mi::host_affine_q16(transform, fixed->dims, fixed->spacing_mm, moving->dims, moving->spacing_mm, q16))
         return fail(MI_ERANGE, "affine does not fit 16.16 fixed point");
     // ---- set-up, once per device (this device is current) ------------------
-    unsigned char *scratch;
+    mi::NoallocScratch *scratch;
     int sms;
     {
         std::lock_guard<std::mutex> lock(g_setup_mutex);
@@ -139,7 +133,7 @@ extern "C" mi_status mi_eval_noalloc(const mi_volume *fixed, const mi_volume *mo
             int n = 0;
             e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
             if (e != cudaSuccess) return fail_cuda(e, "reading the SM count");
-            g_scratch_addr[dev] = (unsigned char *)p;
+            g_scratch_addr[dev] = (mi::NoallocScratch *)p;
             g_sms[dev] = n;
         }
         scratch = g_scratch_addr[dev];
@@ -147,20 +141,13 @@ extern "C" mi_status mi_eval_noalloc(const mi_volume *fixed, const mi_volume *mo
     }
     // ---- work: the histogram and flags are cleared inside the launcher -----
     cudaStream_t s = (cudaStream_t)stream;
-    const long long rows = (long long)fixed->dims[1] * fixed->dims[2];
-    long long ctas = rows / (32 * 8);
-    if (ctas > sms) ctas = sms;
-    if (ctas < 1) ctas = 1;
-    uint32_t *hist = (uint32_t *)scratch;
-    int *flags = (int *)(scratch + kFlagsOffset);
-    double *out = (double *)(scratch + kOutOffset);
     e = mi::launch_noalloc_eval(fixed->data, fixed->dtype, fdepth, moving->data, moving->dtype, mdepth, fixed->dims,
-                                moving->dims, bins, q16, Q, hist, flags, out, (int)ctas, s);
+                                moving->dims, bins, q16, Q, scratch, sms, s);
     if (e != cudaSuccess) return fail_cuda(e, "mi_eval_noalloc kernels");
     int hflags[2] = {0, 0};
-    if ((e = cudaMemcpyAsync(out_mi, out, (size_t)nq * sizeof(double), cudaMemcpyDefault, s)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(out_mi, scratch->mi, (size_t)nq * sizeof(double), cudaMemcpyDefault, s)) != cudaSuccess)
         return fail_cuda(e, "copying results");
-    if ((e = cudaMemcpyAsync(hflags, flags, sizeof hflags, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(hflags, scratch->flags, sizeof hflags, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return fail_cuda(e, "reading flags");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail_cuda(e, "mi_eval_noalloc");
     if (hflags[1]) return fail(MI_ECUDA, "internal: 16-bit counter drain failed");

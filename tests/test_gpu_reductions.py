@@ -77,3 +77,29 @@ def test_split_pairs_of_unequal_size(cuda_lib, fraction):
         assert cnt[t] == cw[0]
         np.testing.assert_allclose(mi[t], want[0], rtol=0, atol=1e-11)
         np.testing.assert_allclose(h[t], hw[0], rtol=0, atol=1e-11)
+
+
+@pytest.mark.parametrize("shape,dtype,depth,bins", [((2, 2, 2), np.uint8, 8, 2), ((5, 7, 33), np.uint16, 16, 256),
+                                                    ((40, 44, 52), np.uint16, 12, 160), ((40, 44, 52), np.uint16, 12, 161),
+                                                    ((64, 64, 64), np.uint8, 7, 32)])
+def test_noalloc_rows_counters_and_terms(cuda_lib, shape, dtype, depth, bins):
+    """The allocation-free call against the oracle: fewer rows than warps and many, 32- and 16-bit counters
+    at the bin count where they change, a depth below the type's, counts below 256, in the series' range
+    and (one cell of a constant pair) at the volume's size, q above the series' range."""
+    import torch
+
+    rng = np.random.default_rng(70)
+    if min(shape) < 8:
+        f, m = (rng.integers(0, 1 << depth, shape).astype(dtype) for _ in range(2))
+    else:
+        f, m = (v.astype(dtype) for v in phantoms.head_pair(shape=shape, spacing=(1, 1, 1), seed=71, depth=depth, dtype=dtype))
+    qs = [1.0, 0.5, 1.5, 2.0, 7.0, 8.5]
+    prm = np.concatenate([phantoms.identity_params(1), phantoms.random_transforms(2, seed=72, t_mm=0.5, r_deg=6, s_range=(0.95, 1.05))])
+    for a, b in ((f, m), (np.zeros_like(f), np.zeros_like(m))):
+        mi_o, h_o, cnt = oracle.mi_eval(a, b, bins, prm, qs, fixed_depth=depth, moving_depth=depth, nthreads=8)
+        ad, bd = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+        for t in range(len(prm)):
+            if cnt[t] == 0:
+                continue
+            got = cuda_lib.eval_noalloc(ad, bd, bins, prm[t], qs, fixed_depth=depth, moving_depth=depth)
+            assert np.all(np.abs(got - mi_o[t]) <= 1e-6 * np.maximum(np.abs(mi_o[t]), h_o[t, :, 2]) + 1e-12)
