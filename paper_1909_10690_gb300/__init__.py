@@ -78,6 +78,15 @@ class _Arg:
             self.obj, self.ptr, self.on_gpu = a, a.ctypes.data, False
 
 
+def _wait_for(*args):
+    """Waits for the torch work that produces device inputs (and last used the memory of outputs allocated
+    beside them): a context works on a stream of its own, which nothing orders after torch's."""
+    for a in args:
+        if a.on_gpu:
+            _torch().cuda.current_stream(a.obj.device).synchronize()
+            return
+
+
 def _np_dtype(x):
     if _is_torch(x):
         torch = _torch()
@@ -191,6 +200,7 @@ class Context:
             bins_arr[i] = int(p["bins"])
             self.shapes.append(tuple(p["fixed"].shape))
             self.bins.append(int(p["bins"]))
+        _wait_for(*keep)
         if batch:
             st = self._lib.mi_batch_create(ctypes.byref(self._h), fx, mv, ctypes.cast(bins_arr, ctypes.c_void_p), n,
                                            ctypes.byref(opt))
@@ -233,6 +243,7 @@ class Context:
         mi = _out((n, nq), gpu, np.float64, dev)
         h = _out((n, nq, 3), gpu, np.float64, dev) if with_entropies and self.kernel != "parzen" else None
         cnt = _out((n,), gpu, np.int64, dev) if with_entropies else None
+        _wait_for(T, Q)
         st = self._lib.mi_eval(self._h, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
         self._check(st, allow_empty)
         return (mi, h, cnt) if with_entropies else mi
@@ -247,6 +258,7 @@ class Context:
         mi = _out((n, nq), gpu, np.float64, dev)
         h = _out((n, nq, 3), gpu, np.float64, dev) if with_entropies else None
         cnt = _out((n,), gpu, np.int64, dev) if with_entropies else None
+        _wait_for(A, Q)
         st = self._lib.mi_eval_q16(self._h, A.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
         self._check(st, allow_empty)
         return (mi, h, cnt) if with_entropies else mi
@@ -262,6 +274,7 @@ class Context:
         mi = _out((n, nq), gpu, np.float64, dev)
         h = _out((n, nq, 3), gpu, np.float64, dev) if with_entropies else None
         cnt = _out((n,), gpu, np.int64, dev) if with_entropies else None
+        _wait_for(P, T, Q)
         st = self._lib.mi_batch_eval(self._h, P.ptr, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
         self._check(st, allow_empty)
         return (mi, h, cnt) if with_entropies else mi
@@ -276,6 +289,7 @@ class Context:
         dev = T.obj.device if gpu else None
         mi = _out((n, nq), gpu, np.float64, dev)
         g = _out((n, nq, self.nparams), gpu, np.float64, dev)
+        _wait_for(T, Q)
         st = self._lib.mi_grad(self._h, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(g))
         self._check(st, allow_empty)
         return mi, g
@@ -292,6 +306,7 @@ class Context:
         dev = T.obj.device if gpu else None
         mi = _out((n, nq), gpu, np.float64, dev)
         g = _out((n, nq, self.nparams), gpu, np.float64, dev)
+        _wait_for(P, T, Q)
         st = self._lib.mi_batch_grad(self._h, P.ptr, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(g))
         self._check(st, allow_empty)
         return mi, g
@@ -304,6 +319,7 @@ class Context:
         n = int(np.prod(src.obj.shape) // (self.nparams if transforms is not None else 12))
         B = self.bins[pair]
         out = np.empty((n, B, B), dtype=np.uint32)
+        _wait_for(src)
         st = self._lib.mi_hist(self._h, pair, src.ptr if transforms is not None else None,
                                src.ptr if affines is not None else None, n, int(path), out.ctypes.data)
         self._check(st)
