@@ -357,15 +357,18 @@ struct mi_ctx {
     // per-q FP64 tables, keyed by the float bits of q
     std::map<uint32_t, std::unique_ptr<DevBuf>> tables;
     // call scratch
-    // (d_in: affines, work items and slots of a call, staged in h_in or v_in; d_work: the zeroed workspace of a
-    // launch: ticket, slot counters, slot histograms; d_part: partial entropy sums)
-    DevBuf d_aff, d_in, d_mi, d_h, d_cnt, d_flags, d_work, d_part, d_dump;
+    // (d_in: affines, work items and slots of a call, staged in h_in or v_in; d_work: its results, then what a
+    // launch needs cleared: flags, ticket, slot counters, slot histograms; d_part: partial entropy sums)
+    DevBuf d_aff, d_in, d_work, d_part, d_dump;
     HostBuf h_in, h_read;
-    std::vector<char> v_in;  // the same staging where no graph replays it
+    std::vector<char> v_in, v_out;  // the same staging where no graph replays it, and the results'
+    std::vector<Choice> cands;      // the hard path's candidates (fixed by the pairs and options)
     // Parzen: the pairs' descriptors (device array), per-call pair indices and row offsets, scratch
-    DevBuf p_pairs, p_pair_of, p_row_start;
+    DevBuf p_pairs;
     int p_bmax = 0, p_nxmax = 0;
-    DevBuf p_aff, p_jac, p_hist, p_cnt, p_marg, p_ment, p_mterm, p_jsum, p_w, p_mom, p_grad;
+    // (p_in: affines, Jacobians and, for several pairs, pair indices and row offsets; p_out: overlap counts,
+    // MI, gradients)
+    DevBuf p_in, p_out, p_hist, p_marg, p_ment, p_mterm, p_jsum, p_w, p_mom;
     // autotune and graph caches
     std::map<std::tuple<int, int, int>, Choice> tuned;  // (path, pair-or--1, n bucket)
     std::map<std::string, std::unique_ptr<GraphEntry>> graphs;
@@ -917,7 +920,6 @@ mi_status create_common(mi_ctx **out, const mi_volume *fixed, const mi_volume *m
             g_create_error = ctx->err;
             return st;
         }
-        MI_CU(ctx->d_flags.ensure(2 * sizeof(int)), "allocating flags");
     }
     *out = ctx.release();
     return MI_OK;
@@ -1014,6 +1016,43 @@ mi_status deliver(mi_ctx *ctx, void *dst, const void *src, size_t bytes) {
     MI_CU(cudaMemcpyAsync(dst, src, bytes, is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                           ctx->stream),
           "copying results");
+    return MI_OK;
+}
+
+// One result of a call: `bytes` at offset `at` of a device buffer, for the caller's pointer (host or device
+// memory, or null: not wanted).
+struct Result {
+    void *dst;
+    size_t at, bytes;
+};
+
+// Copies a call's results out of `base` in stream order, waits for the stream and fills the host ones: those
+// come in one copy through `staging` (pinned, at least as long as the buffer's results) or, without it,
+// through pageable memory of the context.  A copy each to pageable memory waited four times a call.
+mi_status deliver_all(mi_ctx *ctx, const char *base, const Result *res, int nres, char *staging) {
+    size_t lo = SIZE_MAX, hi = 0;
+    bool on_host[8] = {};
+    for (int i = 0; i < nres; ++i) {
+        if (!res[i].dst || res[i].bytes == 0) continue;
+        if (is_device_ptr(res[i].dst)) {
+            MI_CU(cudaMemcpyAsync(res[i].dst, base + res[i].at, res[i].bytes, cudaMemcpyDeviceToDevice, ctx->stream),
+                  "copying results");
+        } else {
+            on_host[i] = true;
+            lo = std::min(lo, res[i].at);
+            hi = std::max(hi, res[i].at + res[i].bytes);
+        }
+    }
+    if (hi > lo) {
+        if (!staging) {
+            ctx->v_out.resize(hi);
+            staging = ctx->v_out.data();
+        }
+        MI_CU(cudaMemcpyAsync(staging + lo, base + lo, hi - lo, cudaMemcpyDeviceToHost, ctx->stream), "copying results");
+    }
+    MI_CU(cudaStreamSynchronize(ctx->stream), "evaluation");
+    for (int i = 0; i < nres; ++i)
+        if (on_host[i]) memcpy(res[i].dst, staging + res[i].at, res[i].bytes);
     return MI_OK;
 }
 
@@ -1175,10 +1214,10 @@ cudaError_t record_event(cudaEvent_t ev, cudaStream_t s) {
 }
 
 // One launch of the hard-path kernel over whole items (the autotuner's unit).
-mi_status launch_whole(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, const QSet &Q,
+mi_status launch_whole(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, int *d_ticket, const QSet &Q,
                        const Outputs &O, const Choice &ch) {
-    MI_CU(cudaMemsetAsync(ctx->d_work.p, 0, 2 * sizeof(int), ctx->stream), "resetting the work queue");
-    MI_CU(launch_batched(ctx->d_pairs.as<PairDev>(), d_aff, d_items, nitems, ctx->d_work.as<int>(), ctx->max_bins,
+    MI_CU(cudaMemsetAsync(d_ticket, 0, 2 * sizeof(int), ctx->stream), "resetting the work queue");
+    MI_CU(launch_batched(ctx->d_pairs.as<PairDev>(), d_aff, d_items, nitems, d_ticket, ctx->max_bins,
                          ctx->max_rows_words, ctx->max_zplanes, ch.variant, ch.threads, ch.ctas, ch.tile, Q, O, nullptr,
                          0, ctx->stream),
           "batched kernel");
@@ -1266,8 +1305,8 @@ void cache_store(const std::string &path, const std::string &key, const Choice &
 // Autotune: time every candidate on the first items of this call (up to three
 // waves, so that effects that build up across waves, such as CTAs drifting to
 // different parts of the volumes, show in the timing).
-mi_status autotune(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, const QSet &Q, const Outputs &O,
-                   Choice &best, const std::vector<Choice> &cands) {
+mi_status autotune(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, int *d_ticket, const QSet &Q,
+                   const Outputs &O, Choice &best, const std::vector<Choice> &cands) {
     if (cands.empty()) return ctx->fail(MI_EUNSUPPORTED, "no histogram variant fits this bin count and volume size");
     if (cands.size() == 1 || !ctx->opt.autotune) {
         best = cands.front();
@@ -1287,7 +1326,7 @@ mi_status autotune(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int n
     auto time_per_item = [&](const Choice &c, int items, float &ms) -> mi_status {
         Choice cc = c;
         cudaEventRecord(e0, ctx->stream);
-        mi_status st = launch_whole(ctx, d_aff, d_items, items, Q, Ot, cc);
+        mi_status st = launch_whole(ctx, d_aff, d_items, items, d_ticket, Q, Ot, cc);
         if (st != MI_OK) return st;
         cudaEventRecord(e1, ctx->stream);
         cudaError_t e = cudaEventSynchronize(e1);
@@ -1300,7 +1339,7 @@ mi_status autotune(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int n
     mi_status st = MI_OK;
     for (size_t i = 0; i < cands.size() && st == MI_OK; ++i) {
         Choice cc = cands[i];
-        if ((st = launch_whole(ctx, d_aff, d_items, std::min(nitems, 8), Q, Ot, cc)) != MI_OK) break;  // warm-up
+        if ((st = launch_whole(ctx, d_aff, d_items, std::min(nitems, 8), d_ticket, Q, Ot, cc)) != MI_OK) break;  // warm-up
         float ms = 0;
         if ((st = time_per_item(cands[i], std::min(nitems, cands[i].ctas), ms)) == MI_OK) first.push_back({ms, i});
     }
@@ -1340,25 +1379,31 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     QSet Q;
     mi_status st = make_qset(ctx, qv, nq, Q);
     if (st != MI_OK) return st;
-    MI_CU(ctx->d_mi.ensure((size_t)n * nq * 8), "allocating outputs");
-    MI_CU(ctx->d_h.ensure((size_t)n * nq * 3 * 8), "allocating outputs");
-    MI_CU(ctx->d_cnt.ensure((size_t)n * 8), "allocating outputs");
-    MI_CU(cudaMemsetAsync(ctx->d_flags.p, 0, 2 * sizeof(int), ctx->stream), "resetting flags");
-    Outputs O;
-    O.mi = ctx->d_mi.as<double>();
-    O.h = ctx->d_h.as<double>();
-    O.count = ctx->d_cnt.as<long long>();
-    O.dump = R.dump;
-    O.flags = ctx->d_flags.as<int>();
     const bool multi = ctx->pairs.size() > 1;
     int path = R.path;
     if (path == MI_PATH_AUTO) path = (multi || n >= ctx->sms) ? MI_PATH_BATCHED : MI_PATH_PLAIN;
     if (multi && path == MI_PATH_PLAIN) return ctx->fail(MI_EINVAL, "multi-pair contexts use the batched path");
     const bool plain = path == MI_PATH_PLAIN;
-    long long nvox_max = 0;
-    for (auto &p : ctx->pairs) nvox_max = std::max(nvox_max, p->nvf);
-    std::vector<Choice> cands = candidates(ctx, ctx->max_bins, nvox_max);
+    if (ctx->cands.empty()) {
+        long long nvox_max = 0;
+        for (auto &p : ctx->pairs) nvox_max = std::max(nvox_max, p->nvf);
+        ctx->cands = candidates(ctx, ctx->max_bins, nvox_max);
+    }
+    const std::vector<Choice> &cands = ctx->cands;
     if (cands.empty()) return ctx->fail(MI_EUNSUPPORTED, "no histogram variant fits this bin count and volume size");
+    // d_work: results h, mi and counts (in one piece, what every call reads last), then what is cleared
+    const size_t mi_at = align256((size_t)n * nq * 3 * 8), cnt_at = mi_at + (size_t)n * nq * 8,
+                 flags_at = cnt_at + (size_t)n * 8, ticket_at = align256(flags_at + 2 * sizeof(int)),
+                 done_at = ticket_at + 256;
+    Outputs O;
+    auto set_outputs = [&]() {
+        char *work = ctx->d_work.as<char>();
+        O.h = (double *)work;
+        O.mi = (double *)(work + mi_at);
+        O.count = (long long *)(work + cnt_at);
+        O.flags = (int *)(work + flags_at);
+        O.dump = R.dump;
+    };
     const int bucket = plain ? plain_bucket(n) : n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0);
     auto key = std::make_tuple(path, plain ? 0 : -1, bucket);
     Choice ch;
@@ -1377,16 +1422,17 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
             plan_items(ctx, R.pair_of, 0, n, cands.front(), kPlanWhole, whole);
             const size_t aff_bytes = align256((size_t)n * 48), item_bytes = (size_t)n * sizeof(Item);
             MI_CU(ctx->d_in.ensure(aff_bytes + item_bytes), "allocating the call's inputs");
-            MI_CU(ctx->d_work.ensure(256), "allocating the ticket");
+            MI_CU(ctx->d_work.ensure(done_at), "allocating the workspace");
+            set_outputs();
             MI_CU(cudaMemcpyAsync(ctx->d_in.p, R.d_q16 ? R.d_q16 : R.q16.data(), (size_t)n * 48, cudaMemcpyDefault,
                                   ctx->stream),
                   "affines");
             const Item *d_items = (const Item *)(ctx->d_in.as<char>() + aff_bytes);
             MI_CU(cudaMemcpyAsync((void *)d_items, whole.items.data(), item_bytes, cudaMemcpyHostToDevice, ctx->stream),
                   "H2D");
-            st = autotune(ctx, ctx->d_in.as<int32_t>(), d_items, n, Q, O, ch, cands);
+            st = autotune(ctx, ctx->d_in.as<int32_t>(), d_items, n, (int *)(ctx->d_work.as<char>() + ticket_at), Q, O, ch,
+                          cands);
             if (st != MI_OK) return st;
-            MI_CU(cudaMemsetAsync(ctx->d_flags.p, 0, 2 * sizeof(int), ctx->stream), "resetting flags");
             if (!cpath.empty()) cache_store(cpath, ckey, ch);
         }
         ctx->tuned[key] = ch;
@@ -1417,20 +1463,22 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     const size_t aff_bytes = align256((size_t)n * 48), items_at = aff_bytes,
                  slots_at = items_at + align256(plan.items.size() * sizeof(Item)),
                  in_bytes = slots_at + plan.slots.size() * sizeof(Slot);
-    const size_t done_at = 256, hist_at = done_at + align256(max_slots * 4);
+    const size_t hist_at = done_at + align256(max_slots * 4);
     const bool own_hist = !(plain && R.dump);
     const size_t work_bytes = hist_at + (own_hist ? max_slots * B2 * 4 : 0);
     MI_CU(ctx->d_in.ensure(in_bytes), "allocating the call's inputs");
     MI_CU(ctx->d_work.ensure(work_bytes), "allocating the workspace");
     if (max_slots)
         MI_CU(ctx->d_part.ensure(entropy_part_bytes((ctx->max_bins + 7) / 8, (int)max_slots)), "allocating partial sums");
+    set_outputs();
     cudaStream_t s = ctx->stream;
     // A batched call is replayed as a CUDA graph, so its inputs go through pinned staging.  The plain path
     // takes a few launches a call: capturing and instantiating would cost a first call more than it saves.
     const bool use_graph = !plain && ctx->opt.use_graphs && !R.dump && s != nullptr;
     char *staged;
+    const size_t out_at = align256(in_bytes);  // the results' staging follows the inputs'
     if (use_graph) {
-        MI_CU(ctx->h_in.ensure(in_bytes), "pinned staging");
+        MI_CU(ctx->h_in.ensure(out_at + ticket_at), "pinned staging");
         staged = ctx->h_in.as<char>();
     } else {
         ctx->v_in.resize(in_bytes);
@@ -1448,10 +1496,12 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
         MI_CU(record_event(ctx->ev0, s), "event");
         for (const Range &r : ranges) {
             uint32_t *hist = own_hist ? (uint32_t *)(work + hist_at) : R.dump + (size_t)r.t0 * B2;
-            MI_CU(cudaMemsetAsync(work, 0, hist_at + (own_hist ? r.nslots * B2 * 4 : 0), s), "clearing the workspace");
+            const size_t clear_at = r.t0 == 0 ? flags_at : ticket_at;  // the flags gather over all ranges
+            MI_CU(cudaMemsetAsync(work + clear_at, 0, hist_at - clear_at + (own_hist ? r.nslots * B2 * 4 : 0), s),
+                  "clearing the workspace");
             if (!own_hist) MI_CU(cudaMemsetAsync(hist, 0, r.nslots * B2 * 4, s), "clearing histograms");
             MI_CU(launch_batched(ctx->d_pairs.as<PairDev>(), (const int32_t *)in, (const Item *)(in + items_at) + r.item0,
-                                 (int)r.nitems, (int *)work, ctx->max_bins, ctx->max_rows_words, ctx->max_zplanes,
+                                 (int)r.nitems, (int *)(work + ticket_at), ctx->max_bins, ctx->max_rows_words, ctx->max_zplanes,
                                  ch.variant, ch.threads, ch.ctas, ch.tile, Q, O, hist, (long long)B2, s),
                   "histogram kernel");
             if (r.nslots)
@@ -1467,10 +1517,9 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
         if ((st = enqueue()) != MI_OK) return st;
     } else {
         char kb[640];
-        int off = snprintf(kb, sizeof kb, "%d:%d:%d:%d:%d:%d:%d:%zu:%zu:%d:%p:%p:%p:%p:%p:%p:%p:%d:%d", n, nq, ch.variant,
+        int off = snprintf(kb, sizeof kb, "%d:%d:%d:%d:%d:%d:%d:%zu:%zu:%d:%p:%p:%p:%p:%d:%d", n, nq, ch.variant,
                            ch.threads, ch.ctas, ch.tile.lpr_log2, ch.tile.slabs, plan.items.size(), plan.slots.size(),
-                           R.d_q16 ? 1 : 0, ctx->d_in.p, ctx->d_work.p, ctx->d_part.p, ctx->d_mi.p, ctx->d_h.p,
-                           ctx->d_cnt.p, ctx->h_in.p, Q.form, Q.bits);
+                           R.d_q16 ? 1 : 0, ctx->d_in.p, ctx->d_work.p, ctx->d_part.p, ctx->h_in.p, Q.form, Q.bits);
         for (int i = 0; i < nq && off < (int)sizeof kb - 40; ++i)
             off += snprintf(kb + off, sizeof kb - off, ":%08x:%p", fbits(Q.q[i]), (const void *)Q.tab[i]);
         auto it = ctx->graphs.find(kb);
@@ -1498,12 +1547,12 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     ctx->timed = true;
     ctx->last_launches = 0;
     for (const Range &r : ranges) ctx->last_launches += r.nslots ? 2 : 1;
-    if ((st = deliver(ctx, out_mi, ctx->d_mi.p, (size_t)n * nq * 8)) != MI_OK) return st;
-    if ((st = deliver(ctx, out_h, ctx->d_h.p, (size_t)n * nq * 3 * 8)) != MI_OK) return st;
-    if ((st = deliver(ctx, out_count, ctx->d_cnt.p, (size_t)n * 8)) != MI_OK) return st;
     int flags[2] = {0, 0};
-    MI_CU(cudaMemcpyAsync(flags, ctx->d_flags.p, sizeof flags, cudaMemcpyDeviceToHost, ctx->stream), "reading flags");
-    MI_CU(cudaStreamSynchronize(ctx->stream), "evaluation");
+    const Result res[] = {{out_h, 0, (size_t)n * nq * 3 * 8},
+                          {out_mi, mi_at, (size_t)n * nq * 8},
+                          {out_count, cnt_at, (size_t)n * 8},
+                          {flags, flags_at, sizeof flags}};
+    if ((st = deliver_all(ctx, ctx->d_work.as<char>(), res, 4, use_graph ? staged + out_at : nullptr)) != MI_OK) return st;
     if (flags[1]) return ctx->fail(MI_ECUDA, "internal: 16-bit counter drain failed (flags " + std::to_string(flags[1]) + ")");
     if (flags[0]) return ctx->fail(MI_EEMPTY, "at least one transform has an empty overlap (its MI is NaN)");
     return MI_OK;
@@ -1524,9 +1573,13 @@ mi_status parzen_core(mi_ctx *ctx, const std::vector<float> &prm, int n, const f
     if (st != MI_OK) return st;
     const int np = ctx->nparams();
     const bool multi = pair_of != nullptr;
-    std::vector<ParzenAffine> pa(n);
-    std::vector<double> jac((size_t)n * 12 * np);
-    std::vector<long long> row_start(multi ? n + 1 : 0);
+    const size_t jac_at = align256((size_t)n * sizeof(ParzenAffine)), rows_at = jac_at + align256((size_t)n * 12 * np * 8),
+                 pair_at = rows_at + (multi ? align256((size_t)(n + 1) * sizeof(long long)) : 0),
+                 in_bytes = multi ? pair_at + (size_t)n * sizeof(int) : jac_at + (size_t)n * 12 * np * 8;
+    ctx->v_in.resize(std::max(in_bytes, pair_at));
+    ParzenAffine *pa = (ParzenAffine *)ctx->v_in.data();
+    double *jac = (double *)(ctx->v_in.data() + jac_at);
+    long long *row_start = (long long *)(ctx->v_in.data() + rows_at);
     long long total_rows = 0;
     for (int t = 0; t < n; ++t) {
         const int pi = multi ? (*pair_of)[t] : 0;
@@ -1574,52 +1627,49 @@ mi_status parzen_core(mi_ctx *ctx, const std::vector<float> &prm, int n, const f
     const int actas = out_grad ? parzen_adj_ctas(rep, n, nq, ctx->sms) : 1;
     const int cblocks = parzen_cell_blocks(Bmax);
     if (multi) {
-        MI_CU(ctx->p_pair_of.ensure((size_t)n * sizeof(int)), "alloc");
-        MI_CU(ctx->p_row_start.ensure((size_t)(n + 1) * sizeof(long long)), "alloc");
-        MI_CU(cudaMemcpyAsync(ctx->p_pair_of.p, pair_of->data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, s),
-              "H2D");
-        MI_CU(cudaMemcpyAsync(ctx->p_row_start.p, row_start.data(), (size_t)(n + 1) * sizeof(long long),
-                              cudaMemcpyHostToDevice, s),
-              "H2D");
-        L.d_pair_of = ctx->p_pair_of.as<int>();
-        L.d_row_start = ctx->p_row_start.as<long long>();
+        memcpy(ctx->v_in.data() + pair_at, pair_of->data(), (size_t)n * sizeof(int));
     }
-    MI_CU(ctx->p_aff.ensure((size_t)n * sizeof(ParzenAffine)), "alloc");
-    MI_CU(ctx->p_jac.ensure((size_t)n * 12 * np * 8), "alloc");
+    MI_CU(ctx->p_in.ensure(in_bytes), "alloc");
+    if (multi) {
+        L.d_pair_of = (const int *)(ctx->p_in.as<char>() + pair_at);
+        L.d_row_start = (const long long *)(ctx->p_in.as<char>() + rows_at);
+    }
+    // results: overlap counts, MI, gradients
+    const size_t mi_at = (size_t)n * 8, grad_at = mi_at + (size_t)n * nq * 8;
+    MI_CU(ctx->p_out.ensure(grad_at + (size_t)n * nq * np * 8), "alloc");
     MI_CU(ctx->p_hist.ensure((size_t)n * BM2 * 8), "alloc");
-    MI_CU(ctx->p_cnt.ensure((size_t)n * 8), "alloc");
     MI_CU(ctx->p_marg.ensure((size_t)n * 2 * Bmax * 8), "alloc");
     MI_CU(ctx->p_ment.ensure((size_t)n * nq * 2 * 8), "alloc");
     MI_CU(ctx->p_mterm.ensure((size_t)n * nq * 2 * Bmax * 8), "alloc");
     MI_CU(ctx->p_jsum.ensure((size_t)n * nq * cblocks * 8), "alloc");
     MI_CU(ctx->p_w.ensure((size_t)n * nq * BM2 * 4), "alloc");
     MI_CU(ctx->p_mom.ensure((size_t)n * nq * actas * 12 * 8), "alloc");
-    MI_CU(ctx->p_grad.ensure((size_t)n * nq * np * 8), "alloc");
-    MI_CU(ctx->d_mi.ensure((size_t)n * nq * 8), "alloc");
-    MI_CU(cudaMemcpyAsync(ctx->p_aff.p, pa.data(), (size_t)n * sizeof(ParzenAffine), cudaMemcpyHostToDevice, s), "H2D");
-    MI_CU(cudaMemcpyAsync(ctx->p_jac.p, jac.data(), (size_t)n * 12 * np * 8, cudaMemcpyHostToDevice, s), "H2D");
-    const ParzenAffine *d_aff = ctx->p_aff.as<ParzenAffine>();
-    auto *cnt = ctx->p_cnt.as<unsigned long long>();
+    MI_CU(cudaMemcpyAsync(ctx->p_in.p, ctx->v_in.data(), in_bytes, cudaMemcpyHostToDevice, s), "H2D");
+    const ParzenAffine *d_aff = ctx->p_in.as<ParzenAffine>();
+    const double *d_jac = (const double *)(ctx->p_in.as<char>() + jac_at);
+    char *out = ctx->p_out.as<char>();
+    auto *cnt = (unsigned long long *)out;
+    double *d_mi = (double *)(out + mi_at), *d_grad = (double *)(out + grad_at);
     auto *hist = ctx->p_hist.as<unsigned long long>();
     MI_CU(cudaEventRecord(ctx->ev0, s), "event");
     MI_CU(launch_parzen_hist(L, d_aff, ctx->sms, hist, cnt, s), "Parzen histogram");
     MI_CU(launch_parzen_weights(hist, cnt, L, Q, ctx->p_marg.as<double>(), ctx->p_ment.as<double>(),
-                                ctx->p_mterm.as<double>(), ctx->p_jsum.as<double>(), ctx->d_mi.as<double>(),
+                                ctx->p_mterm.as<double>(), ctx->p_jsum.as<double>(), d_mi,
                                 ctx->p_w.as<float>(), s),
           "Parzen entropies");
     if (out_grad)
-        MI_CU(launch_parzen_adjoint(L, d_aff, ctx->p_jac.as<double>(), np, nq, actas, ctx->p_w.as<float>(), cnt,
-                                    ctx->p_mom.as<double>(), ctx->p_grad.as<double>(), s),
+        MI_CU(launch_parzen_adjoint(L, d_aff, d_jac, np, nq, actas, ctx->p_w.as<float>(), cnt,
+                                    ctx->p_mom.as<double>(), d_grad, s),
               "Parzen adjoint");
     MI_CU(cudaEventRecord(ctx->ev1, s), "event");
     ctx->timed = true;
     ctx->last_launches = 4 + (out_grad ? (nq + 3) / 4 + 1 : 0);
-    if ((st = deliver(ctx, out_mi, ctx->d_mi.p, (size_t)n * nq * 8)) != MI_OK) return st;
-    if (out_grad && (st = deliver(ctx, out_grad, ctx->p_grad.p, (size_t)n * nq * np * 8)) != MI_OK) return st;
-    if (out_count && (st = deliver(ctx, out_count, cnt, (size_t)n * 8)) != MI_OK) return st;
     std::vector<unsigned long long> hc(n);
-    MI_CU(cudaMemcpyAsync(hc.data(), cnt, (size_t)n * 8, cudaMemcpyDeviceToHost, s), "reading counts");
-    MI_CU(cudaStreamSynchronize(s), "Parzen evaluation");
+    const Result res[] = {{hc.data(), 0, (size_t)n * 8},
+                          {out_count, 0, (size_t)n * 8},
+                          {out_mi, mi_at, (size_t)n * nq * 8},
+                          {out_grad, grad_at, (size_t)n * nq * np * 8}};
+    if ((st = deliver_all(ctx, out, res, 4, nullptr)) != MI_OK) return st;
     for (int t = 0; t < n; ++t)
         if (hc[t] == 0) return ctx->fail(MI_EEMPTY, "at least one transform has an empty overlap (its MI is NaN)");
     return MI_OK;

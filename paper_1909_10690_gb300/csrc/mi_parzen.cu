@@ -638,22 +638,216 @@ __global__ void k_parzen_final(int n, const unsigned long long *__restrict__ gco
 // Adjoint: moments M[q][a][c] = sum_x s_q(x) d_a m(u_x) x_c, x = (i - ci, j - cj, k - ck, 1)
 // ---------------------------------------------------------------------------
 
+// Two FP32 values in one 64-bit register pair: one instruction does both (the same roundings).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float low2(f32x2 v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float high2(f32x2 v) { return __uint_as_float((unsigned)(v >> 32)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// trilinear_x<true> with the two z planes of every stage in one register pair.
+__device__ __forceinline__ MG trilinear_x2(const float *__restrict__ movx, int m0, int m01, long long Ux, long long Uy,
+                                           long long Uz) {
+    constexpr float k2m32 = 2.3283064365386963e-10f;  // 2^-32
+    const int cx = (int)(Ux >> 32), cy = (int)(Uy >> 32), cz = (int)(Uz >> 32);
+    const float wx = __uint2float_rn((unsigned)Ux) * k2m32, wy = __uint2float_rn((unsigned)Uy) * k2m32,
+                wz = __uint2float_rn((unsigned)Uz) * k2m32;
+    const float *p = movx + (cx + m0 * cy + m01 * cz), *pz = p + m01;
+    const f32x2 v00 = pack2(__ldg(p), __ldg(pz)), v01 = pack2(__ldg(p + 1), __ldg(pz + 1));
+    const f32x2 v10 = pack2(__ldg(p + m0), __ldg(pz + m0)), v11 = pack2(__ldg(p + m0 + 1), __ldg(pz + m0 + 1));
+    const f32x2 wx2 = pack2(wx, wx), wy2 = pack2(wy, wy);
+    const f32x2 d0 = sub2(v01, v00), d1 = sub2(v11, v10);
+    const f32x2 a0 = fma2(wx2, d0, v00), a1 = fma2(wx2, d1, v10);
+    const f32x2 y = sub2(a1, a0), b = fma2(wy2, y, a0), e = fma2(wy2, sub2(d1, d0), d0);
+    MG r;
+    r.gz = high2(b) - low2(b);
+    r.m = fmaf(wz, r.gz, low2(b));
+    r.gy = fmaf(wz, high2(y) - low2(y), low2(y));
+    r.gx = fmaf(wz, high2(e) - low2(e), low2(e));
+    return r;
+}
+
 // Where an adjoint launch keeps the W table of its q values: in the shared memory of one 512-thread
-// CTA an SM when it fits, else in global memory read by 256-thread CTAs (two an SM).  Either gives 16
-// warps an SM at 128 registers a thread; the larger CTA measured 4 % faster at 64 bins (fewer, larger
-// row shares), and one float a cell 1.5 % faster than (W[k], W[k + 1]) pairs read as two 8-byte words.
+// CTA an SM when it fits (two q of a cell side by side, one load for both; the last of an odd number
+// apart), else in global memory read by 256-thread CTAs (two an SM).  Either gives 16 warps an SM at 128
+// registers a thread; the larger CTA measured 4 % faster at 64 bins (fewer, larger row shares).
 enum { kWGlobal = 0, kWShared = 1 };
 
+// s(x) = sum_k W(fb, k) beta3'(k - m~) of every q at a voxel whose taps are cells cb .. cb + 3 (the last
+// one clamped to cb, with weight 0, past the table's end).
+template <int NQ, int MODE>
+__device__ __forceinline__ void adj_slopes(const float *__restrict__ tab, int cells, int cb, int i3, const float (&d)[4],
+                                           float (&sv)[NQ]) {
+    auto dot = [&](const float *__restrict__ w) {
+        return fmaf(w[i3], d[3], fmaf(w[cb + 2], d[2], fmaf(w[cb], d[0], w[cb + 1] * d[1])));
+    };
+    if constexpr (MODE == kWShared) {
+        if constexpr (NQ >= 2) {
+            const f32x2 d0 = pack2(d[0], d[0]), d1 = pack2(d[1], d[1]), d2 = pack2(d[2], d[2]), d3 = pack2(d[3], d[3]);
+#pragma unroll
+            for (int p = 0; p < NQ / 2; ++p) {
+                const f32x2 *w = (const f32x2 *)tab + (size_t)p * cells;
+                const f32x2 v = fma2(w[i3], d3, fma2(w[cb + 2], d2, fma2(w[cb], d0, mul2(w[cb + 1], d1))));
+                sv[2 * p] = low2(v);
+                sv[2 * p + 1] = high2(v);
+            }
+        }
+        if constexpr (NQ % 2) sv[NQ - 1] = dot(tab + (size_t)(NQ - 1) * cells);
+    } else {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) sv[q] = dot(tab + (size_t)q * cells);
+    }
+}
+
+// The moments of a thread: per q and axis a, ms = (sum s d_a m (i - ci), sum s d_a m over the current row)
+// and the row's folded share of the moments in j - cj, k - ck and 1 (along a row j and k are constant).
+template <int NQ>
+struct AdjMoments {
+    f32x2 ms[NQ][3];
+    float mj[NQ][3], mk[NQ][3], m1[NQ][3];
+    __device__ void zero() {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                ms[q][a] = 0;
+                mj[q][a] = mk[q][a] = m1[q][a] = 0.0f;
+            }
+    }
+    __device__ __forceinline__ void end_row(float j, float k) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const float s0 = high2(ms[q][a]);
+                mj[q][a] = fmaf(s0, j, mj[q][a]);
+                mk[q][a] = fmaf(s0, k, mk[q][a]);
+                m1[q][a] += s0;
+                ms[q][a] = pack2(low2(ms[q][a]), 0.0f);
+            }
+    }
+    __device__ __forceinline__ float get(int q, int e) const {  // e = 4 a + c, c of (i, j, k, 1)
+        const int a = e >> 2, c = e & 3;
+        return c == 0 ? low2(ms[q][a]) : c == 1 ? mj[q][a] : c == 2 ? mk[q][a] : m1[q][a];
+    }
+};
+
+// The rows of one CTA's share: warp w of CTA b takes rows (b nwarps + w) + gridDim.x nwarps n, 32 of them
+// clipped at once (lane l: the l-th, with its j and k) and walked one by one, 32 voxels (or, under random
+// sampling, 32 sampled entries) a step.  tab: W with row stride rs and `cells` entries a q.
+template <int NQ, bool SAMPLED, int MODE>
+__device__ __forceinline__ void adj_rows(const ParzenPair &P, const long long *A, const float *__restrict__ tab, int rs,
+                                         int cells, AdjMoments<NQ> &M) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int nf0 = P.nf[0], nf1 = P.nf[1], B = P.B;
+    const int R = nf1 * P.nf[2];  // fewer than 2^31
+    const int n0 = P.nm[0], n1 = P.nm[1], n2 = P.nm[2];
+    const int m0 = n0 + 1, m01 = m0 * (n1 + 1);
+    const float Bm4 = (float)(B - 4);
+    // moments are taken about the fixed-volume centre, where the rotation and
+    // scale columns of du/dtheta have no constant part (no cancellation)
+    const float ci = 0.5f * (float)(nf0 - 1), cj = 0.5f * (float)(nf1 - 1), ck = 0.5f * (float)(P.nf[2] - 1);
+    // one voxel (x index i, fixed bin bf) at 32.32 index V
+    auto acc_voxel = [&](long long V0, long long V1, long long V2, int i, int bf) {
+        const MG g = trilinear_x2(P.movx, m0, m01, V0, V1, V2);
+        const float ic = (float)i - ci;
+        const float mt = fmaf(fminf(fmaxf(g.m, 0.0f), 1.0f), Bm4, 2.0f);
+        const int k0 = (int)mt;
+        float d[4], sv[NQ];
+        bspline_dw(mt - (float)k0, d);
+        if (k0 + 2 >= B) d[3] = 0.0f;
+        const int cb = bf * rs + (k0 - 1);
+        adj_slopes<NQ, MODE>(tab, cells, cb, k0 + 2 < B ? cb + 3 : cb, d, sv);
+        const f32x2 gx = pack2(g.gx * ic, g.gx), gy = pack2(g.gy * ic, g.gy), gz = pack2(g.gz * ic, g.gz);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const f32x2 s2 = pack2(sv[q], sv[q]);
+            M.ms[q][0] = fma2(s2, gx, M.ms[q][0]);
+            M.ms[q][1] = fma2(s2, gy, M.ms[q][1]);
+            M.ms[q][2] = fma2(s2, gz, M.ms[q][2]);
+        }
+    };
+    const long long D0 = 32 * A[0], D1 = 32 * A[4], D2 = 32 * A[8];
+    const long long step = (long long)gridDim.x * nwarps;
+    for (long long g = (long long)blockIdx.x * nwarps + warp; g < R; g += 32 * step) {
+        Clip64 mine;
+        mine.lo = 1;
+        mine.hi = 0;
+        mine.u0 = mine.u1 = mine.u2 = 0;
+        int jl = 0, kl = 0;
+        const long long rl = g + step * lane;
+        if (rl < R) {
+            kl = (int)rl / nf1;
+            jl = (int)rl - kl * nf1;
+            mine = clip_row64(A, jl, kl, nf0, n0, n1, n2);
+        }
+        for (int s = 0; s < 32; ++s) {
+            const long long r = g + step * s;
+            if (r >= R) break;  // warp-uniform
+            const int lo = __shfl_sync(kFull, mine.lo, s), hi = __shfl_sync(kFull, mine.hi, s);
+            if (lo > hi) continue;
+            const long long u0 = __shfl_sync(kFull, mine.u0, s), u1 = __shfl_sync(kFull, mine.u1, s),
+                            u2 = __shfl_sync(kFull, mine.u2, s);
+            const float j = (float)__shfl_sync(kFull, jl, s) - cj, k = (float)__shfl_sync(kFull, kl, s) - ck;
+            if constexpr (SAMPLED) {
+                const uint32_t e0 = __ldg(P.srow + r), e1 = __ldg(P.srow + r + 1);
+                for (uint32_t eb = e0; eb < e1; eb += 32) {
+                    const uint32_t e = eb + lane;
+                    const int i = e < e1 ? (int)__ldg(P.scol + e) : -1;
+                    if (e < e1 && i >= lo && i <= hi) {
+                        const long long dd = i - lo;
+                        acc_voxel(u0 + A[0] * dd, u1 + A[4] * dd, u2 + A[8] * dd, i, (int)__ldg(P.sbin + e));
+                    }
+                }
+            } else {
+                long long U0 = u0 + A[0] * lane, U1 = u1 + A[4] * lane, U2 = u2 + A[8] * lane;
+                const uint8_t *__restrict__ frow = P.fbins + (size_t)r * nf0;
+                int i = lo + lane;
+                for (; i - lane <= hi; i += 32) {
+                    if (i <= hi) acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
+                    U0 += D0;
+                    U1 += D1;
+                    U2 += D2;
+                }
+            }
+            M.end_row(j, k);
+        }
+    }
+}
+
+// What bounds it: instruction issue and latency at 16 warps an SM (45 moment accumulators for three q hold
+// 128 registers), so instructions are saved where the FP32 results stay the same to the bit (the sums run
+// over thousands of voxels, and another order moves the gradient by 1e-7): two values an instruction in the
+// trilinear stages, the moments and the slopes of paired q, and a row's j and k by shuffle from the lane
+// that clipped it instead of two 64-bit divisions a row.  50 poses, 192 x 192 x 128, 64 bins, three q: 1628
+// -> 1458 us; six pairs of up to 128 bins, 48 poses: 3266 -> 2921.  (With other sums allowed: quadratic
+// coefficients of s per cell instead of W, 160 KB of shared memory, 1533 and, with two rows a step, 2516.)
 template <int NQ, bool SAMPLED, bool MULTI, int TPB>
 __global__ void __launch_bounds__(TPB, 512 / TPB)
     k_parzen_adj(ParzenPair P0, const ParzenPair *__restrict__ pairs, const int *__restrict__ pair_of, int Bmax,
                  const ParzenAffine *__restrict__ aff, int nq_total, int q0, const float *__restrict__ wtab,
-                 int w_mode, double *__restrict__ mom) {
+                 double *__restrict__ mom) {
     // mom: n x nq_total x gridDim.x x 12 per-CTA partial moments (no atomics: fixed-order reduction later)
-    // NQ x B x SB weights in shared memory (w_mode kWShared); the row stride SB >= B + 1 is 7 mod 32, so
-    // neighbouring voxels' cells, a bin or two apart on either axis, are read from different banks.
     // W of transform t is its slot of Bmax^2 entries per q (the first B^2 used, row stride B).
-    extern __shared__ float sw[];
+    extern __shared__ __align__(16) float sw[];
     const int t = blockIdx.y;
     const ParzenPair P = MULTI ? pairs[pair_of[t]] : P0;
     const int B = P.B, SB = parzen_stride(B);
@@ -662,123 +856,30 @@ __global__ void __launch_bounds__(TPB, 512 / TPB)
     if (threadIdx.x < 12) A[threadIdx.x] = aff[t].A[threadIdx.x];
     const size_t BM2 = (size_t)Bmax * Bmax;
     const float *W = wtab + ((size_t)t * nq_total + q0) * BM2;
-    int RS = B, QS = (int)BM2;  // row stride and per-q stride of the table in use
-    if (w_mode == kWShared) {
+    AdjMoments<NQ> M;
+    M.zero();
+    if constexpr (TPB == 256) {
+        __syncthreads();
+        adj_rows<NQ, SAMPLED, kWGlobal>(P, A, W, B, (int)BM2, M);
+    } else {
+        // NQ x B x SB weights; the row stride SB >= B + 1 is 7 mod 32, so neighbouring voxels' cells, a bin
+        // or two apart on either axis, are read from different banks
+        const int cells = B * SB;
         for (int c = threadIdx.x; c < NQ * B * B; c += blockDim.x) {
-            const int qq = c / (B * B), cc = c % (B * B);
-            sw[qq * B * SB + (cc / B) * SB + cc % B] = W[(size_t)qq * BM2 + cc];
+            const int q = c / (B * B), cc = c % (B * B), at = (cc / B) * SB + cc % B;
+            const bool apart = NQ % 2 && q == NQ - 1;
+            sw[apart ? q * cells + at : 2 * ((q / 2) * cells + at) + q % 2] = W[(size_t)q * BM2 + cc];
         }
-        RS = SB;
-        QS = B * SB;
+        __syncthreads();
+        adj_rows<NQ, SAMPLED, kWShared>(P, A, sw, SB, cells, M);
     }
-    __syncthreads();
+    // warp reduction in FP32, then the warps in FP64 into global memory
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int nf0 = P.nf[0], nf1 = P.nf[1];
-    const int n0 = P.nm[0], n1 = P.nm[1], n2 = P.nm[2];
-    const long long R = (long long)nf1 * P.nf[2];
-    const float Bm4 = (float)(B - 4);
-    const long long D0 = 32 * A[0], D1 = 32 * A[4], D2 = 32 * A[8];
-    // moments are taken about the fixed-volume centre, where the rotation and
-    // scale columns of du/dtheta have no constant part (no cancellation)
-    const float ci = 0.5f * (float)(nf0 - 1), cj = 0.5f * (float)(nf1 - 1), ck = 0.5f * (float)(P.nf[2] - 1);
-    float M[NQ][12];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-#pragma unroll
-        for (int e = 0; e < 12; ++e) M[q][e] = 0.0f;
-    // warp w of CTA b takes rows (b nwarps + w) + gridDim.x nwarps n; a group of 32 is clipped at once
-    const long long rstep = (long long)gridDim.x * nwarps;
-    for (long long g = (long long)blockIdx.x * nwarps + warp; g < R; g += 32 * rstep) {
-        Clip64 mine;
-        mine.lo = 1;
-        mine.hi = 0;
-        mine.u0 = mine.u1 = mine.u2 = 0;
-        const long long rl = g + rstep * lane;
-        if (rl < R) mine = clip_row64(A, rl % nf1, rl / nf1, nf0, n0, n1, n2);
-        for (int s = 0; s < 32; ++s) {
-            const long long r = g + rstep * s;
-            if (r >= R) break;  // warp-uniform
-            const int lo = __shfl_sync(kFull, mine.lo, s), hi = __shfl_sync(kFull, mine.hi, s);
-            if (lo > hi) continue;
-            long long U0 = __shfl_sync(kFull, mine.u0, s) + A[0] * lane;
-            long long U1 = __shfl_sync(kFull, mine.u1, s) + A[4] * lane;
-            long long U2 = __shfl_sync(kFull, mine.u2, s) + A[8] * lane;
-            const float j = (float)(r % nf1) - cj, k = (float)(r / nf1) - ck;
-            const uint8_t *__restrict__ frow = P.fbins + (size_t)r * nf0;
-            // along the row j and k are constant: per row, S0[q][a] = sum s d_a m, and the moments in
-            // j, k and 1 follow from it at the row's end; sum s d_a m (i - ci) goes to M directly
-            float S0[NQ][3];
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) S0[q][a] = 0.0f;
-            // one voxel (x index i, fixed bin bf) at 32.32 index U: its share of S0 and M
-            auto acc_voxel = [&](long long V0, long long V1, long long V2, int i, int bf) {
-                const MG g3 = trilinear_x<true>(P.movx, P.nm[0] + 1, (P.nm[0] + 1) * (P.nm[1] + 1), V0, V1, V2);
-                const float ic = (float)i - ci;
-                // d_a m and d_a m (i - ci), shared by every q
-                const float hx = g3.gx * ic, hy = g3.gy * ic, hz = g3.gz * ic;
-                const float mt = fmaf(fminf(fmaxf(g3.m, 0.0f), 1.0f), Bm4, 2.0f);
-                const int k0 = (int)mt;
-                float d[4];
-                bspline_dw(mt - (float)k0, d);
-                if (k0 + 2 >= B) d[3] = 0.0f;
-                const int cb = bf * RS + (k0 - 1);
-                const int i3 = k0 + 2 < B ? cb + 3 : cb;  // in range; weight 0 when clamped
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    float sv;
-                    if (w_mode == kWShared) {
-                        const float *Wq = sw + (size_t)q * QS;
-                        sv = Wq[cb] * d[0] + Wq[cb + 1] * d[1] + Wq[cb + 2] * d[2] + Wq[i3] * d[3];
-                    } else {
-                        const float *Wq = W + (size_t)q * QS;
-                        sv = Wq[cb] * d[0] + Wq[cb + 1] * d[1] + Wq[cb + 2] * d[2] + Wq[i3] * d[3];
-                    }
-                    M[q][0] = fmaf(sv, hx, M[q][0]);
-                    S0[q][0] = fmaf(sv, g3.gx, S0[q][0]);
-                    M[q][4] = fmaf(sv, hy, M[q][4]);
-                    S0[q][1] = fmaf(sv, g3.gy, S0[q][1]);
-                    M[q][8] = fmaf(sv, hz, M[q][8]);
-                    S0[q][2] = fmaf(sv, g3.gz, S0[q][2]);
-                }
-            };
-            if constexpr (SAMPLED) {  // random sampling: the row's sampled voxels inside [lo, hi]
-                const long long ub0 = U0 - A[0] * lane, ub1 = U1 - A[4] * lane, ub2 = U2 - A[8] * lane;
-                const uint32_t e0 = __ldg(P.srow + r), e1 = __ldg(P.srow + r + 1);
-                for (uint32_t eb = e0; eb < e1; eb += 32) {
-                    const uint32_t e = eb + lane;
-                    const int i = e < e1 ? (int)__ldg(P.scol + e) : -1;
-                    if (e < e1 && i >= lo && i <= hi) {
-                        const long long dd = i - lo;
-                        acc_voxel(ub0 + A[0] * dd, ub1 + A[4] * dd, ub2 + A[8] * dd, i, (int)__ldg(P.sbin + e));
-                    }
-                }
-            } else {
-                for (int base = lo; base <= hi; base += 32) {
-                    const int i = base + lane;
-                    if (i <= hi) acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
-                    U0 += D0;
-                    U1 += D1;
-                    U2 += D2;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    M[q][4 * a + 1] = fmaf(S0[q][a], j, M[q][4 * a + 1]);
-                    M[q][4 * a + 2] = fmaf(S0[q][a], k, M[q][4 * a + 2]);
-                    M[q][4 * a + 3] += S0[q][a];
-                }
-        }
-    }
-    // warp reduction in FP32, then the 8 warps in FP64 into global memory
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
 #pragma unroll
         for (int e = 0; e < 12; ++e) {
-            float v = M[q][e];
+            float v = M.get(q, e);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
             if (lane == 0) s_red[warp][q * 12 + e] = v;
@@ -986,12 +1087,12 @@ cudaError_t launch_parzen_adjoint(const ParzenLaunch &L, const ParzenAffine *d_a
     for (int q0 = 0; q0 < nq; q0 += 4) {
         const int g = nq - q0 < 4 ? nq - q0 : 4;
         const size_t smem = parzen_adj_smem(L.Bmax, g);
-        const int wmode = parzen_adj_wmode(L.Bmax, g), tpb = parzen_adj_threads(L.Bmax, g);
+        const int tpb = parzen_adj_threads(L.Bmax, g);
 #define MI_ADJ_T(NQV, SV, MV, TV)                                                                              \
     do {                                                                                                       \
         if ((e = allow_smem((const void *)k_parzen_adj<NQV, SV, MV, TV>, smem)) != cudaSuccess) return e;      \
         k_parzen_adj<NQV, SV, MV, TV><<<grid, TV, smem, s>>>(L.p0, L.d_pairs, L.d_pair_of, L.Bmax, d_aff, nq, q0, \
-                                                             d_w, wmode, d_mom);                               \
+                                                             d_w, d_mom);                               \
     } while (0)
 #define MI_ADJ_S(NQV, SV, MV)            \
     do {                                 \

@@ -103,3 +103,30 @@ def test_noalloc_rows_counters_and_terms(cuda_lib, shape, dtype, depth, bins):
                 continue
             got = cuda_lib.eval_noalloc(ad, bd, bins, prm[t], qs, fixed_depth=depth, moving_depth=depth)
             assert np.all(np.abs(got - mi_o[t]) <= 1e-6 * np.maximum(np.abs(mi_o[t]), h_o[t, :, 2]) + 1e-12)
+
+
+@pytest.mark.parametrize("bins,nq,sampled", [(8, 1, False), (64, 2, False), (128, 3, False), (96, 4, False),
+                                             (97, 4, False), (33, 7, False), (64, 3, True)])
+def test_adjoint_tables(cuda_lib, bins, nq, sampled):
+    """Paired and single q tables in shared and in global memory (four q from 97 bins on), an odd number of
+    fixed rows, saturated intensities (the last moving bin, whose last tap is outside the table), random
+    sampling, and a second pair with fewer bins in the same call."""
+    rng = np.random.default_rng(78)
+    f, m = phantoms.head_pair(shape=(27, 31, 37), spacing=(1, 1, 1), seed=77, dtype=np.float32)
+    f[rng.random(f.shape) < 0.05] = 1.0
+    m[10:14, 8:20, 5:30] = 1.0
+    qs = [1.0, 1.3, 2.0, 3.0, 4.0, 1.5, 2.5][:nq]
+    prm = phantoms.random_transforms(3, seed=79, t_mm=6, r_deg=15, s_range=(0.9, 1.1))
+    kw = dict(kernel="parzen", sample_fraction=0.3 if sampled else 0.0, sample_seed=4)
+    thr = oracle.sample_threshold(0.3)
+    keep = np.array([oracle.sampled(x, 4, thr) for x in range(f.size)]).reshape(f.shape) if sampled else None
+    _, g = cuda_lib.Context(f, m, bins=bins, **kw).grad(prm, qs)
+    _, gm = cuda_lib.Context(pairs=[dict(fixed=f, moving=m, bins=b) for b in (bins, 16)], **kw).batch_grad(
+        np.array([0, 1, 0], np.int32), prm, qs)
+    for t in range(3):
+        aff, J = oracle.affine(prm[t], f.shape, (1, 1, 1), m.shape, (1, 1, 1), with_jacobian=True)
+        mask = keep & oracle.overlap_mask(f.shape, m.shape, aff) if sampled else None
+        for got, b in ((g[t], bins), (gm[t], (bins, 16, bins)[t])):
+            _, want, _ = oracle.parzen(f, m, aff, b, qs, daff=J, mask=mask)
+            for iq in range(nq):
+                assert np.abs(got[iq] - want[iq]).max() <= 1e-4 * np.abs(want[iq]).max(), (t, b, iq)
