@@ -105,49 +105,14 @@ __global__ void k_pmov_f32(const float *__restrict__ in, long long n, float *__r
     }
 }
 
-// FP32 trilinear value and gradient (w.r.t. the moving index) at a 32.32
-// index u inside [0, n-1]^3, read from the extended volume (dims n + 1 per
-// axis): the cell is the integer part of u and the weight its fraction, also
-// on the last plane, where the extension makes the value v[n-1] and the
-// derivative v[n-1] - v[n-2] (those of the last cell of the volume).
+// FP32 trilinear value and gradient with respect to the moving index.
 struct MG {
     float m, gx, gy, gz;
 };
 
-// m0 = n0 + 1 and m01 = (n0 + 1)(n1 + 1): element offsets fit 32 bits (the extended volume holds fewer
-// than 2^31 elements, checked when the context is created).
-template <bool GRAD>
-__device__ __forceinline__ MG trilinear_x(const float *__restrict__ movx, int m0, int m01, long long Ux,
-                                          long long Uy, long long Uz) {
-    constexpr float k2m32 = 2.3283064365386963e-10f;  // 2^-32
-    const int cx = (int)(Ux >> 32), cy = (int)(Uy >> 32), cz = (int)(Uz >> 32);
-    const float wx = __uint2float_rn((unsigned)Ux) * k2m32, wy = __uint2float_rn((unsigned)Uy) * k2m32,
-                wz = __uint2float_rn((unsigned)Uz) * k2m32;
-    const float *p = movx + (cx + m0 * cy + m01 * cz);
-    const float v000 = __ldg(p), v001 = __ldg(p + 1), v010 = __ldg(p + m0), v011 = __ldg(p + m0 + 1);
-    const float v100 = __ldg(p + m01), v101 = __ldg(p + m01 + 1), v110 = __ldg(p + m01 + m0),
-                v111 = __ldg(p + m01 + m0 + 1);
-    const float d00 = v001 - v000, d01 = v011 - v010, d10 = v101 - v100, d11 = v111 - v110;
-    const float a00 = fmaf(wx, d00, v000), a01 = fmaf(wx, d01, v010);
-    const float a10 = fmaf(wx, d10, v100), a11 = fmaf(wx, d11, v110);
-    const float b0 = fmaf(wy, a01 - a00, a00), b1 = fmaf(wy, a11 - a10, a10);
-    MG r;
-    r.m = fmaf(wz, b1 - b0, b0);
-    if (GRAD) {
-        r.gz = b1 - b0;
-        const float y0 = a01 - a00, y1 = a11 - a10;
-        r.gy = fmaf(wz, y1 - y0, y0);
-        const float e0 = fmaf(wy, d01 - d00, d00), e1 = fmaf(wy, d11 - d10, d10);
-        r.gx = fmaf(wz, e1 - e0, e0);
-    } else {
-        r.gx = r.gy = r.gz = 0.0f;
-    }
-    return r;
-}
-
 // The trilinear value (no gradient) through the texture of 2 x 2 (y, z) quads of the extended volume:
 // two fetches at integer texel coordinates, columns cx and cx + 1, return the eight neighbours, so the
-// value equals trilinear_x's.  Column cx + 1 = n0 lies past the texture only where the position sits
+// value equals trilinear_x2's.  Column cx + 1 = n0 lies past the texture only where the position sits
 // on the last x plane, whose fraction wx is then 0: the clamped texel is read with weight 0 (the
 // derivative along x there needs the extension's column, so the gradient reads the volume itself).
 // Neighbouring lanes step along x, so one lane's second column is mostly the next lane's first.
@@ -178,16 +143,33 @@ struct Clip64 {
     long long u0, u1, u2;
 };
 
-__device__ __forceinline__ long long floor_div(long long a, long long b) {
-    long long q = a / b;
-    if (a % b != 0 && ((a < 0) != (b < 0))) --q;
+// floor(a / b) for b > 0 where it lies within +-kFarIndex, else beyond it on the same side: the FP32 quotient
+// is within a step or two of the exact one, which the remainder then fixes (a 64-bit division is some 70
+// instructions, and a lane clipping its row takes six: one pose's adjoint, whose warps walk two or three
+// rows each, 60 -> 54 us).
+constexpr int kFarIndex = 1 << 18;  // past every fixed row (at most 2^16 voxels)
+__device__ __forceinline__ int floor_div(long long a, long long b) {
+    const float f = floorf((float)a / (float)b);
+    if (f > (float)kFarIndex) return kFarIndex + 8;
+    if (f < -(float)kFarIndex) return -kFarIndex - 8;
+    int q = (int)f;
+    long long r = a - (long long)q * b;
+    while (r < 0) {
+        --q;
+        r += b;
+    }
+    while (r >= b) {
+        ++q;
+        r -= b;
+    }
     return q;
 }
 
-__device__ __forceinline__ long long ceil_div(long long a, long long b) { return -floor_div(-a, b); }
+__device__ __forceinline__ int ceil_div(long long a, long long b) { return -floor_div(-a, b); }
 
 __device__ Clip64 clip_row64(const long long *A, long long j, long long k, int nf0, int n0, int n1, int n2) {
-    long long lo = 0, hi = nf0 - 1, b[3];
+    long long b[3];
+    int lo = 0, hi = nf0 - 1;
     const int nm[3] = {n0, n1, n2};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -197,8 +179,8 @@ __device__ Clip64 clip_row64(const long long *A, long long j, long long k, int n
             lo = max(lo, ceil_div(-b[a], st));
             hi = min(hi, floor_div(umax - b[a], st));
         } else if (st < 0) {
-            lo = max(lo, ceil_div(umax - b[a], st));
-            hi = min(hi, floor_div(-b[a], st));
+            lo = max(lo, ceil_div(b[a] - umax, -st));
+            hi = min(hi, floor_div(b[a], -st));
         } else if (b[a] < 0 || b[a] > umax) {
             hi = -1;
         }
@@ -208,8 +190,8 @@ __device__ Clip64 clip_row64(const long long *A, long long j, long long k, int n
     c.hi = 0;
     c.u0 = c.u1 = c.u2 = 0;
     if (lo <= hi) {
-        c.lo = (int)lo;
-        c.hi = (int)hi;
+        c.lo = lo;
+        c.hi = hi;
         c.u0 = b[0] + A[0] * lo;
         c.u1 = b[1] + A[4] * lo;
         c.u2 = b[2] + A[8] * lo;
@@ -251,8 +233,6 @@ __device__ __forceinline__ void bspline_dw(float t, float d[4]) {
 // copies, goes to the global histogram.
 constexpr int kParzenMaxVox = 65536;  // also the longest fixed row (MI_MAX_PARZEN_NX)
 constexpr int kParzenBankSkew = 7;    // row stride of the forward's shared histogram, mod 32
-constexpr bool kParzenFwdTex = true;   // forward gathers through the quad texture (the adjoint loads
-                                       // the extended volume's eight neighbours, whose L1 serves it best)
 constexpr int kParzenRowsPerStep = 1;  // rows a warp of the forward works on at a time
 
 // Row stride of the shared tables: the least SB >= B + 1 with SB = kParzenBankSkew (mod 32).
@@ -344,9 +324,7 @@ __global__ void __launch_bounds__(kParzenFwdThreads)
         unsigned int cnt = 0;  // overlap voxels counted by this lane
         // one voxel at 32.32 index U with fixed bin bf: its four quantised B-spline weights
         auto add_voxel = [&](long long U0, long long U1, long long U2, int bf) {
-            const float mv = kParzenFwdTex ? trilinear_qv(P.texq, U0, U1, U2)
-                                           : trilinear_x<false>(P.movx, P.nm[0] + 1, (P.nm[0] + 1) * (P.nm[1] + 1),
-                                                                U0, U1, U2).m;
+            const float mv = trilinear_qv(P.texq, U0, U1, U2);
             const float mt = fmaf(fminf(fmaxf(mv, 0.0f), 1.0f), Bm4, 2.0f);
             const int k0 = (int)mt;
             float w[4];
@@ -373,7 +351,7 @@ __global__ void __launch_bounds__(kParzenFwdThreads)
             mine.hi = 0;
             mine.u0 = mine.u1 = mine.u2 = 0;
             const long long rl = g + (long long)nwarps * lane;
-            if (rl < r1) mine = clip_row64(A, rl % nf1, rl / nf1, nf0, n0, n1, n2);
+            if (rl < r1) mine = clip_row64(A, (int)rl % nf1, (int)rl / nf1, nf0, n0, n1, n2);  // rows of one pair: int
             if constexpr (SAMPLED) {  // random sampling: each row's sampled voxels inside its interval
                 for (int s = 0; s < 32; ++s) {
                     const long long r = g + (long long)nwarps * s;
@@ -663,7 +641,12 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
     return r;
 }
 
-// trilinear_x<true> with the two z planes of every stage in one register pair.
+// Trilinear value and gradient at a 32.32 index u inside [0, n-1]^3, read from the extended volume (dims
+// n + 1 per axis): the cell is the integer part of u and the weight its fraction, also on the last plane,
+// where the extension makes the value v[n-1] and the derivative v[n-1] - v[n-2] (those of the last cell of
+// the volume).  m0 = n0 + 1 and m01 = (n0 + 1)(n1 + 1): element offsets fit 32 bits (the extended volume
+// holds fewer than 2^31 elements, checked when the context is created).  The two z planes of every stage
+// share a register pair.
 __device__ __forceinline__ MG trilinear_x2(const float *__restrict__ movx, int m0, int m01, long long Ux, long long Uy,
                                            long long Uz) {
     constexpr float k2m32 = 2.3283064365386963e-10f;  // 2^-32

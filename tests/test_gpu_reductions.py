@@ -130,3 +130,29 @@ def test_adjoint_tables(cuda_lib, bins, nq, sampled):
             _, want, _ = oracle.parzen(f, m, aff, b, qs, daff=J, mask=mask)
             for iq in range(nq):
                 assert np.abs(got[iq] - want[iq]).max() <= 1e-4 * np.abs(want[iq]).max(), (t, b, iq)
+
+
+def test_parzen_row_clipping(cuda_lib):
+    """Overlap counts and MI where a row's interval comes from very small, zero, negative and very large
+    steps, on a dark, a bright and a full-range volume."""
+    rng = np.random.default_rng(81)
+    base = np.array([1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0], np.float32)
+    prm = np.repeat(base[None], 8, axis=0)
+    prm[1, [0, 3]] = (-1.0, 0.25)
+    prm[2, 0] = 0.0
+    prm[3, [0, 5]] = (1e-7, -1e-7)
+    prm[4, [0, 7]] = (37.0, 2.5)
+    prm[5, 0] = -3e-10
+    prm[6, [0, 4, 8]] = (0.7, 0.7, -0.7)
+    prm[7, [0, 10]] = (-250.0, 0.5)
+    for shape, lo, hi, bins in (((9, 17, 70), 0.0, 0.1, 8), ((9, 17, 70), 0.93, 1.0, 128), ((12, 9, 33), 0.0, 1.0, 64)):
+        f, m = (rng.uniform(lo, hi, shape).astype(np.float32) for _ in range(2))
+        f[:, :, :9] = rng.uniform(0, 1)
+        ctx = cuda_lib.Context(f, m, bins=bins, kernel="parzen", transform="affine")
+        mi, _, cnt = ctx.eval(prm, [1.0, 2.0], with_entropies=True)
+        for t in range(len(prm)):
+            aff = oracle.affine(prm[t], f.shape, (1, 1, 1), m.shape, (1, 1, 1), transform="affine")
+            want, _, n = oracle.parzen(f, m, aff, bins, [1.0, 2.0])
+            assert cnt[t] == n, (t, cnt[t], n)
+            if n > 1:
+                assert np.all(np.abs(mi[t] - want) <= 1e-6 * np.maximum(np.abs(want), 1.0)), (t, mi[t], want)
