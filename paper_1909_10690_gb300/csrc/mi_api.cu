@@ -1188,7 +1188,8 @@ void plan_items(const mi_ctx *ctx, const std::vector<int> &pair_of, int t0, int 
         double parts = 1.0;
         if (mode != kPlanWhole) {
             parts = once ? floor(c * P / total) : std::min(ceil(2.0 * c * P / left), floor(c / (8.0 * overhead(pair))));
-            const long long blocks = ((long long)p.nf[1] * p.nf[2] + nwarps - 1) / nwarps;
+            const int block_rows = nwarps * walk_rows_per_step(hv_fetch(ch.variant), ch.tile.lpr_log2, p.srow.p != nullptr);
+            const long long blocks = ((long long)p.nf[1] * p.nf[2] + block_rows - 1) / block_rows;
             parts = std::max(1.0, std::min({parts, (double)P, (double)blocks, 65535.0}));
         }
         left -= c;

@@ -102,6 +102,10 @@ struct Tile {
     int slabs;
 };
 constexpr int kMaxSlabs = 16;
+// Fixed rows each warp takes of a row block: the row-group walk's rows per step, else one.
+__host__ __device__ inline int walk_rows_per_step(int fetch, int lpr_log2, bool sampled) {
+    return fetch >= FM_QUAD && lpr_log2 > 0 && !sampled ? 32 >> lpr_log2 : 1;
+}
 
 // Shared memory needed by a hard-path CTA of `threads` threads for `bins` bins
 // (rows_words: words of the row-bound layout, used by HV_ROWS*).
