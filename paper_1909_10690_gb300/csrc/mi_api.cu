@@ -675,7 +675,9 @@ mi_status add_pair(mi_ctx *ctx, const mi_volume *fx, const mi_volume *mv, int bi
             DevBuf quads;
             MI_CU(quads.ensure(qext.width * qext.height * qext.depth * qsz), "allocating the quads");
             MI_CU(launch_make_quads(P->mov.p, P->mdtype, P->nm, quads.p, s), "building the quads");
-            cudaChannelFormatDesc cq = cudaCreateChannelDesc(cb, cb, cb, cb, cudaChannelFormatKindUnsigned);
+            // (8-bit quads are one 32-bit texel: the kernels interpolate its bytes two at a time)
+            cudaChannelFormatDesc cq = cb == 8 ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned)
+                                               : cudaCreateChannelDesc(cb, cb, cb, cb, cudaChannelFormatKindUnsigned);
             MI_CU(cudaMalloc3DArray(&P->arrq, &cq, qext), "allocating the quad array");
             cudaMemcpy3DParms cq3;
             memset(&cq3, 0, sizeof cq3);

@@ -20,7 +20,8 @@ struct PairDev {
     const void *movp;      // x-paired copy (v[x], v[x+1]), uint16 / uint32, dims (nx, ny + 1, nz + 1)
     unsigned long long texp;  // the same pairs as a 3D texture (point sampling, clamped), dims (nx, ny, nz)
     unsigned long long texq;  // 2 x 2 quads (y, z), (y + 1, z), (y, z + 1), (y + 1, z + 1) as a 3D texture
-    unsigned long long texg;  // z-pair texels v(x, y, z) | v(x, y, z + 1) << 20 in a 2D atlas, read by gathers
+                              // (one 32-bit texel of four bytes for uint8 volumes)
+    unsigned long long texg;  // z-pair texels v(x, y, z) | v(x, y, z + 1) << 20 (uint8: << 16) in a 2D atlas, gathered
                               // (moving depth <= 12 only; 0 when not built)
     const float2 *zoff;       // per moving plane z: atlas offset of the plane + 1 - 2^23, (x, y)
     const uint32_t *rowinfo;  // row-bound layout: per fixed bin, word offset << 6 | wide << 5 | shift (0 or 16)
@@ -134,7 +135,7 @@ cudaError_t set_drain_cap(int cap);
 cudaError_t launch_make_quads(const void *mov, int dtype, const int nm[3], void *out, cudaStream_t s);
 // z-pair atlas of the moving volume (depth <= 12): out is a W x H uint32 image (zeroed here) in which
 // plane z occupies the nm[0] x nm[1] tile at ((z / ph) nm[0], (z % ph) nm[1]) and texel (x, y) of that
-// tile holds v(x, y, z) | v(x, y, min(z + 1, nm[2] - 1)) << 20.
+// tile holds v(x, y, z) | v(x, y, min(z + 1, nm[2] - 1)) << 20 (<< 16 for uint8).
 cudaError_t launch_make_zpairs(const void *mov, int dtype, const int nm[3], int ph, int W, int H, uint32_t *out,
                                cudaStream_t s);
 cudaError_t launch_bin_fixed(const void *data, int dtype, int depth, long long n, int bins, uint8_t *out,

@@ -156,3 +156,30 @@ def test_parzen_row_clipping(cuda_lib):
             assert cnt[t] == n, (t, cnt[t], n)
             if n > 1:
                 assert np.all(np.abs(mi[t] - want) <= 1e-6 * np.maximum(np.abs(want), 1.0)), (t, mi[t], want)
+
+
+@pytest.mark.parametrize("variant", ["HV_U32_QUAD", "HV_U16_QUAD", "HV_ROWS_QUAD", "HV_U32_GATHER", "HV_U16_GATHER", "HV_ROWS_GATHER"])
+@pytest.mark.parametrize("rows", [1, 2, 4, 32])
+def test_byte_volumes_in_paired_lanes(cuda_lib, variant, rows):
+    """8-bit moving volumes at full range (0 and 255 beside each other: the largest 16-bit lane sums), through
+    both texture fetches and every walk, whole and split: histograms equal the oracle's, also in a
+    context that holds a 16-bit pair beside them; 31 fixed rows a slice leave every group ragged."""
+    rng = np.random.default_rng(83)
+    f = rng.integers(0, 256, (9, 31, 45), dtype=np.uint8)
+    m = np.where(rng.random((11, 27, 40)) < 0.5, 0, 255).astype(np.uint8)
+    m[:5] = rng.integers(0, 256, (5, 27, 40), dtype=np.uint8)
+    kw = dict(hist_variant=getattr(cuda_lib, variant), tile_rows=rows)
+    prm = phantoms.random_transforms(4, seed=84, t_mm=3, r_deg=20, s_range=(0.8, 1.2))
+    ctx = cuda_lib.Context(f, m, bins=64, **kw)
+    f16, m16 = phantoms.head_pair(shape=(12, 14, 20), spacing=(1, 1, 1), seed=85)
+    both = cuda_lib.Context(pairs=[dict(fixed=f, moving=m, bins=64),
+                                   dict(fixed=f16, moving=m16, bins=32, fixed_depth=12, moving_depth=12)], **kw)
+    got, _, cnt = both.batch_eval(np.zeros(4, np.int32), prm, [1.0, 2.0], with_entropies=True)
+    mi_o, h_o, cnt_o = oracle.mi_eval(f, m, 64, prm, [1.0, 2.0], nthreads=8)
+    np.testing.assert_array_equal(cnt, cnt_o)
+    assert np.all(np.abs(got - mi_o) <= 1e-6 * np.maximum(np.abs(mi_o), h_o[..., 2]) + 1e-12)
+    for path in (cuda_lib.PATH_PLAIN, cuda_lib.PATH_BATCHED):
+        H = ctx.hist(transforms=prm, path=path)
+        for t in range(4):
+            q16 = oracle.affine_q16(oracle.affine(prm[t], f.shape, (1, 1, 1), m.shape, (1, 1, 1)))
+            np.testing.assert_array_equal(H[t], oracle.joint_hist(f, m, q16, 64)[0].astype(np.uint32))
