@@ -1071,7 +1071,9 @@ bool variant_fits(int variant, int bins, int threads, long long nvox, int rows_w
 
 // Walks the tile shape may take for a variant: quad and gather fetches walk the warp's 32 rows as one
 // voxel stream (lpr_log2 0) or 1, 2 or 4 rows per step (lanes per row 2^5, 2^4, 2^3); the others one
-// row at a time.
+// row at a time.  With a step's rows beside one another four rows win nearly everywhere (four, two, one rows
+// and the stream, quads: 608 transforms of 256^3 at 256 bins 19.3, 20.1, 22.7 and 23.2 ms; 288 of 144 x 144 x 96
+// at 64 bins 1.10, 1.21, 1.36 and 1.40; eight rows 21.2 and 3 % more), so one row is tried only when asked for.
 std::vector<int> tile_lpr(mi_ctx *ctx, int variant) {
     if (hv_fetch(variant) < FM_QUAD) return {5};
     switch (ctx->opt.tile_rows) {
@@ -1079,7 +1081,7 @@ std::vector<int> tile_lpr(mi_ctx *ctx, int variant) {
         case 2: return {4};
         case 4: return {3};
         case 32: return {0};  // the warp's 32 rows as one voxel stream
-        default: return {0, 5, 4};
+        default: return {0, 4, 3};
     }
 }
 
@@ -1108,32 +1110,30 @@ std::vector<Choice> candidates(mi_ctx *ctx, int bins, long long nvox_max) {
     return c;
 }
 
-// The plain path's variant (it is not autotuned): the first of these kinds that fits, 1024 threads.  A few
-// transforms wait for the moving volume's first use, where the gather atlas is half the quads' bytes; from
-// kPlainQuads on its reuse weighs more and the quads' fewer instructions win.  A lone transform's parts are
-// a dozen rows a warp, whose ends the stream walk packs; more take two rows a step.  128 bins, 256 x 256 x
-// 160, us: one transform 72 (gather, stream), 74 (two rows), above 79 (quads); 8: 288 gather, 300 quads;
-// 24: 705 and 690; 81: 2201 and 2035.
-constexpr int kPlainQuads = 24, kPlainRows = 4;
+// The plain path's variant (it is not autotuned): the first of these kinds that fits, 1024 threads, four rows
+// a step.  A few transforms wait for the moving volume's first use, where the gather atlas is half the
+// quads' bytes; from kPlainQuads on its reuse weighs more and the quads' fewer instructions win.  us, gather
+// and quads: 256 x 256 x 160 at 128 bins, one transform 65 and 66, two 93 and 96, four 162 and 159, eight 262
+// and 251, 81 1990 and 1804; 256^3 at 256 bins, one 96 and 98, two 145 and 127, four 276 and 263.
+constexpr int kPlainQuads = 3;
 
 Choice plain_choice(mi_ctx *ctx, const std::vector<Choice> &cands, int n) {
     const int gather[] = {HV_U32_GATHER, HV_ROWS_GATHER, HV_U16_GATHER, HV_U32_QUAD, HV_ROWS_QUAD, HV_U16_QUAD,
                           HV_U32, HV_U16};
     const int quads[] = {HV_U32_QUAD, HV_ROWS_QUAD, HV_U16_QUAD, HV_U32, HV_U16};
     const bool many = n >= kPlainQuads;
-    const int lpr = n >= kPlainRows ? 4 : 0;
     for (const int *v = many ? quads : gather, *end = many ? std::end(quads) : std::end(gather); v != end; ++v) {
         if (hv_kind(*v) == HV_U32 && ctx->max_bins > 181) continue;
         for (const Choice &c : cands)
             if (c.variant == *v && (c.threads == 1024 || ctx->opt.block_threads) &&
-                (hv_fetch(*v) < FM_QUAD || ctx->opt.tile_rows || c.tile.lpr_log2 == lpr))
+                (hv_fetch(*v) < FM_QUAD || ctx->opt.tile_rows || c.tile.lpr_log2 == 3))
                 return c;
     }
     return cands.front();
 }
 
 // How the plain path's choices are kept: by the rule's ranges of the transform count.
-int plain_bucket(int n) { return n >= kPlainQuads ? 2 : n >= kPlainRows ? 1 : 0; }
+int plain_bucket(int n) { return n >= kPlainQuads ? 1 : 0; }
 
 // ---------------------------------------------------------------------------
 // Work items of a call
