@@ -301,15 +301,24 @@ struct Pair {
     int mdtype;  // stored moving type: 0 u8, 1 u16
     long long nvf, nvm;
     long long nsampled = 0;     // sampled fixed voxels (random sampling only)
-    DevBuf fbins, mov, movp;    // hard path (movp: x-paired moving volume)
+    // hard path: one allocation (row-bound table, plane offsets, fixed bins, moving volume clamped to its
+    // depth); what the fetches of a variant read (movp: x-paired moving volume, tex, texq, texg) is built
+    // when a call first needs it
+    DevBuf store;
+    uint8_t *fbins = nullptr;
+    void *mov = nullptr;
+    uint32_t *rowinfo = nullptr;  // row-bound layout table (bins entries)
+    float2 *zoff = nullptr;       // per moving plane: atlas offset + 1 - 2^23
+    std::vector<char> meta;       // what goes up to the table and the offsets
+    int atlas_rows = 0;           // planes a column of the z-pair atlas (0: the pair has none)
+    DevBuf movp;
     cudaArray_t arr = nullptr;  // the pairs as a 3D array, read through tex
     cudaTextureObject_t tex = 0;
     cudaArray_t arrq = nullptr;  // 2 x 2 (y, z) quads as a 3D array, read through texq
     cudaTextureObject_t texq = 0;
+    cudaSurfaceObject_t surfq = 0, surfg = 0;  // what the layout kernels write arrq and arrg through
     cudaArray_t arrg = nullptr;  // z-pair atlas (moving depth <= 12), read by 2D gathers through texg
     cudaTextureObject_t texg = 0;
-    DevBuf zoff;                 // per moving plane: float2 atlas offset + 1 - 2^23
-    DevBuf rowinfo;             // row-bound layout table (bins entries)
     DevBuf srow, scol, sbin;    // random sampling: per-row lists of the sampled fixed voxels
     int rows_words = 0;
     DevBuf pfbins, pmov, pmovx;  // Parzen path (pmovx: pmov extended by one plane per axis)
@@ -319,8 +328,10 @@ struct Pair {
         if (tex) cudaDestroyTextureObject(tex);
         if (arr) cudaFreeArray(arr);
         if (texq) cudaDestroyTextureObject(texq);
+        if (surfq) cudaDestroySurfaceObject(surfq);
         if (arrq) cudaFreeArray(arrq);
         if (texg) cudaDestroyTextureObject(texg);
+        if (surfg) cudaDestroySurfaceObject(surfg);
         if (arrg) cudaFreeArray(arrg);
         if (ptex) cudaDestroyTextureObject(ptex);
         if (parr) cudaFreeArray(parr);
@@ -349,7 +360,8 @@ struct mi_ctx {
     mi_options opt;
     std::string err;
     std::vector<std::unique_ptr<Pair>> pairs;
-    DevBuf d_pairs;     // PairDev[npairs]
+    DevBuf d_pairs;     // PairDev[npairs], uploaded from v_pairs when layouts are built
+    std::vector<PairDev> v_pairs;
     int max_bins = 0;
     int max_rows_words = 0;
     int max_zplanes = 0;      // moving planes of the largest pair (gather offsets in shared memory)
@@ -463,13 +475,23 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 size_t dtype_size(int dt) { return dt == MI_U8 ? 1 : (dt == MI_U16 ? 2 : 4); }
 
-// Copy a caller volume (host or device) into a fresh device buffer.
-mi_status upload_volume(mi_ctx *ctx, const mi_volume *v, DevBuf &dst) {
-    const size_t bytes = (size_t)v->dims[0] * v->dims[1] * v->dims[2] * dtype_size(v->dtype);
-    MI_CU(dst.ensure(bytes), "allocating a volume");
-    MI_CU(cudaMemcpyAsync(dst.p, v->data, bytes, is_device_ptr(v->data) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                          ctx->stream),
-          "copying a volume to the device");
+// A caller's volume in device memory: where it is if the kernels can read it there (memory of this device,
+// aligned to its elements), else a copy in `copy`.
+mi_status device_volume(mi_ctx *ctx, const mi_volume *v, DevBuf &copy, const void **data) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, v->data) != cudaSuccess) {
+        cudaGetLastError();
+        at.type = cudaMemoryTypeUnregistered;
+    }
+    const size_t esz = dtype_size(v->dtype);
+    if (at.type == cudaMemoryTypeDevice && at.device == ctx->device && (uintptr_t)v->data % esz == 0) {
+        *data = v->data;
+        return MI_OK;
+    }
+    const size_t bytes = (size_t)v->dims[0] * v->dims[1] * v->dims[2] * esz;
+    MI_CU(copy.ensure(bytes), "allocating a volume");
+    MI_CU(cudaMemcpyAsync(copy.p, v->data, bytes, cudaMemcpyDefault, ctx->stream), "copying a volume to the device");
+    *data = copy.p;
     return MI_OK;
 }
 
@@ -548,14 +570,15 @@ mi_status add_pair(mi_ctx *ctx, const mi_volume *fx, const mi_volume *mv, int bi
     P->nvm = (long long)P->nm[0] * P->nm[1] * P->nm[2];
     cudaStream_t s = ctx->stream;
     DevBuf rawf, rawm;
-    if ((st = upload_volume(ctx, fx, rawf)) != MI_OK) return st;
-    if ((st = upload_volume(ctx, mv, rawm)) != MI_OK) return st;
+    const void *fdata, *mdata;
+    if ((st = device_volume(ctx, fx, rawf, &fdata)) != MI_OK) return st;
+    if ((st = device_volume(ctx, mv, rawm, &mdata)) != MI_OK) return st;
     if (parzen) {
         MI_CU(P->pfbins.ensure((size_t)P->nvf), "allocating Parzen fixed bins");
-        MI_CU(launch_parzen_prep_fixed(rawf.p, fx->dtype, P->fdepth, P->nvf, bins, P->pfbins.as<uint8_t>(), s),
+        MI_CU(launch_parzen_prep_fixed(fdata, fx->dtype, P->fdepth, P->nvf, bins, P->pfbins.as<uint8_t>(), s),
               "Parzen fixed bins");
         MI_CU(P->pmov.ensure((size_t)P->nvm * 4), "allocating the normalised moving volume");
-        MI_CU(launch_parzen_prep_moving(rawm.p, mv->dtype, P->mdepth, P->nvm, P->pmov.as<float>(), s),
+        MI_CU(launch_parzen_prep_moving(mdata, mv->dtype, P->mdepth, P->nvm, P->pmov.as<float>(), s),
               "normalising the moving volume");
         MI_CU(P->pmovx.ensure((size_t)(P->nm[0] + 1) * (P->nm[1] + 1) * (P->nm[2] + 1) * 4),
               "allocating the extended moving volume");
@@ -590,106 +613,51 @@ mi_status add_pair(mi_ctx *ctx, const mi_volume *fx, const mi_volume *mv, int bi
         }
         P->mdtype = 1;
     } else {
-        // fixed: float -> 16-bit first, then bins
+        // fixed: float -> 16-bit first, then bins and their counts; moving: 16-bit, clamped to its depth
+        P->mdtype = mv->dtype == MI_U8 ? 0 : 1;
+        const size_t counts_at = 1024, zoff_at = counts_at + 2048, meta_bytes = align256(zoff_at + (size_t)P->nm[2] * 8),
+                     mov_at = meta_bytes + align256((size_t)P->nvf);
+        MI_CU(P->store.ensure(mov_at + (size_t)P->nvm * (P->mdtype == 0 ? 1 : 2)), "allocating the volumes");
+        char *store = P->store.as<char>();
+        P->rowinfo = (uint32_t *)store;
+        P->zoff = (float2 *)(store + zoff_at);
+        P->fbins = (uint8_t *)(store + meta_bytes);
+        P->mov = store + mov_at;
+        auto *d_counts = (unsigned long long *)(store + counts_at);
         int fdt = fx->dtype;
-        const void *fsrc = rawf.p;
         DevBuf conv;
         if (fdt == MI_F32) {
             MI_CU(conv.ensure((size_t)P->nvf * 2), "allocating a conversion buffer");
-            MI_CU(launch_f32_to_u16(rawf.as<float>(), P->nvf, conv.as<uint16_t>(), s), "converting the fixed volume");
-            fsrc = conv.p;
+            MI_CU(launch_f32_to_u16((const float *)fdata, P->nvf, conv.as<uint16_t>(), s), "converting the fixed volume");
+            fdata = conv.p;
             fdt = MI_U16;
         }
-        MI_CU(P->fbins.ensure((size_t)P->nvf), "allocating fixed bins");
-        MI_CU(launch_bin_fixed(fsrc, fdt, P->fdepth, P->nvf, bins, P->fbins.as<uint8_t>(), s), "binning the fixed volume");
+        MI_CU(launch_bin_fixed(fdata, fdt, P->fdepth, P->nvf, bins, P->fbins, d_counts, s), "binning the fixed volume");
+        unsigned long long F[256];
+        MI_CU(cudaMemcpyAsync(F, d_counts, (size_t)bins * 8, cudaMemcpyDeviceToHost, s), "bin counts D2H");
+        if (mv->dtype == MI_F32)
+            MI_CU(launch_f32_to_u16((const float *)mdata, P->nvm, (uint16_t *)P->mov, s), "converting the moving volume");
+        else
+            MI_CU(launch_copy_clamp(mdata, P->mdtype, P->mdepth, P->nvm, P->mov, s), "copying the moving volume");
+        MI_CU(cudaStreamSynchronize(s), "bin counts");
         // row-bound layout: a row whose bin holds at most 65535 fixed voxels can never count past 16 bits
-        {
-            DevBuf dF;
-            std::vector<unsigned long long> F(bins);
-            MI_CU(dF.ensure((size_t)bins * 8), "allocating bin counts");
-            MI_CU(launch_fixed_hist(P->fbins.as<uint8_t>(), P->nvf, bins, dF.as<unsigned long long>(), s), "bin counts");
-            MI_CU(cudaMemcpyAsync(F.data(), dF.p, (size_t)bins * 8, cudaMemcpyDeviceToHost, s), "bin counts D2H");
-            MI_CU(cudaStreamSynchronize(s), "bin counts");
-            std::vector<uint32_t> info(bins);
-            const uint32_t S = (uint32_t)bins + 1;
-            uint32_t off = 0;
-            for (int r = 0; r < bins; ++r)
-                if (F[r] > 65535) {
-                    info[r] = off << 6 | 32u;
-                    off += S;
-                }
-            int k = 0;
-            for (int r = 0; r < bins; ++r)
-                if (F[r] <= 65535) {
-                    info[r] = (off + (uint32_t)(k / 2) * S) << 6 | (uint32_t)(k % 2 ? 16 : 0);
-                    ++k;
-                }
-            off += (uint32_t)((k + 1) / 2) * S;
-            P->rows_words = (int)off;
-            MI_CU(P->rowinfo.ensure((size_t)bins * 4), "allocating the row table");
-            MI_CU(cudaMemcpyAsync(P->rowinfo.p, info.data(), (size_t)bins * 4, cudaMemcpyHostToDevice, s), "row table");
-            MI_CU(cudaStreamSynchronize(s), "row table");
-        }
-        if ((st = build_samples(ctx, *P, P->fbins.as<uint8_t>(), s)) != MI_OK) return st;
-        if (mv->dtype == MI_F32) {
-            MI_CU(P->mov.ensure((size_t)P->nvm * 2), "allocating the moving volume");
-            MI_CU(launch_f32_to_u16(rawm.as<float>(), P->nvm, P->mov.as<uint16_t>(), s), "converting the moving volume");
-            P->mdtype = 1;
-        } else {
-            MI_CU(P->mov.ensure((size_t)P->nvm * dtype_size(mv->dtype)), "allocating the moving volume");
-            MI_CU(cudaMemcpyAsync(P->mov.p, rawm.p, (size_t)P->nvm * dtype_size(mv->dtype), cudaMemcpyDeviceToDevice, s),
-                  "copying the moving volume");
-            P->mdtype = mv->dtype == MI_U8 ? 0 : 1;
-            MI_CU(launch_clamp_depth(P->mov.p, P->mdtype, P->mdepth, P->nvm, s), "clamping the moving volume");
-        }
-        const size_t npairs = (size_t)P->nm[0] * (P->nm[1] + 1) * (P->nm[2] + 1);
-        MI_CU(P->movp.ensure(npairs * (P->mdtype == 0 ? 2 : 4)), "allocating the paired moving volume");
-        MI_CU(launch_make_pairs(P->mov.p, P->mdtype, P->nm, P->movp.p, s), "pairing the moving volume");
-        // the same pairs (without the padding row / plane) as a 3D array for the texture path
-        const size_t esz = P->mdtype == 0 ? 2 : 4;
-        cudaChannelFormatDesc cd = cudaCreateChannelDesc((int)esz * 8, 0, 0, 0, cudaChannelFormatKindUnsigned);
-        MI_CU(cudaMalloc3DArray(&P->arr, &cd, make_cudaExtent(P->nm[0], P->nm[1], P->nm[2])), "allocating the 3D array");
-        cudaMemcpy3DParms cp;
-        memset(&cp, 0, sizeof cp);
-        cp.srcPtr = make_cudaPitchedPtr(P->movp.p, (size_t)P->nm[0] * esz, P->nm[0], P->nm[1] + 1);
-        cp.dstArray = P->arr;
-        cp.extent = make_cudaExtent(P->nm[0], P->nm[1], P->nm[2]);
-        cp.kind = cudaMemcpyDeviceToDevice;
-        MI_CU(cudaMemcpy3DAsync(&cp, s), "filling the 3D array");
-        cudaResourceDesc rd;
-        memset(&rd, 0, sizeof rd);
-        rd.resType = cudaResourceTypeArray;
-        rd.res.array.array = P->arr;
-        cudaTextureDesc td;
-        memset(&td, 0, sizeof td);
-        td.addressMode[0] = td.addressMode[1] = td.addressMode[2] = cudaAddressModeClamp;
-        td.filterMode = cudaFilterModePoint;
-        td.readMode = cudaReadModeElementType;
-        td.normalizedCoords = 0;
-        MI_CU(cudaCreateTextureObject(&P->tex, &rd, &td, nullptr), "creating the texture object");
-        // 2 x 2 (y, z) quads (uchar4 / ushort4), read at integer texel coordinates
-        {
-            const int cb = P->mdtype == 0 ? 8 : 16;
-            const size_t qsz = (size_t)cb / 2;  // bytes per quad
-            const cudaExtent qext = make_cudaExtent(P->nm[0], P->nm[1], P->nm[2]);
-            DevBuf quads;
-            MI_CU(quads.ensure(qext.width * qext.height * qext.depth * qsz), "allocating the quads");
-            MI_CU(launch_make_quads(P->mov.p, P->mdtype, P->nm, quads.p, s), "building the quads");
-            // (8-bit quads are one 32-bit texel: the kernels interpolate its bytes two at a time)
-            cudaChannelFormatDesc cq = cb == 8 ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned)
-                                               : cudaCreateChannelDesc(cb, cb, cb, cb, cudaChannelFormatKindUnsigned);
-            MI_CU(cudaMalloc3DArray(&P->arrq, &cq, qext), "allocating the quad array");
-            cudaMemcpy3DParms cq3;
-            memset(&cq3, 0, sizeof cq3);
-            cq3.srcPtr = make_cudaPitchedPtr(quads.p, qext.width * qsz, qext.width, qext.height);
-            cq3.dstArray = P->arrq;
-            cq3.extent = qext;
-            cq3.kind = cudaMemcpyDeviceToDevice;
-            MI_CU(cudaMemcpy3DAsync(&cq3, s), "filling the quad array");
-            rd.res.array.array = P->arrq;
-            MI_CU(cudaCreateTextureObject(&P->texq, &rd, &td, nullptr), "creating the quad texture object");
-            MI_CU(cudaStreamSynchronize(s), "building the quads");
-        }
+        P->meta.assign(meta_bytes, 0);
+        uint32_t *info = (uint32_t *)P->meta.data();
+        const uint32_t S = (uint32_t)bins + 1;
+        uint32_t off = 0;
+        for (int r = 0; r < bins; ++r)
+            if (F[r] > 65535) {
+                info[r] = off << 6 | 32u;
+                off += S;
+            }
+        int k = 0;
+        for (int r = 0; r < bins; ++r)
+            if (F[r] <= 65535) {
+                info[r] = (off + (uint32_t)(k / 2) * S) << 6 | (uint32_t)(k % 2 ? 16 : 0);
+                ++k;
+            }
+        off += (uint32_t)((k + 1) / 2) * S;
+        P->rows_words = (int)off;
         // z-pair atlas for moving depths <= 12: plane z is the tile at ((z / ph) nx, (z % ph) ny) of a 2D
         // image no larger than the device's gather extent; a gather at (ix + 1 + ox, iy + 1 + oy) returns
         // the plane's 2 x 2 footprint with each texel's z + 1 neighbour packed beside it
@@ -701,69 +669,154 @@ mi_status add_pair(mi_ctx *ctx, const mi_volume *fx, const mi_volume *mv, int bi
             const int ph = std::min(nz, gh / ny);
             const int cols = ph > 0 ? (nz + ph - 1) / ph : 0;
             if (ph > 0 && (long long)cols * nx <= gw) {
-                const int W = cols * nx, H = ph * ny;
-                DevBuf img;
-                MI_CU(img.ensure((size_t)W * H * 4), "allocating the z-pair atlas");
-                MI_CU(launch_make_zpairs(P->mov.p, P->mdtype, P->nm, ph, W, H, img.as<uint32_t>(), s),
-                      "building the z-pair atlas");
-                cudaChannelFormatDesc cg = cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned);
-                MI_CU(cudaMallocArray(&P->arrg, &cg, W, H, cudaArrayTextureGather), "allocating the z-pair array");
-                MI_CU(cudaMemcpy2DToArrayAsync(P->arrg, 0, 0, img.p, (size_t)W * 4, (size_t)W * 4, H,
-                                               cudaMemcpyDeviceToDevice, s),
-                      "filling the z-pair array");
-                rd.res.array.array = P->arrg;
-                MI_CU(cudaCreateTextureObject(&P->texg, &rd, &td, nullptr), "creating the z-pair texture object");
-                std::vector<float2> off(nz);
+                P->atlas_rows = ph;
+                float2 *zo = (float2 *)(P->meta.data() + zoff_at);
                 for (int z = 0; z < nz; ++z) {
-                    off[z].x = (float)((z / ph) * nx + 1) - 8388608.0f;
-                    off[z].y = (float)((z % ph) * ny + 1) - 8388608.0f;
+                    zo[z].x = (float)((z / ph) * nx + 1) - 8388608.0f;
+                    zo[z].y = (float)((z % ph) * ny + 1) - 8388608.0f;
                 }
-                MI_CU(P->zoff.ensure((size_t)nz * sizeof(float2)), "allocating the plane offsets");
-                MI_CU(cudaMemcpyAsync(P->zoff.p, off.data(), (size_t)nz * sizeof(float2), cudaMemcpyHostToDevice, s),
-                      "plane offsets");
-                MI_CU(cudaStreamSynchronize(s), "building the z-pair atlas");
             }
         }
+        MI_CU(cudaMemcpyAsync(store, P->meta.data(), meta_bytes, cudaMemcpyHostToDevice, s), "pair tables");
+        if ((st = build_samples(ctx, *P, P->fbins, s)) != MI_OK) return st;
     }
-    MI_CU(cudaStreamSynchronize(s), "preparing the volumes");
+    // what read the caller's volumes has been waited for; buffers of this call are freed in stream order
+    if (parzen || rawf.p || rawm.p) MI_CU(cudaStreamSynchronize(s), "preparing the volumes");
     ctx->max_bins = std::max(ctx->max_bins, bins);
     ctx->max_rows_words = std::max(ctx->max_rows_words, P->rows_words);
     ctx->max_zplanes = std::max(ctx->max_zplanes, P->nm[2]);
-    if (!P->texg) ctx->all_gather = false;
+    if (!parzen && P->atlas_rows == 0) ctx->all_gather = false;
     ctx->pairs.push_back(std::move(P));
     return MI_OK;
 }
 
-mi_status upload_pairs(mi_ctx *ctx) {
-    std::vector<PairDev> pd(ctx->pairs.size());
-    for (size_t i = 0; i < ctx->pairs.size(); ++i) {
-        const Pair &P = *ctx->pairs[i];
-        PairDev &d = pd[i];
-        memset(&d, 0, sizeof d);
-        d.fbins = P.fbins.as<uint8_t>();
-        d.mov = P.mov.p;
-        d.movp = P.movp.p;
-        d.texp = P.tex;
-        d.texq = P.texq;
-        d.texg = P.texg;
-        d.zoff = P.zoff.as<float2>();
-        d.rowinfo = P.rowinfo.as<uint32_t>();
-        d.srow = P.srow.p ? P.srow.as<uint32_t>() : nullptr;
-        d.scol = P.scol.as<uint16_t>();
-        d.sbin = P.sbin.as<uint8_t>();
-        d.rows_words = P.rows_words;
-        for (int a = 0; a < 3; ++a) {
-            d.nf[a] = P.nf[a];
-            d.nm[a] = P.nm[a];
-        }
-        d.bins = P.bins;
-        d.mdepth = P.mdepth;
-        d.mdtype = P.mdtype;
+PairDev host_pairdev(const Pair &P) {
+    PairDev d;
+    memset(&d, 0, sizeof d);
+    d.fbins = P.fbins;
+    d.mov = P.mov;
+    d.movp = P.movp.p;
+    d.texp = P.tex;
+    d.texq = P.texq;
+    d.texg = P.texg;
+    d.zoff = P.zoff;
+    d.rowinfo = P.rowinfo;
+    d.srow = P.srow.p ? P.srow.as<uint32_t>() : nullptr;
+    d.scol = P.scol.as<uint16_t>();
+    d.sbin = P.sbin.as<uint8_t>();
+    d.rows_words = P.rows_words;
+    for (int a = 0; a < 3; ++a) {
+        d.nf[a] = P.nf[a];
+        d.nm[a] = P.nm[a];
     }
+    d.bins = P.bins;
+    d.mdepth = P.mdepth;
+    d.mdtype = P.mdtype;
+    return d;
+}
+
+cudaError_t array_surface(cudaArray_t arr, cudaSurfaceObject_t *surf) {
+    if (*surf) return cudaSuccess;
+    cudaResourceDesc rd;
+    memset(&rd, 0, sizeof rd);
+    rd.resType = cudaResourceTypeArray;
+    rd.res.array.array = arr;
+    return cudaCreateSurfaceObject(surf, &rd);
+}
+
+// A point-sampled texture of a whole array with clamped addressing.
+cudaError_t array_texture(cudaArray_t arr, cudaTextureObject_t *tex) {
+    cudaResourceDesc rd;
+    memset(&rd, 0, sizeof rd);
+    rd.resType = cudaResourceTypeArray;
+    rd.res.array.array = arr;
+    cudaTextureDesc td;
+    memset(&td, 0, sizeof td);
+    td.addressMode[0] = td.addressMode[1] = td.addressMode[2] = cudaAddressModeClamp;
+    td.filterMode = cudaFilterModePoint;
+    td.readMode = cudaReadModeElementType;
+    td.normalizedCoords = 0;
+    return cudaCreateTextureObject(tex, &rd, &td, nullptr);
+}
+
+// The padded x-pairs of the moving volume (FM_LDG) and, with tex, the same pairs (without the padding row
+// and plane) as a 3D array for the texture path.
+mi_status build_xpairs(mi_ctx *ctx, Pair &P, bool tex) {
+    cudaStream_t s = ctx->stream;
+    const size_t esz = P.mdtype == 0 ? 2 : 4;
+    if (!P.movp.p) {
+        MI_CU(P.movp.ensure((size_t)P.nm[0] * (P.nm[1] + 1) * (P.nm[2] + 1) * esz), "allocating the paired moving volume");
+        MI_CU(launch_make_pairs(P.mov, P.mdtype, P.nm, P.movp.p, s), "pairing the moving volume");
+    }
+    if (!tex || P.tex) return MI_OK;
+    if (!P.arr) {
+        cudaChannelFormatDesc cd = cudaCreateChannelDesc((int)esz * 8, 0, 0, 0, cudaChannelFormatKindUnsigned);
+        MI_CU(cudaMalloc3DArray(&P.arr, &cd, make_cudaExtent(P.nm[0], P.nm[1], P.nm[2])), "allocating the 3D array");
+    }
+    cudaMemcpy3DParms cp;
+    memset(&cp, 0, sizeof cp);
+    cp.srcPtr = make_cudaPitchedPtr(P.movp.p, (size_t)P.nm[0] * esz, P.nm[0], P.nm[1] + 1);
+    cp.dstArray = P.arr;
+    cp.extent = make_cudaExtent(P.nm[0], P.nm[1], P.nm[2]);
+    cp.kind = cudaMemcpyDeviceToDevice;
+    MI_CU(cudaMemcpy3DAsync(&cp, s), "filling the 3D array");
+    MI_CU(array_texture(P.arr, &P.tex), "creating the texture object");
+    return MI_OK;
+}
+
+// 2 x 2 (y, z) quads (four bytes in one 32-bit texel, or ushort4), written straight into their 3D array and
+// read at integer texel coordinates.
+mi_status build_quads(mi_ctx *ctx, Pair &P) {
+    if (P.texq) return MI_OK;
+    if (!P.arrq) {
+        // (8-bit quads are one 32-bit texel: the kernels interpolate its bytes two at a time)
+        cudaChannelFormatDesc cq = P.mdtype == 0 ? cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned)
+                                                 : cudaCreateChannelDesc(16, 16, 16, 16, cudaChannelFormatKindUnsigned);
+        MI_CU(cudaMalloc3DArray(&P.arrq, &cq, make_cudaExtent(P.nm[0], P.nm[1], P.nm[2]), cudaArraySurfaceLoadStore),
+              "allocating the quad array");
+    }
+    MI_CU(array_surface(P.arrq, &P.surfq), "creating the quad surface");
+    MI_CU(launch_make_quads(P.mov, P.mdtype, P.nm, P.surfq, ctx->stream), "building the quads");
+    MI_CU(array_texture(P.arrq, &P.texq), "creating the quad texture object");
+    return MI_OK;
+}
+
+mi_status build_atlas(mi_ctx *ctx, Pair &P) {
+    if (P.texg) return MI_OK;
+    const int ph = P.atlas_rows, cols = (P.nm[2] + ph - 1) / ph;
+    if (!P.arrg) {
+        cudaChannelFormatDesc cg = cudaCreateChannelDesc(32, 0, 0, 0, cudaChannelFormatKindUnsigned);
+        MI_CU(cudaMallocArray(&P.arrg, &cg, (size_t)cols * P.nm[0], (size_t)ph * P.nm[1],
+                              cudaArrayTextureGather | cudaArraySurfaceLoadStore),
+              "allocating the z-pair array");
+    }
+    MI_CU(array_surface(P.arrg, &P.surfg), "creating the z-pair surface");
+    MI_CU(launch_make_zpairs(P.mov, P.mdtype, P.nm, ph, P.surfg, ctx->stream), "building the z-pair atlas");
+    MI_CU(array_texture(P.arrg, &P.texg), "creating the z-pair texture object");
+    return MI_OK;
+}
+
+// Builds what the fetch modes in `modes` (bits 1 << FM_*) read and the pairs do not have yet, and brings the
+// device's pair descriptors up to date.  A context built all four layouts when it was created; one pose of
+// a new pair reads one (context, evaluation and release at 192 x 160 x 128: 1454 -> 693 us, most of it the
+// allocations and releases of volumes copied twice and of layouts that were not read).
+mi_status ensure_layouts(mi_ctx *ctx, unsigned modes) {
+    std::vector<PairDev> pd;
+    mi_status st;
+    for (auto &p : ctx->pairs) {
+        if ((modes & (1u << FM_LDG | 1u << FM_TEX)) && (st = build_xpairs(ctx, *p, modes >> FM_TEX & 1u)) != MI_OK) return st;
+        if ((modes >> FM_QUAD & 1u) && (st = build_quads(ctx, *p)) != MI_OK) return st;
+        if ((modes >> FM_GATHER & 1u) && (st = build_atlas(ctx, *p)) != MI_OK) return st;
+        pd.push_back(host_pairdev(*p));
+    }
+    if (ctx->d_pairs.p && pd.size() == ctx->v_pairs.size() &&
+        memcmp(pd.data(), ctx->v_pairs.data(), pd.size() * sizeof(PairDev)) == 0)
+        return MI_OK;
     MI_CU(ctx->d_pairs.ensure(pd.size() * sizeof(PairDev)), "allocating pair descriptors");
-    MI_CU(cudaMemcpyAsync(ctx->d_pairs.p, pd.data(), pd.size() * sizeof(PairDev), cudaMemcpyHostToDevice, ctx->stream),
+    ctx->v_pairs = pd;  // (kept: the copy may read it after this returns)
+    MI_CU(cudaMemcpyAsync(ctx->d_pairs.p, ctx->v_pairs.data(), pd.size() * sizeof(PairDev), cudaMemcpyHostToDevice,
+                          ctx->stream),
           "uploading pair descriptors");
-    MI_CU(cudaStreamSynchronize(ctx->stream), "uploading pair descriptors");
     return MI_OK;
 }
 
@@ -799,31 +852,6 @@ mi_status upload_parzen_pairs(mi_ctx *ctx) {
           "uploading Parzen pair descriptors");
     MI_CU(cudaStreamSynchronize(ctx->stream), "uploading Parzen pair descriptors");
     return MI_OK;
-}
-
-PairDev host_pairdev(const Pair &P) {
-    PairDev d;
-    memset(&d, 0, sizeof d);
-    d.fbins = P.fbins.as<uint8_t>();
-    d.mov = P.mov.p;
-    d.movp = P.movp.p;
-    d.texp = P.tex;
-    d.texq = P.texq;
-    d.texg = P.texg;
-    d.zoff = P.zoff.as<float2>();
-    d.rowinfo = P.rowinfo.as<uint32_t>();
-    d.srow = P.srow.p ? P.srow.as<uint32_t>() : nullptr;
-    d.scol = P.scol.as<uint16_t>();
-    d.sbin = P.sbin.as<uint8_t>();
-    d.rows_words = P.rows_words;
-    for (int a = 0; a < 3; ++a) {
-        d.nf[a] = P.nf[a];
-        d.nm[a] = P.nm[a];
-    }
-    d.bins = P.bins;
-    d.mdepth = P.mdepth;
-    d.mdtype = P.mdtype;
-    return d;
 }
 
 mi_status create_common(mi_ctx **out, const mi_volume *fixed, const mi_volume *moving, const int *bins, int npairs,
@@ -911,13 +939,6 @@ mi_status create_common(mi_ctx **out, const mi_volume *fixed, const mi_volume *m
     }
     if (ctx->opt.kernel == MI_PARZEN) {
         mi_status st = upload_parzen_pairs(ctx.get());
-        if (st != MI_OK) {
-            g_create_error = ctx->err;
-            return st;
-        }
-    }
-    if (ctx->opt.kernel == MI_HARD) {
-        mi_status st = upload_pairs(ctx.get());
         if (st != MI_OK) {
             g_create_error = ctx->err;
             return st;
@@ -1420,7 +1441,10 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
         const std::string cpath = ctx->opt.autotune && cands.size() > 1 ? cache_path() : std::string();
         const std::string ckey = cpath.empty() ? std::string() : tune_key(ctx, bucket, nq);
         if (cpath.empty() || !cache_lookup(cpath, ckey, cands, ch)) {
-            // tuning needs the affines and whole items on the device
+            // tuning needs every candidate's layout, the affines and whole items on the device
+            unsigned modes = 0;
+            for (const Choice &c : cands) modes |= 1u << hv_fetch(c.variant);
+            if ((st = ensure_layouts(ctx, modes)) != MI_OK) return st;
             HardPlan whole;
             plan_items(ctx, R.pair_of, 0, n, cands.front(), kPlanWhole, whole);
             const size_t aff_bytes = align256((size_t)n * 48), item_bytes = (size_t)n * sizeof(Item);
@@ -1441,6 +1465,7 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
         ctx->tuned[key] = ch;
     }
 
+    if ((st = ensure_layouts(ctx, 1u << hv_fetch(ch.variant))) != MI_OK) return st;
     // The plain path sums every histogram in global memory, in chunks of at most 64 MB of them; the
     // batched path reduces whole transforms in place and splits the last ones, unless the caller asked
     // for the batched path of a single pair by name or wants the histograms themselves.
@@ -1765,6 +1790,10 @@ const char *mi_last_error(const mi_ctx *ctx) { return ctx ? ctx->err.c_str() : g
 
 mi_status mi_set_stream(mi_ctx *ctx, void *stream) {
     if (!ctx) return MI_EINVAL;
+    {  // the pairs' tables and layouts were built on the stream so far
+        DeviceGuard guard(ctx->device);
+        MI_CU(cudaStreamSynchronize(ctx->stream), "switching streams");
+    }
     ctx->stream = stream ? (cudaStream_t)stream : ctx->own_stream;
     ctx->graphs.clear();
     return MI_OK;
@@ -1964,8 +1993,8 @@ mi_status mi_fixed_bins(mi_ctx *ctx, int pair, uint8_t *out) {
     DeviceGuard guard(ctx->device);
     if (pair < 0 || pair >= (int)ctx->pairs.size() || !out) return ctx->fail(MI_EINVAL, "bad pair or output");
     const Pair &P = *ctx->pairs[pair];
-    const DevBuf &src = ctx->opt.kernel == MI_PARZEN ? P.pfbins : P.fbins;
-    mi_status st = deliver(ctx, out, src.p, (size_t)P.nvf);
+    const void *src = ctx->opt.kernel == MI_PARZEN ? P.pfbins.p : P.fbins;
+    mi_status st = deliver(ctx, out, src, (size_t)P.nvf);
     if (st != MI_OK) return st;
     MI_CU(cudaStreamSynchronize(ctx->stream), "copying bins");
     return MI_OK;
@@ -1984,6 +2013,8 @@ mi_status mi_resample(mi_ctx *ctx, int pair, const int32_t *affine, void *out) {
     } else {
         memcpy(q, affine, 48);
     }
+    mi_status st2 = ensure_layouts(ctx, 0);
+    if (st2 != MI_OK) return st2;
     MI_CU(ctx->d_aff.ensure(48), "alloc");
     MI_CU(cudaMemcpyAsync(ctx->d_aff.p, q, 48, cudaMemcpyHostToDevice, ctx->stream), "H2D");
     const size_t bytes = (size_t)P.nvf * (P.mdtype == 0 ? 1 : 2);

@@ -49,22 +49,60 @@ __global__ void k_f32_to_u16(const float *__restrict__ in, long long n, uint16_t
     }
 }
 
+// Eight elements of a volume, loaded and stored at once where both are aligned to it.
 template <typename T>
-__global__ void k_clamp_depth(T *__restrict__ data, long long n, uint32_t vmax) {
-    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
-        uint32_t v = data[x];
-        if (v > vmax) data[x] = (T)vmax;
-    }
+struct alignas(8 * sizeof(T)) Eight {
+    T v[8];
+};
+
+template <typename T>
+bool aligned8(const void *p) {
+    return (uintptr_t)p % (8 * sizeof(T)) == 0;
 }
 
-// bin(v) = (min(v, 2^d - 1) * bins) >> d
 template <typename T>
-__global__ void k_bin_fixed(const T *__restrict__ in, long long n, int depth, int bins, uint8_t *__restrict__ out) {
+__global__ void k_copy_clamp(const T *__restrict__ in, long long n, uint32_t vmax, bool vec, T *__restrict__ out) {
+    const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    const long long groups = vec ? n / 8 : 0;
+    for (long long g = first; g < groups; g += step) {
+        Eight<T> e = ((const Eight<T> *)in)[g];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) e.v[k] = (T)min((uint32_t)e.v[k], vmax);
+        ((Eight<T> *)out)[g] = e;
+    }
+    for (long long x = 8 * groups + first; x < n; x += step) out[x] = (T)min((uint32_t)in[x], vmax);
+}
+
+// bin(v) = (min(v, 2^d - 1) * bins) >> d, and the voxels per bin (in shared memory, then one addition per
+// CTA and bin).
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_bin_fixed(const T *__restrict__ in, long long n, int depth, int bins, bool vec, uint8_t *__restrict__ out,
+                unsigned long long *__restrict__ counts) {
+    __shared__ unsigned int h[4][256];  // a copy per two warps
+    for (int c = threadIdx.x; c < 4 * 256; c += blockDim.x) (&h[0][0])[c] = 0;
+    __syncthreads();
+    unsigned int *mine = h[threadIdx.x >> 6];
     const uint32_t vmax = (uint32_t)((1ull << depth) - 1ull);
-    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
-        uint32_t v = in[x];
-        v = v > vmax ? vmax : v;
-        out[x] = (uint8_t)(((uint64_t)v * (uint32_t)bins) >> depth);
+    auto bin = [&](uint32_t v) {
+        const uint32_t b = (min(v, vmax) * (uint32_t)bins) >> depth;  // at most 65535 x 256
+        atomicAdd(&mine[b], 1u);
+        return (uint8_t)b;
+    };
+    const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    const long long groups = vec ? n / 8 : 0;
+    for (long long g = first; g < groups; g += step) {
+        const Eight<T> e = ((const Eight<T> *)in)[g];
+        Eight<uint8_t> o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o.v[k] = bin(e.v[k]);
+        ((Eight<uint8_t> *)out)[g] = o;
+    }
+    for (long long x = 8 * groups + first; x < n; x += step) out[x] = bin(in[x]);
+    __syncthreads();
+    for (int c = threadIdx.x; c < bins; c += blockDim.x) {
+        const unsigned int v = h[0][c] + h[1][c] + h[2][c] + h[3][c];
+        if (v) atomicAdd(counts + c, (unsigned long long)v);
     }
 }
 
@@ -247,40 +285,29 @@ __device__ __forceinline__ int quad_value8(unsigned long long tex, unsigned ux, 
     return pair_lerp(ux, uy, uz, x0, x1);
 }
 
-// Builds the z-pair atlas (see launch_make_zpairs).
+// The layouts of the moving volume, written straight into their arrays (blocks of 32 x 8 voxels of a plane).
 template <typename T>
-__global__ void k_make_zpairs(const T *__restrict__ in, int n0, int n1, int n2, int ph, int W,
-                              uint32_t *__restrict__ out) {
-    const long long plane = (long long)n0 * n1, n = plane * n2;
-    for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < n; o += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(o % n0);
-        const int y = (int)((o / n0) % n1);
-        const int z = (int)(o / plane);
-        const int z1 = min(z + 1, n2 - 1);
-        const long long src = (long long)y * n0 + x;
-        const uint32_t v = (uint32_t)in[plane * z + src] | ((uint32_t)in[plane * z1 + src] << (sizeof(T) == 1 ? 16 : 20));
-        const long long ox = (long long)(z / ph) * n0 + x, oy = (long long)(z % ph) * n1 + y;
-        out[oy * W + ox] = v;
-    }
+__global__ void __launch_bounds__(256)
+    k_make_zpairs(const T *__restrict__ in, int n0, int n1, int n2, int ph, cudaSurfaceObject_t out) {
+    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
+    if (x >= n0 || y >= n1) return;
+    const long long plane = (long long)n0 * n1, at = (long long)y * n0 + x;
+    const uint32_t a = in[plane * z + at], b = in[plane * min(z + 1, n2 - 1) + at];
+    surf2Dwrite(a | b << (sizeof(T) == 1 ? 16 : 20), out, ((z / ph) * n0 + x) * 4, (z % ph) * n1 + y);
 }
 
-// Builds the 2 x 2 (y, z) quads: out has dims (n0, n1, n2); element (x, y, z) holds v(x, y, z),
-// v(x, y + 1, z), v(x, y, z + 1), v(x, y + 1, z + 1), upper indices clamped to the last ones.
-template <typename T, typename QT>
-__global__ void k_make_quads(const T *__restrict__ in, int n0, int n1, int n2, QT *__restrict__ out) {
-    const long long plane = (long long)n0 * n1, n = plane * n2;
-    for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < n; o += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(o % n0);
-        const int y = (int)((o / n0) % n1);
-        const int z = (int)(o / plane);
-        const int y1 = min(y + 1, n1 - 1), z1 = min(z + 1, n2 - 1);
-        QT q;
-        q.x = in[plane * z + (long long)y * n0 + x];
-        q.y = in[plane * z + (long long)y1 * n0 + x];
-        q.z = in[plane * z1 + (long long)y * n0 + x];
-        q.w = in[plane * z1 + (long long)y1 * n0 + x];
-        out[o] = q;
-    }
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_make_quads(const T *__restrict__ in, int n0, int n1, int n2, cudaSurfaceObject_t out) {
+    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
+    if (x >= n0 || y >= n1) return;
+    const T *p0 = in + (long long)n0 * n1 * z + x, *p1 = in + (long long)n0 * n1 * min(z + 1, n2 - 1) + x;
+    const long long r0 = (long long)n0 * y, r1 = (long long)n0 * min(y + 1, n1 - 1);
+    const uint32_t a = p0[r0], b = p0[r1], c = p1[r0], d = p1[r1];
+    if (sizeof(T) == 1)
+        surf3Dwrite(a | b << 8 | c << 16 | d << 24, out, x * 4, y, z);
+    else
+        surf3Dwrite(make_ushort4((unsigned short)a, (unsigned short)b, (unsigned short)c, (unsigned short)d), out, x * 8, y, z);
 }
 
 // Builds the padded x-paired volume: out has dims (n0, n1 + 1, n2 + 1).
@@ -1485,17 +1512,6 @@ __global__ void k_sample_fill(int n0, long long R, uint32_t hseed, uint32_t thr,
     }
 }
 
-__global__ void k_fixed_hist(const uint8_t *__restrict__ fb, long long n, int bins, unsigned long long *__restrict__ out) {
-    __shared__ unsigned int h[256];
-    for (int c = threadIdx.x; c < 256; c += blockDim.x) h[c] = 0;
-    __syncthreads();
-    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x)
-        atomicAdd(&h[fb[x]], 1u);
-    __syncthreads();
-    for (int c = threadIdx.x; c < bins; c += blockDim.x)
-        if (h[c]) atomicAdd(out + c, (unsigned long long)h[c]);
-}
-
 cudaError_t launch_sample_count(int n0, long long R, uint32_t seed, uint32_t threshold, uint32_t *counts,
                                 cudaStream_t s) {
     k_sample_count<<<grid_for(R, 256), 256, 0, s>>>(n0, R, fmix32(seed), threshold, counts);
@@ -1508,29 +1524,24 @@ cudaError_t launch_sample_fill(int n0, long long R, uint32_t seed, uint32_t thre
     return cudaGetLastError();
 }
 
-cudaError_t launch_fixed_hist(const uint8_t *fbins, long long n, int bins, unsigned long long *out, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out, 0, (size_t)bins * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    long long g = (n + 255) / 256;
-    if (g > 1024) g = 1024;
-    k_fixed_hist<<<(int)(g < 1 ? 1 : g), 256, 0, s>>>(fbins, n, bins, out);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_f32_to_u16(const float *in, long long n, uint16_t *out, cudaStream_t s) {
     k_f32_to_u16<<<grid_for(n, 256), 256, 0, s>>>(in, n, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_clamp_depth(void *data, int dtype, int depth, long long n, cudaStream_t s) {
+// Blocks of 256 threads for n elements, eight a thread, at most eight blocks an SM.
+static int eight_grid(long long n) {
+    const long long g = (n + 2047) / 2048;
+    return (int)(g < 1 ? 1 : (g > 1216 ? 1216 : g));
+}
+
+cudaError_t launch_copy_clamp(const void *in, int dtype, int depth, long long n, void *out, cudaStream_t s) {
     const uint32_t vmax = (uint32_t)((1ull << depth) - 1ull);
-    if (dtype == 0) {
-        if (depth >= 8) return cudaSuccess;
-        k_clamp_depth<uint8_t><<<grid_for(n, 256), 256, 0, s>>>((uint8_t *)data, n, vmax);
-    } else {
-        if (depth >= 16) return cudaSuccess;
-        k_clamp_depth<uint16_t><<<grid_for(n, 256), 256, 0, s>>>((uint16_t *)data, n, vmax);
-    }
+    if (dtype == 0)
+        k_copy_clamp<uint8_t><<<eight_grid(n), 256, 0, s>>>((const uint8_t *)in, n, vmax, aligned8<uint8_t>(in), (uint8_t *)out);
+    else
+        k_copy_clamp<uint16_t><<<eight_grid(n), 256, 0, s>>>((const uint16_t *)in, n, vmax, aligned8<uint16_t>(in),
+                                                             (uint16_t *)out);
     return cudaGetLastError();
 }
 
@@ -1545,35 +1556,35 @@ cudaError_t launch_make_pairs(const void *mov, int dtype, const int nm[3], void 
     return cudaGetLastError();
 }
 
-cudaError_t launch_make_zpairs(const void *mov, int dtype, const int nm[3], int ph, int W, int H, uint32_t *out,
+cudaError_t launch_make_zpairs(const void *mov, int dtype, const int nm[3], int ph, cudaSurfaceObject_t out,
                                cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out, 0, (size_t)W * H * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
-    const long long n = (long long)nm[0] * nm[1] * nm[2];
+    const dim3 grid((nm[0] + 31) / 32, (nm[1] + 7) / 8, nm[2]), block(32, 8);
     if (dtype == 0)
-        k_make_zpairs<uint8_t><<<grid_for(n, 256), 256, 0, s>>>((const uint8_t *)mov, nm[0], nm[1], nm[2], ph, W, out);
+        k_make_zpairs<uint8_t><<<grid, block, 0, s>>>((const uint8_t *)mov, nm[0], nm[1], nm[2], ph, out);
     else
-        k_make_zpairs<uint16_t><<<grid_for(n, 256), 256, 0, s>>>((const uint16_t *)mov, nm[0], nm[1], nm[2], ph, W, out);
+        k_make_zpairs<uint16_t><<<grid, block, 0, s>>>((const uint16_t *)mov, nm[0], nm[1], nm[2], ph, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_make_quads(const void *mov, int dtype, const int nm[3], void *out, cudaStream_t s) {
-    const long long n = (long long)nm[0] * nm[1] * nm[2];
+cudaError_t launch_make_quads(const void *mov, int dtype, const int nm[3], cudaSurfaceObject_t out, cudaStream_t s) {
+    const dim3 grid((nm[0] + 31) / 32, (nm[1] + 7) / 8, nm[2]), block(32, 8);
     if (dtype == 0)
-        k_make_quads<uint8_t, uchar4><<<grid_for(n, 256), 256, 0, s>>>((const uint8_t *)mov, nm[0], nm[1], nm[2],
-                                                                        (uchar4 *)out);
+        k_make_quads<uint8_t><<<grid, block, 0, s>>>((const uint8_t *)mov, nm[0], nm[1], nm[2], out);
     else
-        k_make_quads<uint16_t, ushort4><<<grid_for(n, 256), 256, 0, s>>>((const uint16_t *)mov, nm[0], nm[1], nm[2],
-                                                                          (ushort4 *)out);
+        k_make_quads<uint16_t><<<grid, block, 0, s>>>((const uint16_t *)mov, nm[0], nm[1], nm[2], out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin_fixed(const void *data, int dtype, int depth, long long n, int bins, uint8_t *out,
-                             cudaStream_t s) {
+                             unsigned long long *counts, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(counts, 0, (size_t)bins * sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
     if (dtype == 0)
-        k_bin_fixed<uint8_t><<<grid_for(n, 256), 256, 0, s>>>((const uint8_t *)data, n, depth, bins, out);
+        k_bin_fixed<uint8_t><<<eight_grid(n), 256, 0, s>>>((const uint8_t *)data, n, depth, bins, aligned8<uint8_t>(data), out,
+                                                           counts);
     else
-        k_bin_fixed<uint16_t><<<grid_for(n, 256), 256, 0, s>>>((const uint16_t *)data, n, depth, bins, out);
+        k_bin_fixed<uint16_t><<<eight_grid(n), 256, 0, s>>>((const uint16_t *)data, n, depth, bins, aligned8<uint16_t>(data),
+                                                            out, counts);
     return cudaGetLastError();
 }
 

@@ -119,27 +119,26 @@ cudaError_t launch_sample_count(int n0, long long R, uint32_t seed, uint32_t thr
                                 cudaStream_t s);
 cudaError_t launch_sample_fill(int n0, long long R, uint32_t seed, uint32_t threshold, const uint8_t *fbins,
                                const uint32_t *row_ptr, uint16_t *cols, uint8_t *bins, cudaStream_t s);
-// Per-bin voxel counts of a binned fixed volume (bins u64, zeroed here).
-cudaError_t launch_fixed_hist(const uint8_t *fbins, long long n, int bins, unsigned long long *out, cudaStream_t s);
-
 // ---- launchers (all asynchronous on `s`) ---------------------------------
 cudaError_t launch_f32_to_u16(const float *in, long long n, uint16_t *out, cudaStream_t s);
-cudaError_t launch_clamp_depth(void *data, int dtype, int depth, long long n, cudaStream_t s);
+// out = min(in, 2^depth - 1)
+cudaError_t launch_copy_clamp(const void *in, int dtype, int depth, long long n, void *out, cudaStream_t s);
 // Padded x-paired moving volume, dims (n0, n1 + 1, n2 + 1).
 cudaError_t launch_make_pairs(const void *mov, int dtype, const int nm[3], void *out, cudaStream_t s);
 // Iteration cap of the 16-bit counter drain on the current device (default 2^16; test hook).
 cudaError_t set_drain_cap(int cap);
-// 2 x 2 (y, z) quads of the moving volume, dims (n0, n1, n2): element (x, y, z) holds
-// v(x, y, z), v(x, y + 1, z), v(x, y, z + 1), v(x, y + 1, z + 1), upper indices
-// clamped to the last ones (uchar4 for uint8, ushort4 for uint16 volumes).
-cudaError_t launch_make_quads(const void *mov, int dtype, const int nm[3], void *out, cudaStream_t s);
-// z-pair atlas of the moving volume (depth <= 12): out is a W x H uint32 image (zeroed here) in which
-// plane z occupies the nm[0] x nm[1] tile at ((z / ph) nm[0], (z % ph) nm[1]) and texel (x, y) of that
-// tile holds v(x, y, z) | v(x, y, min(z + 1, nm[2] - 1)) << 20 (<< 16 for uint8).
-cudaError_t launch_make_zpairs(const void *mov, int dtype, const int nm[3], int ph, int W, int H, uint32_t *out,
+// 2 x 2 (y, z) quads of the moving volume into a surface (dims nm): texel (x, y, z) holds
+// v(x, y, z), v(x, y + 1, z), v(x, y, z + 1), v(x, y + 1, z + 1), upper indices clamped to the last ones (the
+// bytes of one 32-bit texel for uint8 volumes, ushort4 for uint16 ones).
+cudaError_t launch_make_quads(const void *mov, int dtype, const int nm[3], cudaSurfaceObject_t out, cudaStream_t s);
+// z-pair atlas of the moving volume (depth <= 12) into a 2D surface of 32-bit texels: plane z
+// occupies the nm[0] x nm[1] tile at ((z / ph) nm[0], (z % ph) nm[1]) and texel (x, y) of that tile holds
+// v(x, y, z) | v(x, y, min(z + 1, nm[2] - 1)) << 20 (<< 16 for uint8).
+cudaError_t launch_make_zpairs(const void *mov, int dtype, const int nm[3], int ph, cudaSurfaceObject_t out,
                                cudaStream_t s);
+// Fixed bins (one byte a voxel) and the voxels per bin (bins u64, cleared here).
 cudaError_t launch_bin_fixed(const void *data, int dtype, int depth, long long n, int bins, uint8_t *out,
-                             cudaStream_t s);
+                             unsigned long long *counts, cudaStream_t s);
 cudaError_t launch_table(double *tab, float q, cudaStream_t s);
 // The hard-path kernel: persistent CTAs pull items from *d_ticket (reset by the caller); the parts of split
 // transforms are added to slot_hist + slot * slot_stride (bins^2 u32 each, zeroed by the caller).

@@ -183,3 +183,39 @@ def test_byte_volumes_in_paired_lanes(cuda_lib, variant, rows):
         for t in range(4):
             q16 = oracle.affine_q16(oracle.affine(prm[t], f.shape, (1, 1, 1), m.shape, (1, 1, 1)))
             np.testing.assert_array_equal(H[t], oracle.joint_hist(f, m, q16, 64)[0].astype(np.uint32))
+
+
+@pytest.mark.parametrize("dtype,depth,offset", [(np.uint8, 8, 3), (np.uint8, 5, 0), (np.uint16, 12, 1), (np.uint16, 16, 5),
+                                                (np.float32, 0, 1)])
+def test_layouts_from_unaligned_device_volumes(cuda_lib, dtype, depth, offset):
+    """Volumes used where they lie on the device: any element offset, voxel counts that leave a remainder of
+    the eight-wide loads, values above the declared depth; then one context walks through its layouts (one
+    pose, several, forced variants of every fetch) with the same histograms, also on another stream."""
+    import torch
+
+    rng = np.random.default_rng(86)
+    shape, mshape = (7, 9, 13), (11, 6, 17)
+    top = 2 if dtype == np.float32 else np.iinfo(dtype).max + 1
+    f, m = ((rng.random(s).astype(dtype) if dtype == np.float32 else rng.integers(0, top, s, dtype=dtype)) for s in (shape, mshape))
+    dev = []
+    for a in (f, m):
+        flat = torch.zeros(a.size + 16, dtype=getattr(torch, np.dtype(dtype).name), device="cuda")
+        flat[offset:offset + a.size] = torch.from_numpy(a).reshape(-1).cuda()
+        dev.append(flat[offset:offset + a.size].reshape(a.shape))
+    kw = dict(bins=32, fixed_depth=depth or None, moving_depth=depth or None)
+    ctx = cuda_lib.Context(dev[0], dev[1], **kw)
+    for d in dev:
+        d.zero_()  # the context has its own copy
+    prm = phantoms.random_transforms(400, seed=87, t_mm=2, r_deg=15, s_range=(0.9, 1.1))
+    mi_o, h_o, cnt_o = oracle.mi_eval(f, m, 32, prm, [1.0], fixed_depth=depth or None, moving_depth=depth or None, nthreads=8)
+    ok = cnt_o > 0
+    np.testing.assert_array_equal(ctx.fixed_bins(), oracle.bin_volume(f, 32, depth or None).reshape(shape))
+    for n in (1, 5, 400):
+        mi, _, cnt = ctx.eval(prm[:n], [1.0], with_entropies=True)
+        np.testing.assert_array_equal(cnt, cnt_o[:n])
+        g = ok[:n]
+        assert np.all(np.abs(mi[g] - mi_o[:n][g]) <= 1e-6 * np.maximum(np.abs(mi_o[:n][g]), h_o[:n][g][..., 2]) + 1e-12)
+    for v in (cuda_lib.HV_U32, cuda_lib.HV_U32_TEX, cuda_lib.HV_U32_QUAD) + ((cuda_lib.HV_U32_GATHER,) if 0 < depth <= 12 else ()):
+        other = cuda_lib.Context(f, m, hist_variant=v, **kw)
+        other.set_stream(torch.cuda.Stream())
+        np.testing.assert_array_equal(other.hist(transforms=prm[:4]), ctx.hist(transforms=prm[:4]))
