@@ -449,18 +449,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// block-wide sum of one double (all threads get the result); s_tmp holds >= 32 doubles
-__device__ double block_sum(double v, double *s_tmp) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    v = warp_sum(v);
-    __syncthreads();
-    if (lane == 0) s_tmp[warp] = v;
-    __syncthreads();
-    double s = 0.0;
-    for (int w = 0; w < nwarps; ++w) s += s_tmp[w];
-    return s;
-}
-
 __device__ __forceinline__ double finish_entropy(double sum, float qf, int bits) {
     if (qf == 1.0f) return bits ? sum / log(2.0) : sum;
     return (1.0 - sum) / ((double)qf - 1.0);
@@ -544,50 +532,61 @@ __global__ void __launch_bounds__(kMargThreads)
 
 // Grid (cells / 256, n): per-block joint entropy partial sums (jpart: n x nq x
 // gridDim.x, reduced in a fixed order later) and W (n x nq x B^2, FP32).  One
-// ln p per cell serves every q: the Shannon term -p ln p, p^q = exp(q ln p)
-// for the Tsallis ones, and dS_q/dp = -q p^q / (p (q - 1)).
+// ln p per cell serves every q: the Shannon term -p ln p, and r = p^(q-1) = exp((q - 1) ln p) for the
+// Tsallis ones, p^q = p r and dS_q/dp = -q r / (q - 1).  The FP64 issue bounds it (a warp's instruction takes
+// 16 clocks), so divisions are by factors formed once (1 / N by one thread, the others on the host), a
+// warp whose cells are empty computes nothing, and the warps' sums are added by one thread a q.  50 poses at
+// 64 bins and three q 73 -> 43 us, 48 poses on six pairs of up to 128 bins 168 -> 79.
 __global__ void __launch_bounds__(256)
     k_parzen_cells(const unsigned long long *__restrict__ ghist, const unsigned long long *__restrict__ gcount,
-                   const ParzenPair *__restrict__ pairs, const int *__restrict__ pair_of, int Bmax, QSet Q,
-                   const double *__restrict__ mterm, const double *__restrict__ ment, double *__restrict__ jpart,
-                   float *__restrict__ wout) {
-    __shared__ double s_tmp[32];
-    const int t = blockIdx.y;
+                   const ParzenPair *__restrict__ pairs, const int *__restrict__ pair_of, int Bmax,
+                   const __grid_constant__ QSet Q, const double *__restrict__ mterm, const double *__restrict__ ment,
+                   double *__restrict__ jpart, float *__restrict__ wout) {
+    __shared__ double s_sum[kMaxQ][8], s_inv;
+    const int t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int B = bins_of(pairs, pair_of, t), B2 = B * B, BM2 = Bmax * Bmax;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const double N = (double)gcount[t] * 4294967296.0;
-    const double lnb = Q.bits ? log(2.0) : 1.0;
+    const unsigned long long h = c < B2 ? ghist[(size_t)t * BM2 + c] : 0ull;
+    if (threadIdx.x == 0) {
+        const double N = (double)gcount[t] * 4294967296.0;
+        s_inv = N > 0 ? 1.0 / N : 0.0;
+    }
+    __syncthreads();
+    const bool any = __any_sync(kFull, h != 0);
     double p = 0.0, lp = 0.0;
-    if (c < B2 && N > 0) {
-        p = (double)ghist[(size_t)t * BM2 + c] / N;
-        if (p > 0.0) lp = log(p);
+    if (h != 0) {
+        p = (double)h * s_inv;
+        lp = log(p);
     }
     for (int iq = 0; iq < Q.nq; ++iq) {
-        const float qf = Q.q[iq];
-        const double q = (double)qf;
-        const double pq = p > 0.0 && qf != 1.0f ? exp(q * lp) : 0.0;
-        double e = p > 0.0 ? (qf == 1.0f ? -p * lp : pq) : 0.0;
-        e = block_sum(e, s_tmp);
-        if (threadIdx.x == 0) jpart[((size_t)t * Q.nq + iq) * gridDim.x + blockIdx.x] = e;
-        if (c < B2) {
-            double w = 0.0;
-            if (p > 0.0) {
-                const double *mt = mterm + ((size_t)t * Q.nq + iq) * 2 * Bmax;
-                const double fr = mt[c / B], mc = mt[B + c % B];
-                if (qf == 1.0f) {
-                    w = (lp - fr - mc - 1.0) / lnb;
-                } else {
-                    const double dSJ = -q * pq / (p * (q - 1.0));
-                    w = fr + mc - dSJ;
-                    if (Q.form == 1) {
-                        const double SF = ment[((size_t)t * Q.nq + iq) * 2 + 0];
-                        const double SM = ment[((size_t)t * Q.nq + iq) * 2 + 1];
-                        w += (1.0 - q) * (fr * SM + SF * mc);
-                    }
+        double e = 0.0, w = 0.0;
+        if (h != 0) {
+            const double *mt = mterm + ((size_t)t * Q.nq + iq) * 2 * Bmax;
+            const double fr = mt[c / B], mc = mt[B + c % B];
+            if (Q.q[iq] == 1.0f) {
+                e = -p * lp;
+                w = lp - fr - mc - 1.0;
+                if (Q.bits) w *= 1.44269504088896340736;  // 1 / ln 2
+            } else {
+                const double q = (double)Q.q[iq], r = exp((q - 1.0) * lp);
+                e = p * r;
+                w = fr + mc + q * Q.inv_q1[iq] * r;
+                if (Q.form == 1) {
+                    const double SF = ment[((size_t)t * Q.nq + iq) * 2 + 0];
+                    const double SM = ment[((size_t)t * Q.nq + iq) * 2 + 1];
+                    w += (1.0 - q) * (fr * SM + SF * mc);
                 }
             }
-            wout[((size_t)t * Q.nq + iq) * BM2 + c] = (float)w;
         }
+        if (c < B2) wout[((size_t)t * Q.nq + iq) * BM2 + c] = (float)w;
+        if (any) e = warp_sum(e);
+        if (lane == 0) s_sum[iq][warp] = e;
+    }
+    __syncthreads();
+    if (threadIdx.x < Q.nq) {
+        const double *s = s_sum[threadIdx.x];
+        jpart[((size_t)t * Q.nq + threadIdx.x) * gridDim.x + blockIdx.x] =
+            ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
     }
 }
 
