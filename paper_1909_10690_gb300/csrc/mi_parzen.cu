@@ -233,7 +233,6 @@ __device__ __forceinline__ void bspline_dw(float t, float d[4]) {
 // copies, goes to the global histogram.
 constexpr int kParzenMaxVox = 65536;  // also the longest fixed row (MI_MAX_PARZEN_NX)
 constexpr int kParzenBankSkew = 7;    // row stride of the forward's shared histogram, mod 32
-constexpr int kParzenRowsPerStep = 1;  // rows a warp of the forward works on at a time
 
 // Row stride of the shared tables: the least SB >= B + 1 with SB = kParzenBankSkew (mod 32).
 __host__ __device__ inline int parzen_stride(int B) { return B + 1 + ((kParzenBankSkew - (B + 1)) % 32 + 32) % 32; }
@@ -265,7 +264,7 @@ __host__ inline int parzen_fwd_copies(int B) { return parzen_fwd_copies_in(B, kP
 // the pair P0 passed by value, whose fields stay kernel parameters.  The shared memory (smem_words
 // words) is sized for the copies of the largest pair's bins; a transform of a pair with fewer bins
 // uses as many copies as fit there.
-template <int RPW, bool SAMPLED, bool MULTI>
+template <bool SAMPLED, bool MULTI>
 __global__ void __launch_bounds__(kParzenFwdThreads)
     k_parzen_hist(ParzenPair P0, const ParzenPair *__restrict__ pairs, const int *__restrict__ pair_of,
                   const long long *__restrict__ row_start, int n, const ParzenAffine *__restrict__ aff,
@@ -285,11 +284,6 @@ __global__ void __launch_bounds__(kParzenFwdThreads)
     const long long R0 = (long long)P0.nf[1] * P0.nf[2];  // rows per transform of a single pair
     const long long c0 = (long long)blockIdx.x * rows_per_cta;
     const long long c1 = c0 + rows_per_cta < total_rows ? c0 + rows_per_cta : total_rows;
-    // a warp works on RPW rows at a time, G = 32 / RPW neighbouring voxels of each: the lanes that
-    // add to one cell at once are then at most the G of a row (neighbouring voxels mostly share
-    // cells, and same-address shared atomics queue), while each row's gathers stay coalesced
-    constexpr int G = 32 / RPW;
-    const int sub = lane / G, pos = lane % G;
     // the transform owning row c0
     int t = 0;
     if (MULTI) {
@@ -320,7 +314,7 @@ __global__ void __launch_bounds__(kParzenFwdThreads)
         for (int c = threadIdx.x; c < NC * CP; c += blockDim.x) sh32[c] = 0u;
         if (threadIdx.x < 12) A[threadIdx.x] = aff[t].A[threadIdx.x];
         __syncthreads();
-        const long long DG0 = G * A[0], DG1 = G * A[4], DG2 = G * A[8];
+        const long long D0 = 32 * A[0], D1 = 32 * A[4], D2 = 32 * A[8];
         unsigned int cnt = 0;  // overlap voxels counted by this lane
         // one voxel at 32.32 index U with fixed bin bf: its four quantised B-spline weights
         auto add_voxel = [&](long long U0, long long U1, long long U2, int bf) {
@@ -372,26 +366,27 @@ __global__ void __launch_bounds__(kParzenFwdThreads)
                     }
                 }
             } else {
-                for (int s = 0; s < 32; s += RPW) {
-                    if (g + (long long)nwarps * s >= r1) break;  // warp-uniform: the rest of the group is past r1
-                    const int src = s + sub;
-                    const long long r = g + (long long)nwarps * src;
-                    int lo = __shfl_sync(kFull, mine.lo, src), hi = __shfl_sync(kFull, mine.hi, src);
-                    if (r >= r1) hi = lo - 1;
-                    const int len = hi - lo + 1 > 0 ? hi - lo + 1 : 0;
-                    if (pos == 0) cnt += (unsigned)len;
-                    const int nsteps = __reduce_max_sync(kFull, (unsigned)((len + G - 1) / G));
-                    long long U0 = __shfl_sync(kFull, mine.u0, src) + A[0] * pos;
-                    long long U1 = __shfl_sync(kFull, mine.u1, src) + A[4] * pos;
-                    long long U2 = __shfl_sync(kFull, mine.u2, src) + A[8] * pos;
-                    const uint8_t *__restrict__ frow = P.fbins + (size_t)(r < r1 ? r : r0) * nf0;
-                    for (int k = 0; k < nsteps; ++k) {
-                        const int i = lo + k * G + pos;
-                        if (i <= hi) add_voxel(U0, U1, U2, (int)__ldg(frow + i));
-                        U0 += DG0;
-                        U1 += DG1;
-                        U2 += DG2;
+                for (int s = 0; s < 32; ++s) {
+                    const long long r = g + (long long)nwarps * s;
+                    if (r >= r1) break;  // warp-uniform
+                    const int lo = __shfl_sync(kFull, mine.lo, s), hi = __shfl_sync(kFull, mine.hi, s);
+                    if (lo > hi) continue;
+                    const int len = hi - lo + 1;
+                    if (lane == 0) cnt += (unsigned)len;
+                    long long U0 = __shfl_sync(kFull, mine.u0, s) + A[0] * lane;
+                    long long U1 = __shfl_sync(kFull, mine.u1, s) + A[4] * lane;
+                    long long U2 = __shfl_sync(kFull, mine.u2, s) + A[8] * lane;
+                    const uint8_t *__restrict__ fp = P.fbins + (size_t)r * nf0 + lo + lane;
+                    // full steps carry no predicate, so two of them overlap (128 bins: 2645 -> 2448 us for 48
+                    // poses on six pairs, 1000 -> 984 for the 50 poses above)
+#pragma unroll 2
+                    for (int full = len >> 5; full > 0; --full, fp += 32) {
+                        add_voxel(U0, U1, U2, (int)__ldg(fp));
+                        U0 += D0;
+                        U1 += D1;
+                        U2 += D2;
                     }
+                    if (lane < (len & 31)) add_voxel(U0, U1, U2, (int)__ldg(fp));
                 }
             }
         }
@@ -735,7 +730,7 @@ struct AdjMoments {
 // The rows of one CTA's share: warp w of CTA b takes rows (b nwarps + w) + gridDim.x nwarps n, 32 of them
 // clipped at once (lane l: the l-th, with its j and k) and walked one by one, 32 voxels (or, under random
 // sampling, 32 sampled entries) a step.  tab: W with row stride rs and `cells` entries a q.
-template <int NQ, bool SAMPLED, int MODE>
+template <int NQ, bool SAMPLED, int MODE, int UNROLL>
 __device__ __forceinline__ void adj_rows(const ParzenPair &P, const long long *A, const float *__restrict__ tab, int rs,
                                          int cells, AdjMoments<NQ> &M) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -803,8 +798,9 @@ __device__ __forceinline__ void adj_rows(const ParzenPair &P, const long long *A
                 long long U0 = u0 + A[0] * lane, U1 = u1 + A[4] * lane, U2 = u2 + A[8] * lane;
                 const uint8_t *__restrict__ frow = P.fbins + (size_t)r * nf0;
                 int i = lo + lane;
-                // full steps carry no predicate, so two of them overlap: 1460 -> 1327 us of the 50 poses below
-#pragma unroll 2
+                // full steps carry no predicate, so UNROLL of them overlap: two 1460 -> 1327 us for the 50 poses
+                // below (three 1378), three 2946 -> 2614 for several pairs (two 2772)
+#pragma unroll UNROLL
                 for (int full = (hi - lo + 1) >> 5; full > 0; --full, i += 32) {
                     acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
                     U0 += D0;
@@ -823,7 +819,7 @@ __device__ __forceinline__ void adj_rows(const ParzenPair &P, const long long *A
 // over thousands of voxels, and another order moves the gradient by 1e-7): two values an instruction in the
 // trilinear stages, the moments and the slopes of paired q, and a row's j and k by shuffle from the lane
 // that clipped it instead of two 64-bit divisions a row.  50 poses, 192 x 192 x 128, 64 bins, three q: 1628
-// -> 1458 us (1327 with two full steps at a time); six pairs of up to 128 bins, 48 poses: 3266 -> 2921 (2772).  (With other sums allowed: quadratic
+// -> 1458 us (1327 with two full steps at a time); six pairs of up to 128 bins, 48 poses: 3266 -> 2921 (2614).  (With other sums allowed: quadratic
 // coefficients of s per cell instead of W, 160 KB of shared memory, 1533 and, with two rows a step, 2516.)
 template <int NQ, bool SAMPLED, bool MULTI, int TPB>
 __global__ void __launch_bounds__(TPB, 512 / TPB)
@@ -832,6 +828,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB)
                  double *__restrict__ mom) {
     // mom: n x nq_total x gridDim.x x 12 per-CTA partial moments (no atomics: fixed-order reduction later)
     // W of transform t is its slot of Bmax^2 entries per q (the first B^2 used, row stride B).
+    constexpr int kUnroll = NQ == 4 ? 1 : MULTI ? 3 : 2;  // (four q leave no registers for a second step)
     extern __shared__ __align__(16) float sw[];
     const int t = blockIdx.y;
     const ParzenPair P = MULTI ? pairs[pair_of[t]] : P0;
@@ -845,7 +842,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB)
     M.zero();
     if constexpr (TPB == 256) {
         __syncthreads();
-        adj_rows<NQ, SAMPLED, kWGlobal>(P, A, W, B, (int)BM2, M);
+        adj_rows<NQ, SAMPLED, kWGlobal, kUnroll>(P, A, W, B, (int)BM2, M);
     } else {
         // NQ x B x SB weights; the row stride SB >= B + 1 is 7 mod 32, so neighbouring voxels' cells, a bin
         // or two apart on either axis, are read from different banks
@@ -856,7 +853,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB)
             sw[apart ? q * cells + at : 2 * ((q / 2) * cells + at) + q % 2] = W[(size_t)q * BM2 + cc];
         }
         __syncthreads();
-        adj_rows<NQ, SAMPLED, kWShared>(P, A, sw, SB, cells, M);
+        adj_rows<NQ, SAMPLED, kWShared, kUnroll>(P, A, sw, SB, cells, M);
     }
     // warp reduction in FP32, then the warps in FP64 into global memory
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -1020,10 +1017,10 @@ cudaError_t launch_parzen_hist(const ParzenLaunch &L, const ParzenAffine *d_aff,
     const int copies = parzen_fwd_copies(L.Bmax);
     const size_t smem = parzen_fwd_smem(L.Bmax, copies);
     const bool multi = L.d_pair_of != nullptr;
-    const void *fn = multi ? (L.sampled ? (const void *)k_parzen_hist<kParzenRowsPerStep, true, true>
-                                        : (const void *)k_parzen_hist<kParzenRowsPerStep, false, true>)
-                           : (L.sampled ? (const void *)k_parzen_hist<kParzenRowsPerStep, true, false>
-                                        : (const void *)k_parzen_hist<kParzenRowsPerStep, false, false>);
+    const void *fn = multi ? (L.sampled ? (const void *)k_parzen_hist<true, true>
+                                        : (const void *)k_parzen_hist<false, true>)
+                           : (L.sampled ? (const void *)k_parzen_hist<true, false>
+                                        : (const void *)k_parzen_hist<false, false>);
     if ((e = allow_smem(fn, smem)) != cudaSuccess) return e;
     // rows per CTA: at most kParzenMaxVox voxels per copy, so that the 16-bit halves cannot overflow
     // (a row of nx voxels, or of at most nx sampled entries, is walked 32 lanes at a time, so copy i,
