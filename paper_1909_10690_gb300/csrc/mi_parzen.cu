@@ -798,16 +798,25 @@ __device__ __forceinline__ void adj_rows(const ParzenPair &P, const long long *A
                 long long U0 = u0 + A[0] * lane, U1 = u1 + A[4] * lane, U2 = u2 + A[8] * lane;
                 const uint8_t *__restrict__ frow = P.fbins + (size_t)r * nf0;
                 int i = lo + lane;
-                // full steps carry no predicate, so UNROLL of them overlap: two 1460 -> 1327 us for the 50 poses
-                // below (three 1378), three 2946 -> 2614 for several pairs (two 2772)
+                if constexpr (UNROLL == 1) {
+                    for (; i - lane <= hi; i += 32) {
+                        if (i <= hi) acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
+                        U0 += D0;
+                        U1 += D1;
+                        U2 += D2;
+                    }
+                } else {
+                    // full steps carry no predicate, so UNROLL of them overlap: two 1460 -> 1327 us for the 50
+                    // poses below (three 1378), three 2946 -> 2614 for several pairs (two 2772)
 #pragma unroll UNROLL
-                for (int full = (hi - lo + 1) >> 5; full > 0; --full, i += 32) {
-                    acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
-                    U0 += D0;
-                    U1 += D1;
-                    U2 += D2;
+                    for (int full = (hi - lo + 1) >> 5; full > 0; --full, i += 32) {
+                        acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
+                        U0 += D0;
+                        U1 += D1;
+                        U2 += D2;
+                    }
+                    if (i <= hi) acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
                 }
-                if (i <= hi) acc_voxel(U0, U1, U2, i, (int)__ldg(frow + i));
             }
             M.end_row(j, k);
         }
