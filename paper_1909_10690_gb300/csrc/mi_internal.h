@@ -103,9 +103,9 @@ struct Tile {
     int slabs;
 };
 constexpr int kMaxSlabs = 16;
-// Fixed rows each warp takes of a row block: the row-group walk's rows per step, else one.
+// Fixed rows each warp takes of a row block: the sampled walk's two, the row-group walk's rows per step, else one.
 __host__ __device__ inline int walk_rows_per_step(int fetch, int lpr_log2, bool sampled) {
-    return fetch >= FM_QUAD && lpr_log2 > 0 && !sampled ? 32 >> lpr_log2 : 1;
+    return sampled ? 2 : fetch >= FM_QUAD && lpr_log2 > 0 ? 32 >> lpr_log2 : 1;
 }
 
 // Shared memory needed by a hard-path CTA of `threads` threads for `bins` bins
