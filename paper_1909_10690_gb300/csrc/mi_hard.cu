@@ -673,11 +673,11 @@ __device__ __forceinline__ int sample_value(const PairDev &P, const float2 *zoff
 }
 
 // Random sampling: the sampled voxels of each clipped row [lo, hi]; U at an entry's x index i is
-// u_lo + st (i - lo), exact inside the interval.  A warp works on two neighbouring rows at once, 16 lanes
-// each: at 192 voxels and a quarter of them a row's entries are three steps of 16 where they were two of
-// 32, one broadcast serves two rows, and the lanes that clip the rows load where their entries lie, so that no
-// step waits for its row's offsets first.  Blocks are nwarps x 2 rows.  400 transforms, a quarter of 192 x 192 x 128
-// at 64 bins: 2687 -> 1982 us.
+// u_lo + st (i - lo), exact inside the interval.  A warp works on kSampledRows neighbouring rows at once: at
+// 192 voxels and a quarter of them a row's entries are six steps of 8 lanes where they were two of 32, one
+// broadcast serves all the rows, and the lanes that clip the rows load where their entries lie, so that no
+// step waits for its row's offsets first.  Blocks are nwarps x kSampledRows rows.  400 transforms, a quarter of
+// 192 x 192 x 128 at 64 bins: 2687 us one row at a time, 1982 with two rows, 1845 with four.
 template <typename PairT, int FM, class Hist>
 __device__ void accumulate_sampled(const PairDev &P, const int *q, const float2 *zoff, long long first_block,
                                    long long block_stride, long long n_end, Hist &H) {
@@ -686,17 +686,18 @@ __device__ void accumulate_sampled(const PairDev &P, const int *q, const float2 
     const long long R = (long long)nf1 * P.nf[2];
     const int st0 = q[0], st1 = q[4], st2 = q[8];
     const int bins = P.bins, mdepth = P.mdepth;
-    const int half = lane >> 4, pos = lane & 15;
-    for (long long n0b = 0;; n0b += 16) {
+    constexpr int G = kSampledRows, L = 32 / G;  // rows a step, lanes a row
+    const int sub = lane / L, pos = lane % L;
+    for (long long n0b = 0;; n0b += L) {
         if (first_block + n0b * block_stride >= n_end) break;
         RowClip mine;
         mine.lo = 0;
         mine.hi = -1;
         mine.u0 = mine.u1 = mine.u2 = 0;
         uint32_t k0 = 0, k1 = 0;  // the row's entries, none for an empty interval
-        const long long nl = first_block + (n0b + (lane >> 1)) * block_stride;
+        const long long nl = first_block + (n0b + lane / G) * block_stride;
         if (nl < n_end) {
-            const long long rl = (nl * nwarps + warp) * 2 + (lane & 1);
+            const long long rl = (nl * nwarps + warp) * G + lane % G;
             if (rl < R) {
                 k0 = __ldg(P.srow + rl);
                 k1 = __ldg(P.srow + rl + 1);
@@ -704,18 +705,18 @@ __device__ void accumulate_sampled(const PairDev &P, const int *q, const float2 
                 if (mine.lo > mine.hi) k1 = k0;
             }
         }
-        for (int s0 = 0; s0 < 32; s0 += 2) {
-            if (first_block + (n0b + (s0 >> 1)) * block_stride >= n_end) break;  // warp-uniform
-            const int s = s0 + half;
+        for (int s0 = 0; s0 < 32; s0 += G) {
+            if (first_block + (n0b + s0 / G) * block_stride >= n_end) break;  // warp-uniform
+            const int s = s0 + sub;
             const uint32_t e0 = __shfl_sync(kFull, k0, s), e1 = __shfl_sync(kFull, k1, s);
-            const int steps = (int)__reduce_max_sync(kFull, (e1 - e0 + 15) >> 4);
+            const int steps = (int)__reduce_max_sync(kFull, (e1 - e0 + L - 1) / L);
             if (steps == 0) continue;
             const int lo = __shfl_sync(kFull, mine.lo, s), hi = __shfl_sync(kFull, mine.hi, s);
             const unsigned ub0 = (unsigned)__shfl_sync(kFull, mine.u0, s), ub1 = (unsigned)__shfl_sync(kFull, mine.u1, s),
                            ub2 = (unsigned)__shfl_sync(kFull, mine.u2, s);
             uint32_t k = e0 + pos;
 #pragma unroll 2
-            for (int step = 0; step < steps; ++step, k += 16) {
+            for (int step = 0; step < steps; ++step, k += L) {
                 int i = -1, bf = 0, bm = 0;
                 if (k < e1) {
                     i = (int)__ldg(P.scol + k);

@@ -103,9 +103,10 @@ struct Tile {
     int slabs;
 };
 constexpr int kMaxSlabs = 16;
-// Fixed rows each warp takes of a row block: the sampled walk's two, the row-group walk's rows per step, else one.
+// Fixed rows each warp takes of a row block: the sampled walk's, the row-group walk's rows per step, else one.
+constexpr int kSampledRows = 4;
 __host__ __device__ inline int walk_rows_per_step(int fetch, int lpr_log2, bool sampled) {
-    return sampled ? 2 : fetch >= FM_QUAD && lpr_log2 > 0 ? 32 >> lpr_log2 : 1;
+    return sampled ? kSampledRows : fetch >= FM_QUAD && lpr_log2 > 0 ? 32 >> lpr_log2 : 1;
 }
 
 // Shared memory needed by a hard-path CTA of `threads` threads for `bins` bins
