@@ -45,10 +45,10 @@ DESIGN_OPS_PER_VOXT = 50
 # kernel source and the selected configuration are the ones measured: DRAM bytes of one full launch
 # (4096 transforms), and from a one-wave capture the issue and L1TEX utilisation and the
 # shared-memory wavefronts per shared atomic instruction.
-K_BATCHED_NCU = {"source_sha16": "a052ba2f01e56eb8", "config": [10, 2, 4],
-                 "dram_bytes_per_launch": 181408323840 + 61779200, "issue_active": 0.815,
-                 "l1tex_throughput": 0.695, "smem_wavefronts_per_atomic": 333607686 / 71766929,
-                 "smem_atomic_wavefronts_per_sm_cycle": 333607686 / 152 / 11992171.03,
+K_BATCHED_NCU = {"source_sha16": "3c94ed9a7ce37b1f", "config": [10, 4, 2],
+                 "dram_bytes_per_launch": 255594189568 + 10100736, "issue_active": 0.847,
+                 "l1tex_throughput": 0.844, "smem_wavefronts_per_atomic": 342238278 / 66419779,
+                 "smem_atomic_wavefronts_per_sm_cycle": 342238278 / 152 / 10787757.87,
                  "profile": "profiles/k_batched_rows_quad_256cubed_256bins.md"}
 # algorithmic FP32 operations per voxel x transform of the Parzen MI + gradient at 3 q values:
 # forward 31 (trilinear 14, bin coordinate 1, B-spline weights 12, 4 increments),
@@ -57,9 +57,9 @@ PARZEN_OPS_PER_VOXT = 120
 # Counters of the Parzen forward (k_parzen_hist) from one ncu capture of the 50-pose call (see profiles/),
 # reported while the kernel source is the one measured: shared-atomic instructions and wavefronts, SM
 # cycles elapsed per launch, and the DRAM bytes read and written by the forward and the adjoint
-K_PARZEN_NCU = {"source_sha16": "c75922c23d63e0fa", "atom_inst": 52167744, "atom_wavefronts": 242402137,
-                "sm_cycles_elapsed": 2143008.79, "time_ms": 1.0395,
-                "dram_bytes_per_call": 416319232 + 4436224 + 26225664,
+K_PARZEN_NCU = {"source_sha16": "010ce02ddcf24dcd", "atom_inst": 52167744, "atom_wavefronts": 242416278,
+                "sm_cycles_elapsed": 2050648.05, "time_ms": 0.9954,
+                "dram_bytes_per_call": 416288512 + 4498944 + 26232320,
                 "profile": "profiles/parzen_fwd_adj_192x192x128_64bins.md"}
 PARZEN_SHAPE = (128, 192, 192)
 PARZEN_SPACING = (1.0, 1.0, 1.2)

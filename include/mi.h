@@ -179,7 +179,7 @@ typedef struct {
                           (one partial step per 32 rows); 0 (default) = autotuned     */
     int tile_slabs;    /* batched kernel: slabs per sweep of the fixed rows (CTAs on
                           different transforms keep to neighbouring slabs): 0 (default)
-                          = 4, or 1..16                                                */
+                          = 2 (one pair, quad and gather variants) or 4, or 1..16      */
 } mi_options;
 
 /* Random voxel sampling (mi_options.sample_fraction in (0, 1), hard and

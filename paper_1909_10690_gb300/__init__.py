@@ -163,7 +163,7 @@ class Context:
     ``nparams`` is the count.
     tile_rows (0 = autotuned, or 1, 2, 4): adjacent fixed rows one warp step of
     the hard path covers, or 32: each warp walks its 32 clipped rows as one
-    stream of voxels; tile_slabs (0 = 4, or 1..16): slabs per sweep of the
+    stream of voxels; tile_slabs (0 = 2 or 4, or 1..16): slabs per sweep of the
     batched kernel.
     """
 

@@ -1123,7 +1123,12 @@ std::vector<Choice> candidates(mi_ctx *ctx, int bins, long long nvox_max) {
                 ch.threads = th;
                 ch.ctas = per_sm * ctx->sms;
                 ch.tile.lpr_log2 = lpr;
-                ch.tile.slabs = ctx->opt.tile_slabs > 0 ? ctx->opt.tile_slabs : 4;
+                // slabs a sweep: two for one pair with texel fetches (four rows a step; 1, 2, 3, 4 and 8 slabs:
+                // 149.5, 144.4, 147.0, 147.0 and 149.8 ms for 4096 transforms of 256^3 at 256 bins, 71.8, 69.2,
+                // 70.5, 71.3 and 73.2 for 2048 at 64), four otherwise (768 transforms of twelve pairs 11.8 ms
+                // a call against 12.1 with two)
+                const int slabs = hv_fetch(v) >= FM_QUAD && ctx->pairs.size() == 1 ? 2 : 4;
+                ch.tile.slabs = ctx->opt.tile_slabs > 0 ? ctx->opt.tile_slabs : slabs;
                 c.push_back(ch);
             }
         }
