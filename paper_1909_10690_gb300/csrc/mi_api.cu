@@ -388,6 +388,7 @@ struct mi_ctx {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     int last_launches = 0;
     bool timed = false;
+    bool fresh = true, building = false;  // tables / layouts queued and not yet waited for
 
     // floats per transform: 9 parameters, or the 12 of a general affine [M | t]
     int nparams() const { return opt.transform == MI_TRANSFORM_AFFINE ? 12 : 9; }
@@ -803,6 +804,7 @@ mi_status build_atlas(mi_ctx *ctx, Pair &P) {
 mi_status ensure_layouts(mi_ctx *ctx, unsigned modes) {
     std::vector<PairDev> pd;
     mi_status st;
+    ctx->building = true;  // until a wait for the stream
     for (auto &p : ctx->pairs) {
         if ((modes & (1u << FM_LDG | 1u << FM_TEX)) && (st = build_xpairs(ctx, *p, modes >> FM_TEX & 1u)) != MI_OK) return st;
         if ((modes >> FM_QUAD & 1u) && (st = build_quads(ctx, *p)) != MI_OK) return st;
@@ -1074,6 +1076,7 @@ mi_status deliver_all(mi_ctx *ctx, const char *base, const Result *res, int nres
         MI_CU(cudaMemcpyAsync(staging + lo, base + lo, hi - lo, cudaMemcpyDeviceToHost, ctx->stream), "copying results");
     }
     MI_CU(cudaStreamSynchronize(ctx->stream), "evaluation");
+    ctx->fresh = ctx->building = false;
     for (int i = 0; i < nres; ++i)
         if (on_host[i]) memcpy(res[i].dst, staging + res[i].at, res[i].bytes);
     return MI_OK;
@@ -1795,10 +1798,12 @@ const char *mi_last_error(const mi_ctx *ctx) { return ctx ? ctx->err.c_str() : g
 
 mi_status mi_set_stream(mi_ctx *ctx, void *stream) {
     if (!ctx) return MI_EINVAL;
-    {  // the pairs' tables and layouts were built on the stream so far
-        DeviceGuard guard(ctx->device);
-        MI_CU(cudaStreamSynchronize(ctx->stream), "switching streams");
-    }
+    // What was queued and not waited for: the pairs' tables on the context's own stream, and layouts of a call
+    // that failed after building them (on a stream the caller may have destroyed since).
+    DeviceGuard guard(ctx->device);
+    if (ctx->fresh) MI_CU(cudaStreamSynchronize(ctx->own_stream), "switching streams");
+    if (ctx->building) MI_CU(cudaDeviceSynchronize(), "switching streams");
+    ctx->fresh = ctx->building = false;
     ctx->stream = stream ? (cudaStream_t)stream : ctx->own_stream;
     ctx->graphs.clear();
     return MI_OK;
