@@ -1086,11 +1086,11 @@ mi_status deliver_all(mi_ctx *ctx, const char *base, const Result *res, int nres
 // Variant selection
 // ---------------------------------------------------------------------------
 
-bool variant_fits(int variant, int bins, int threads, long long nvox, int rows_words, int zmax) {
+bool variant_fits(int variant, int bins, long long nvox, int rows_words, int zmax) {
     const int kind = hv_kind(variant);
     const bool u16 = kind == HV_U16 || kind == HV_U16_MATCH;
     if (u16 && nvox > (long long)(kOvfSlots / 2) * kDrainT) return false;
-    return hard_smem_bytes(variant, bins, threads, rows_words, zmax) <= 227 * 1024;
+    return hard_smem_bytes(variant, bins, rows_words, zmax) <= 227 * 1024;
 }
 
 // Walks the tile shape may take for a variant: quad and gather fetches walk the warp's 32 rows as one
@@ -1117,7 +1117,7 @@ std::vector<Choice> candidates(mi_ctx *ctx, int bins, long long nvox_max) {
         if (hv_fetch(v) == FM_GATHER && !ctx->all_gather) continue;  // moving depth > 12 somewhere
         for (int th : {512, 1024}) {
             if (ctx->opt.block_threads > 0 && th != ctx->opt.block_threads) continue;
-            if (!variant_fits(v, bins, th, nvox_max, ctx->max_rows_words, ctx->max_zplanes)) continue;
+            if (!variant_fits(v, bins, nvox_max, ctx->max_rows_words, ctx->max_zplanes)) continue;
             const int per_sm = batched_ctas_per_sm(v, bins, th, ctx->max_rows_words, ctx->max_zplanes);
             if (per_sm < 1) continue;
             for (int lpr : tile_lpr(ctx, v)) {

@@ -557,11 +557,11 @@ struct SmemLayout {
 constexpr size_t kMaxCtaSmem = 227 * 1024;
 constexpr int kReduceWords = 1024;
 
-// zmax: planes of the largest moving volume (the gather variants keep one float2 offset per plane).
-__host__ __device__ inline SmemLayout smem_layout(int variant, int bins, int threads, int rows_words, int zmax) {
+// zmax: planes of the largest moving volume (gathers keep one float2 offset per plane).  The host, which sizes
+// the allocation, and the kernels, which address it, have to pass the same counter kind and fetch.
+__host__ __device__ inline SmemLayout smem_layout(int kind, int fetch, int bins, int rows_words, int zmax) {
     SmemLayout L;
     const size_t B2 = (size_t)bins * bins;
-    const int kind = hv_kind(variant);
     const bool u16 = kind == HV_U16 || kind == HV_U16_MATCH;
     const size_t S = (size_t)bins + 1, H = ((size_t)bins + 1) / 2;
     size_t o = 0;
@@ -586,12 +586,11 @@ __host__ __device__ inline SmemLayout smem_layout(int variant, int bins, int thr
     L.red = o;
     o += (size_t)(3 * 32 + 3 * kMaxQ + 1) * 8;
     L.zoff = o;
-    if (hv_fetch(variant) == FM_GATHER) o += (size_t)zmax * 8;
+    if (fetch == FM_GATHER) o += (size_t)zmax * 8;
     L.small = o;
     L.has_small = o + kReduceWords * 4 <= kMaxCtaSmem;
     if (L.has_small) o += kReduceWords * 4;
     L.total = o;
-    (void)threads;
     return L;
 }
 
@@ -1390,7 +1389,7 @@ __global__ void __launch_bounds__(1024, 1)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_item, s_slab;
     __shared__ int q[12];
-    const SmemLayout L = smem_layout(HV, max_bins, blockDim.x, rows_words, zmax);
+    const SmemLayout L = smem_layout(HV, FM, max_bins, rows_words, zmax);
     float2 *s_zoff = (float2 *)(smem + L.zoff);
     const int nwarps = blockDim.x >> 5;
     const int slabs = tile.slabs;
@@ -1503,8 +1502,8 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 }  // namespace
 
-size_t hard_smem_bytes(int variant, int bins, int threads, int rows_words, int zmax) {
-    return smem_layout(variant, bins, threads, rows_words, zmax).total;
+size_t hard_smem_bytes(int variant, int bins, int rows_words, int zmax) {
+    return smem_layout(hv_kind(variant), hv_fetch(variant), bins, rows_words, zmax).total;
 }
 
 // MurmurHash3's 32-bit finalizer: xor-shift 16, multiply 0x85ebca6b, xor-shift 13, multiply 0xc2b2ae35,
@@ -1666,7 +1665,7 @@ static const void *batched_fn(int variant) {
 }
 
 int batched_ctas_per_sm(int variant, int max_bins, int threads, int rows_words, int zmax) {
-    const size_t smem = smem_layout(variant, max_bins, threads, rows_words, zmax).total;
+    const size_t smem = hard_smem_bytes(variant, max_bins, rows_words, zmax);
     const void *fn = batched_fn(variant);
     if (!fn) return 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
@@ -1679,7 +1678,7 @@ cudaError_t launch_batched(const PairDev *d_pairs, const int32_t *d_aff, const I
                            int *d_ticket, int max_bins, int rows_words, int zmax, int variant, int threads, int ctas,
                            Tile tile, const QSet &Q, const Outputs &O, uint32_t *slot_hist, long long slot_stride,
                            cudaStream_t s) {
-    const size_t smem = smem_layout(variant, max_bins, threads, rows_words, zmax).total;
+    const size_t smem = hard_smem_bytes(variant, max_bins, rows_words, zmax);
     const void *fn = batched_fn(variant);
     if (!fn) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1800,7 +1799,7 @@ __global__ void __launch_bounds__(1024, 1)
     k_hist_raw(RawPair P, Q12 A, const __grid_constant__ QSet Q, NoallocScratch *__restrict__ D) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int B = P.bins;
-    const SmemLayout L = smem_layout(HV, B, blockDim.x, 0, 0);
+    const SmemLayout L = smem_layout(HV, FM_LDG, B, 0, 0);
     __shared__ int q[12];
     if (threadIdx.x < 12) q[threadIdx.x] = A.q[threadIdx.x];
     auto H = make_hist<HV>(smem, L, B, D->flags);
@@ -1845,7 +1844,7 @@ cudaError_t launch_noalloc_eval(const void *fix, int fdtype, int fdepth, const v
     const long long rows = (long long)nf[1] * nf[2], all = (rows + 31) / 32;  // a row a warp at least
     const int ctas = (int)(all < sms ? all : sms);
     const bool u32 = bins <= kRawU32Bins;
-    const size_t smem = smem_layout(u32 ? HV_U32 : HV_U16, bins, threads, 0, 0).total;
+    const size_t smem = smem_layout(u32 ? HV_U32 : HV_U16, FM_LDG, bins, 0, 0).total;
     cudaError_t e = cudaMemsetAsync(d, 0, offsetof(NoallocScratch, hist) + (size_t)bins * bins * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
 #define MI_RAW_H(FT, MT, HV)                                                                \

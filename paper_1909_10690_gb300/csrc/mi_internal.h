@@ -109,10 +109,10 @@ __host__ __device__ inline int walk_rows_per_step(int fetch, int lpr_log2, bool 
     return sampled ? kSampledRows : fetch >= FM_QUAD && lpr_log2 > 0 ? 32 >> lpr_log2 : 1;
 }
 
-// Shared memory needed by a hard-path CTA of `threads` threads for `bins` bins
+// Shared memory needed by a hard-path CTA for `bins` bins
 // (rows_words: words of the row-bound layout, used by HV_ROWS*).
 // (zmax: moving planes of the largest pair, for the gather variants' per-plane offsets.)
-size_t hard_smem_bytes(int variant, int bins, int threads, int rows_words, int zmax);
+size_t hard_smem_bytes(int variant, int bins, int rows_words, int zmax);
 // Random voxel sampling: voxel x takes part iff fmix32(x ^ fmix32(seed)) < threshold.
 // Per fixed row, the number of sampled voxels (counts: R entries), then the lists themselves
 // (row_ptr: the exclusive prefix sums, R + 1 entries; cols / bins: row_ptr[R] entries).
