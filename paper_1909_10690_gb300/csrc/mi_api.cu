@@ -1090,7 +1090,7 @@ bool variant_fits(int variant, int bins, long long nvox, int rows_words, int zma
     const int kind = hv_kind(variant);
     const bool u16 = kind == HV_U16 || kind == HV_U16_MATCH;
     if (u16 && nvox > (long long)(kOvfSlots / 2) * kDrainT) return false;
-    return hard_smem_bytes(variant, bins, rows_words, zmax) <= 227 * 1024;
+    return hard_smem_bytes(variant, bins, rows_words, zmax) <= kMaxCtaSmem;
 }
 
 // Walks the tile shape may take for a variant: quad and gather fetches walk the warp's 32 rows as one

@@ -554,7 +554,6 @@ struct SmemLayout {
     size_t hist, okey, ocnt, bmap, rinfo, rows, cols, red, zoff, small, total;
     bool has_small;  // the count table of reduce_entropies fits
 };
-constexpr size_t kMaxCtaSmem = 227 * 1024;
 constexpr int kReduceWords = 1024;
 
 // zmax: planes of the largest moving volume (gathers keep one float2 offset per plane).  The host, which sizes
@@ -1389,6 +1388,7 @@ __global__ void __launch_bounds__(1024, 1)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_item, s_slab;
     __shared__ int q[12];
+    static_assert(sizeof s_item + sizeof s_slab + sizeof q <= kStaticSmem, "kMaxCtaSmem leaves room for these");
     const SmemLayout L = smem_layout(HV, FM, max_bins, rows_words, zmax);
     float2 *s_zoff = (float2 *)(smem + L.zoff);
     const int nwarps = blockDim.x >> 5;
@@ -1668,9 +1668,12 @@ int batched_ctas_per_sm(int variant, int max_bins, int threads, int rows_words, 
     const size_t smem = hard_smem_bytes(variant, max_bins, rows_words, zmax);
     const void *fn = batched_fn(variant);
     if (!fn) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) return 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) {
+        cudaGetLastError();  // the answer is "none": the next launch's check must not find this error
+        return 0;
+    }
     return nb;
 }
 

@@ -109,6 +109,10 @@ __host__ __device__ inline int walk_rows_per_step(int fetch, int lpr_log2, bool 
     return sampled ? kSampledRows : fetch >= FM_QUAD && lpr_log2 > 0 ? 32 >> lpr_log2 : 1;
 }
 
+// Dynamic shared memory a hard-path CTA may ask for: the 227 KB a CTA can have hold its static variables too
+// (k_batched: the item, the slab and the transform, 56 bytes before the dynamic part's alignment).
+constexpr size_t kStaticSmem = 64;
+constexpr size_t kMaxCtaSmem = 227 * 1024 - kStaticSmem;
 // Shared memory needed by a hard-path CTA for `bins` bins
 // (rows_words: words of the row-bound layout, used by HV_ROWS*).
 // (zmax: moving planes of the largest pair, for the gather variants' per-plane offsets.)
