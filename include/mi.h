@@ -241,8 +241,10 @@ int mi_transform_size(const mi_ctx *ctx);
 const char *mi_last_error(const mi_ctx *ctx);
 
 /* Orders all later work of ctx on the CUDA stream `stream` (a cudaStream_t of
- * the context's device; NULL = back to the context's own stream).  CUDA-graph
- * replay is skipped on the legacy default stream, which cannot be captured. */
+ * the context's device; NULL = back to the context's own stream): device
+ * inputs are read and device outputs written in that stream's order, and no
+ * other stream is waited for.  CUDA-graph replay is skipped on the legacy
+ * default stream, which cannot be captured. */
 mi_status mi_set_stream(mi_ctx *ctx, void *stream);
 
 /*

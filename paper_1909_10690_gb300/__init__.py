@@ -80,11 +80,55 @@ class _Arg:
 
 def _wait_for(*args):
     """Waits for the torch work that produces device inputs (and last used the memory of outputs allocated
-    beside them): a context works on a stream of its own, which nothing orders after torch's."""
-    for a in args:
-        if a.on_gpu:
-            _torch().cuda.current_stream(a.obj.device).synchronize()
+    beside them), on every device that holds one: a context works on a stream of its own, which nothing
+    orders after torch's."""
+    for dev in dict.fromkeys(a.obj.device for a in args if a.on_gpu):
+        _torch().cuda.current_stream(dev).synchronize()
+
+
+class _Order:
+    """How one call is ordered with torch's work on its device tensors.
+
+    On the context's own stream the host waits for torch's current stream (``wait``).  On a stream the
+    caller gave, the inputs are the caller's to order and nothing is waited for: conversions and outputs
+    are made on that stream, and an output is marked as used by the caller's current stream too, so that
+    its memory is not handed out again while work queued there still reads it.
+    """
+
+    def __init__(self, given, *inputs):
+        self._given = self._caller = self._ctx = None
+        gpu = [x for x in inputs if _is_torch(x) and x.is_cuda] if given is not None else []
+        if not gpu:
             return
+        cuda, dev = _torch().cuda, gpu[0].device
+        if not hasattr(given, "cuda_stream"):  # a raw handle
+            given = cuda.ExternalStream(given, device=dev)
+        if all(x.device == given.device for x in gpu):
+            self._given, self._caller = given, cuda.current_stream(dev)
+            self._ctx = cuda.stream(given)
+
+    def __enter__(self):
+        if self._ctx is not None:
+            self._ctx.__enter__()
+        return self
+
+    def __exit__(self, *exc):
+        if self._ctx is not None:
+            self._ctx.__exit__(*exc)
+
+    def wait(self, *args):
+        if self._given is None:
+            _wait_for(*args)
+
+    def out(self, shape, like, dtype):
+        """An output beside the input ``like``: a tensor on its device, or a numpy array."""
+        if not like.on_gpu:
+            return np.empty(shape, dtype=dtype)
+        torch = _torch()
+        t = torch.empty(shape, dtype=getattr(torch, np.dtype(dtype).name), device=like.obj.device)
+        if self._given is not None and self._caller.cuda_stream != self._given.cuda_stream:
+            t.record_stream(self._caller)
+        return t
 
 
 def _np_dtype(x):
@@ -136,13 +180,6 @@ def _options(kernel, tsallis_form, bits, hist_variant, path, use_graphs, autotun
     return o
 
 
-def _out(shape, like_gpu, dtype, device=None):
-    if like_gpu:
-        torch = _torch()
-        return torch.empty(shape, dtype=getattr(torch, np.dtype(dtype).name), device=device or "cuda")
-    return np.empty(shape, dtype=dtype)
-
-
 def _ptr(x):
     if x is None:
         return None
@@ -174,6 +211,7 @@ class Context:
                  sample_fraction=0.0, sample_seed=0, transform="params", tile_rows=0, tile_slabs=0):
         self._lib = load()
         self._h = ctypes.c_void_p()
+        self._given = None  # set_stream's stream
         self.kernel = kernel
         self.rotation, self.scale, self.transform = rotation, scale, transform
         opt = _options(kernel, tsallis_form, bits, hist_variant, path, use_graphs, autotune, device, block_threads,
@@ -227,87 +265,89 @@ class Context:
         raise MIError(st, self._lib.mi_last_error(self._h).decode())
 
     def set_stream(self, stream):
-        """Order later work on a CUDA stream (a torch.cuda.Stream, a raw handle, or None)."""
+        """Order later work on a CUDA stream (a torch.cuda.Stream, a raw handle, or None: back to
+        the context's own stream).
+
+        On a given stream the calls read device inputs and write device outputs in that stream's order
+        and wait for no other, so work queued elsewhere goes on beside them: inputs that another stream
+        produces need ``stream.wait_stream(other)`` first.  On its own stream a context waits for torch's
+        current stream before it reads a device input."""
         h = getattr(stream, "cuda_stream", stream)
         self._check(self._lib.mi_set_stream(self._h, ctypes.c_void_p(h) if h else None))
+        self._given = stream if h else None
 
     def eval(self, transforms, q=(1.0,), with_entropies=False, allow_empty=True):
         """MI (n x nq) for n transforms; with_entropies adds (H_F, H_M, H_FM) per q and the overlap counts
         (for a Parzen context the entropies are None: only the counts)."""
-        T = _Arg(transforms, np.float32)
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
-        n = int(np.prod(T.obj.shape) // self.nparams)
         nq = int(np.asarray(q).size)
-        gpu = T.on_gpu
-        dev = T.obj.device if gpu else None
-        mi = _out((n, nq), gpu, np.float64, dev)
-        h = _out((n, nq, 3), gpu, np.float64, dev) if with_entropies and self.kernel != "parzen" else None
-        cnt = _out((n,), gpu, np.int64, dev) if with_entropies else None
-        _wait_for(T, Q)
-        st = self._lib.mi_eval(self._h, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
+        with _Order(self._given, transforms) as order:
+            T = _Arg(transforms, np.float32)
+            n = int(np.prod(T.obj.shape) // self.nparams)
+            mi = order.out((n, nq), T, np.float64)
+            h = order.out((n, nq, 3), T, np.float64) if with_entropies and self.kernel != "parzen" else None
+            cnt = order.out((n,), T, np.int64) if with_entropies else None
+            order.wait(T)
+            st = self._lib.mi_eval(self._h, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
         self._check(st, allow_empty)
         return (mi, h, cnt) if with_entropies else mi
 
     def eval_q16(self, affines, q=(1.0,), with_entropies=False, allow_empty=True):
-        A = _Arg(affines, np.int32)
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
-        n = int(np.prod(A.obj.shape) // 12)
         nq = int(np.asarray(q).size)
-        gpu = A.on_gpu
-        dev = A.obj.device if gpu else None
-        mi = _out((n, nq), gpu, np.float64, dev)
-        h = _out((n, nq, 3), gpu, np.float64, dev) if with_entropies else None
-        cnt = _out((n,), gpu, np.int64, dev) if with_entropies else None
-        _wait_for(A, Q)
-        st = self._lib.mi_eval_q16(self._h, A.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
+        with _Order(self._given, affines) as order:
+            A = _Arg(affines, np.int32)
+            n = int(np.prod(A.obj.shape) // 12)
+            mi = order.out((n, nq), A, np.float64)
+            h = order.out((n, nq, 3), A, np.float64) if with_entropies else None
+            cnt = order.out((n,), A, np.int64) if with_entropies else None
+            order.wait(A)
+            st = self._lib.mi_eval_q16(self._h, A.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
         self._check(st, allow_empty)
         return (mi, h, cnt) if with_entropies else mi
 
     def batch_eval(self, pair_of_transform, transforms, q=(1.0,), with_entropies=False, allow_empty=True):
-        P = _Arg(pair_of_transform, np.int32)
-        T = _Arg(transforms, np.float32)
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
-        n = int(np.prod(T.obj.shape) // self.nparams)
         nq = int(np.asarray(q).size)
-        gpu = T.on_gpu
-        dev = T.obj.device if gpu else None
-        mi = _out((n, nq), gpu, np.float64, dev)
-        h = _out((n, nq, 3), gpu, np.float64, dev) if with_entropies else None
-        cnt = _out((n,), gpu, np.int64, dev) if with_entropies else None
-        _wait_for(P, T, Q)
-        st = self._lib.mi_batch_eval(self._h, P.ptr, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
+        with _Order(self._given, pair_of_transform, transforms) as order:
+            P = _Arg(pair_of_transform, np.int32)
+            T = _Arg(transforms, np.float32)
+            n = int(np.prod(T.obj.shape) // self.nparams)
+            mi = order.out((n, nq), T, np.float64)
+            h = order.out((n, nq, 3), T, np.float64) if with_entropies else None
+            cnt = order.out((n,), T, np.int64) if with_entropies else None
+            order.wait(P, T)
+            st = self._lib.mi_batch_eval(self._h, P.ptr, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(h), _ptr(cnt))
         self._check(st, allow_empty)
         return (mi, h, cnt) if with_entropies else mi
 
     def grad(self, transforms, q=(1.0,), allow_empty=False):
         """Parzen MI (n x nq) and dMI/dparam (n x nq x nparams)."""
-        T = _Arg(transforms, np.float32)
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
-        n = int(np.prod(T.obj.shape) // self.nparams)
         nq = int(np.asarray(q).size)
-        gpu = T.on_gpu
-        dev = T.obj.device if gpu else None
-        mi = _out((n, nq), gpu, np.float64, dev)
-        g = _out((n, nq, self.nparams), gpu, np.float64, dev)
-        _wait_for(T, Q)
-        st = self._lib.mi_grad(self._h, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(g))
+        with _Order(self._given, transforms) as order:
+            T = _Arg(transforms, np.float32)
+            n = int(np.prod(T.obj.shape) // self.nparams)
+            mi = order.out((n, nq), T, np.float64)
+            g = order.out((n, nq, self.nparams), T, np.float64)
+            order.wait(T)
+            st = self._lib.mi_grad(self._h, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(g))
         self._check(st, allow_empty)
         return mi, g
 
     def batch_grad(self, pair_of_transform, transforms, q=(1.0,), allow_empty=False):
         """Parzen MI (n x nq) and dMI/dparam (n x nq x nparams) over the pairs of a multi-pair Parzen
         context: transform t on pair pair_of_transform[t], one launch per kernel for all pairs."""
-        P = _Arg(pair_of_transform, np.int32)
-        T = _Arg(transforms, np.float32)
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
-        n = int(np.prod(T.obj.shape) // self.nparams)
         nq = int(np.asarray(q).size)
-        gpu = T.on_gpu
-        dev = T.obj.device if gpu else None
-        mi = _out((n, nq), gpu, np.float64, dev)
-        g = _out((n, nq, self.nparams), gpu, np.float64, dev)
-        _wait_for(P, T, Q)
-        st = self._lib.mi_batch_grad(self._h, P.ptr, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(g))
+        with _Order(self._given, pair_of_transform, transforms) as order:
+            P = _Arg(pair_of_transform, np.int32)
+            T = _Arg(transforms, np.float32)
+            n = int(np.prod(T.obj.shape) // self.nparams)
+            mi = order.out((n, nq), T, np.float64)
+            g = order.out((n, nq, self.nparams), T, np.float64)
+            order.wait(P, T)
+            st = self._lib.mi_batch_grad(self._h, P.ptr, T.ptr, n, Q.ptr, nq, _ptr(mi), _ptr(g))
         self._check(st, allow_empty)
         return mi, g
 
@@ -315,13 +355,14 @@ class Context:
         """Joint histograms (n x bins x bins uint32, row = fixed bin) -- test hook."""
         if (transforms is None) == (affines is None):
             raise ValueError("give exactly one of transforms and affines")
-        src = _Arg(transforms, np.float32) if transforms is not None else _Arg(affines, np.int32)
-        n = int(np.prod(src.obj.shape) // (self.nparams if transforms is not None else 12))
         B = self.bins[pair]
-        out = np.empty((n, B, B), dtype=np.uint32)
-        _wait_for(src)
-        st = self._lib.mi_hist(self._h, pair, src.ptr if transforms is not None else None,
-                               src.ptr if affines is not None else None, n, int(path), out.ctypes.data)
+        with _Order(self._given, transforms, affines) as order:
+            src = _Arg(transforms, np.float32) if transforms is not None else _Arg(affines, np.int32)
+            n = int(np.prod(src.obj.shape) // (self.nparams if transforms is not None else 12))
+            out = np.empty((n, B, B), dtype=np.uint32)
+            order.wait(src)
+            st = self._lib.mi_hist(self._h, pair, src.ptr if transforms is not None else None,
+                                   src.ptr if affines is not None else None, n, int(path), out.ctypes.data)
         self._check(st)
         return out
 
@@ -425,7 +466,9 @@ def mi_function():
     class MIFunction(torch.autograd.Function):
         @staticmethod
         def forward(fctx, theta, ctx, q):
-            mi, g = ctx.grad(theta.detach().to(torch.float32).contiguous(), q)
+            x = _Arg(theta, np.float32)
+            _wait_for(x)  # an operator of torch's current stream, whatever stream the context was given
+            mi, g = ctx.grad(x.obj, q)
             fctx.save_for_backward(g if _is_torch(g) else torch.from_numpy(g))
             mi = mi if _is_torch(mi) else torch.from_numpy(mi)
             return mi.to(theta.device)
