@@ -388,7 +388,9 @@ struct mi_ctx {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     int last_launches = 0;
     bool timed = false;
-    bool fresh = true, building = false;  // tables / layouts queued and not yet waited for
+    // queued and not yet waited for: the pairs' tables on the own stream (fresh), entropy tables and layouts
+    // on `stream` (building)
+    bool fresh = true, building = false;
 
     // floats per transform: 9 parameters, or the 12 of a general affine [M | t]
     int nparams() const { return opt.transform == MI_TRANSFORM_AFFINE ? 12 : 9; }
@@ -411,6 +413,13 @@ namespace {
         cudaError_t e__ = (call);                            \
         if (e__ != cudaSuccess) return ctx->cuda_fail(e__, what); \
     } while (0)
+
+// Waits for the context's stream, after which nothing of the context is pending.
+mi_status wait_stream(mi_ctx *ctx, const char *what) {
+    MI_CU(cudaStreamSynchronize(ctx->stream), what);
+    ctx->fresh = ctx->building = false;
+    return MI_OK;
+}
 
 // Per-call device guard: make the context's device current, restore on exit.
 struct DeviceGuard {
@@ -1001,6 +1010,7 @@ mi_status make_qset(mi_ctx *ctx, const float *qv, int nq, QSet &Q) {
             if (it == ctx->tables.end()) {
                 auto buf = std::make_unique<DevBuf>();
                 MI_CU(buf->ensure(sizeof(double) * kTab), "allocating an entropy table");
+                ctx->building = true;  // until a wait for the stream
                 MI_CU(launch_table(buf->as<double>(), qv[i], ctx->stream), "building an entropy table");
                 it = ctx->tables.emplace(fbits(qv[i]), std::move(buf)).first;
             }
@@ -1075,8 +1085,8 @@ mi_status deliver_all(mi_ctx *ctx, const char *base, const Result *res, int nres
         }
         MI_CU(cudaMemcpyAsync(staging + lo, base + lo, hi - lo, cudaMemcpyDeviceToHost, ctx->stream), "copying results");
     }
-    MI_CU(cudaStreamSynchronize(ctx->stream), "evaluation");
-    ctx->fresh = ctx->building = false;
+    mi_status st = wait_stream(ctx, "evaluation");
+    if (st != MI_OK) return st;
     for (int i = 0; i < nres; ++i)
         if (on_host[i]) memcpy(res[i].dst, staging + res[i].at, res[i].bytes);
     return MI_OK;
@@ -1783,6 +1793,7 @@ void mi_destroy(mi_ctx *ctx) {
     {
         DeviceGuard guard(ctx->device);
         if (ctx->own_stream) cudaStreamSynchronize(ctx->own_stream);
+        if (ctx->building) cudaDeviceSynchronize();  // on a stream the caller may have destroyed
         ctx->graphs.clear();
         ctx->tables.clear();
         ctx->pairs.clear();
@@ -1798,8 +1809,8 @@ const char *mi_last_error(const mi_ctx *ctx) { return ctx ? ctx->err.c_str() : g
 
 mi_status mi_set_stream(mi_ctx *ctx, void *stream) {
     if (!ctx) return MI_EINVAL;
-    // What was queued and not waited for: the pairs' tables on the context's own stream, and layouts of a call
-    // that failed after building them (on a stream the caller may have destroyed since).
+    // What was queued and not waited for: the pairs' tables on the context's own stream, and entropy tables and
+    // layouts of a call that failed after queueing them (on a stream the caller may have destroyed since).
     DeviceGuard guard(ctx->device);
     if (ctx->fresh) MI_CU(cudaStreamSynchronize(ctx->own_stream), "switching streams");
     if (ctx->building) MI_CU(cudaDeviceSynchronize(), "switching streams");
@@ -2006,8 +2017,7 @@ mi_status mi_fixed_bins(mi_ctx *ctx, int pair, uint8_t *out) {
     const void *src = ctx->opt.kernel == MI_PARZEN ? P.pfbins.p : P.fbins;
     mi_status st = deliver(ctx, out, src, (size_t)P.nvf);
     if (st != MI_OK) return st;
-    MI_CU(cudaStreamSynchronize(ctx->stream), "copying bins");
-    return MI_OK;
+    return wait_stream(ctx, "copying bins");
 }
 
 mi_status mi_resample(mi_ctx *ctx, int pair, const int32_t *affine, void *out) {
@@ -2037,8 +2047,7 @@ mi_status mi_resample(mi_ctx *ctx, int pair, const int32_t *affine, void *out) {
     MI_CU(launch_resample(ctx->d_pairs.as<PairDev>() + pair, host_pairdev(P), ctx->d_aff.as<int32_t>(), dst, ctx->stream),
           "resample kernel");
     if (dst != out) MI_CU(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, ctx->stream), "D2H");
-    MI_CU(cudaStreamSynchronize(ctx->stream), "resampling");
-    return MI_OK;
+    return wait_stream(ctx, "resampling");
 }
 
 mi_status mi_last_kernel_ms(mi_ctx *ctx, float *ms, int *launches) {
