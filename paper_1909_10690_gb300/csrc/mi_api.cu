@@ -1344,20 +1344,20 @@ void cache_store(const std::string &path, const std::string &key, const Choice &
     fclose(f);
 }
 
+// The choice where nothing is timed (a single candidate, or mi_options.autotune 0): plain shared atomics, 32-bit
+// counters where they fit, 1024 threads.
+Choice untuned_choice(const std::vector<Choice> &cands) {
+    Choice best = cands.front();
+    for (const Choice &c : cands)
+        if ((c.variant == HV_U32 || (c.variant == HV_U16 && best.variant != HV_U32)) && c.threads == 1024) best = c;
+    return best;
+}
+
 // Autotune: time every candidate on the first items of this call (up to three
 // waves, so that effects that build up across waves, such as CTAs drifting to
 // different parts of the volumes, show in the timing).
 mi_status autotune(mi_ctx *ctx, const int32_t *d_aff, const Item *d_items, int nitems, int *d_ticket, const QSet &Q,
                    const Outputs &O, Choice &best, const std::vector<Choice> &cands) {
-    if (cands.empty()) return ctx->fail(MI_EUNSUPPORTED, "no histogram variant fits this bin count and volume size");
-    if (cands.size() == 1 || !ctx->opt.autotune) {
-        best = cands.front();
-        // heuristic: plain shared atomics (32-bit counters where they fit), 1024 threads
-        for (const Choice &c : cands)
-            if ((c.variant == HV_U32 || (c.variant == HV_U16 && best.variant != HV_U32)) && c.threads == 1024) best = c;
-        if (best.variant < 0) best = cands.front();
-        return MI_OK;
-    }
     // Two stages: every candidate is timed on one wave of items (after a warm-up of a few items, which
     // loads its kernel), then the three fastest on three waves; time per item decides.
     cudaEvent_t e0, e1;
@@ -1455,8 +1455,11 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     } else if (plain) {
         ch = plain_choice(ctx, cands, n);
         ctx->tuned[key] = ch;
+    } else if (cands.size() == 1 || !ctx->opt.autotune) {
+        ch = untuned_choice(cands);
+        ctx->tuned[key] = ch;
     } else {
-        const std::string cpath = ctx->opt.autotune && cands.size() > 1 ? cache_path() : std::string();
+        const std::string cpath = cache_path();
         const std::string ckey = cpath.empty() ? std::string() : tune_key(ctx, bucket, nq);
         if (cpath.empty() || !cache_lookup(cpath, ckey, cands, ch)) {
             // tuning needs every candidate's layout, the affines and whole items on the device
