@@ -49,6 +49,14 @@
  * the context's stream (its own non-blocking stream unless mi_set_stream
  * names another) and every call returns once its results are in the caller's
  * buffers (the call synchronises that stream).
+ * Device memory beyond the volumes is taken when a call first needs it and
+ * kept: the layout of the moving volume that the chosen variant reads (2 to 8
+ * bytes a voxel; every candidate's on a call that is autotuned), so a lack of
+ * memory shows there (MI_ENOMEM) and not in mi_create; the call's scratch; on
+ * the plain path up to 64 MB of histograms; on the batched path a histogram
+ * (4 bins^2 bytes) for each transform that is split over CTAs, up to about
+ * twice the resident CTAs (80 MB at 256 bins), without which, where they find
+ * no room, the call keeps its transforms whole.
  *
  * Errors: every call returns an mi_status; mi_last_error gives a message.
  * A context is not thread-safe; distinct contexts are independent.
@@ -348,8 +356,8 @@ mi_status mi_selected_config(mi_ctx *ctx, int n, int out[5]);
 
 /* Test hook (failure handling): after `after` further successful device
  * allocations by the library in this process, the next one fails as if the
- * device were out of memory (the caller sees MI_ENOMEM), and the hook disarms
- * itself; after < 0 disarms it.  It lets callers check that every entry point
+ * device were out of memory (the caller sees MI_ENOMEM, unless the call can
+ * do without that memory), and the hook disarms itself; after < 0 disarms it.  It lets callers check that every entry point
  * fails cleanly and leaves its context usable.  Host-side only: no GPU fault
  * is raised. */
 void mi_fault_alloc(int after);

@@ -374,6 +374,7 @@ struct mi_ctx {
     DevBuf d_aff, d_in, d_work, d_part, d_dump;
     HostBuf h_in, h_read;
     std::vector<char> v_in, v_out;  // the same staging where no graph replays it, and the results'
+    size_t no_room = SIZE_MAX;      // least d_work of a call that had to keep its transforms whole for it
     std::vector<Choice> cands;      // the hard path's candidates (fixed by the pairs and options)
     // Parzen: the pairs' descriptors (device array), per-call pair indices and row offsets, scratch
     DevBuf p_pairs;
@@ -1489,10 +1490,11 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     if ((st = ensure_layouts(ctx, 1u << hv_fetch(ch.variant))) != MI_OK) return st;
     // The plain path sums every histogram in global memory, in chunks of at most 64 MB of them; the
     // batched path reduces whole transforms in place and splits the last ones, unless the caller asked
-    // for the batched path of a single pair by name or wants the histograms themselves.
+    // for the batched path of a single pair by name or wants the histograms themselves.  The split ones' histograms
+    // (up to about 2 P of them, P the resident CTAs: 80 MB at 256 bins, P = 152) are the only part of a batched
+    // call's memory that it can do without: where they find no room every transform stays whole.
     const size_t B2 = (size_t)ctx->max_bins * ctx->max_bins;
-    const PlanMode mode = plain ? kPlanSlots
-                          : !R.dump && (multi || R.path == MI_PATH_AUTO) ? kPlanTail : kPlanWhole;
+    PlanMode mode = plain ? kPlanSlots : !R.dump && (multi || R.path == MI_PATH_AUTO) ? kPlanTail : kPlanWhole;
     const int chunk = plain ? (int)std::min<size_t>(4096, std::max<size_t>(1, (64u << 20) / (B2 * 4))) : n;
     struct Range {
         int t0, m;
@@ -1500,25 +1502,46 @@ mi_status eval_core(mi_ctx *ctx, const EvalReq &R, const float *qv, int nq, doub
     };
     std::vector<Range> ranges;
     HardPlan plan;
-    size_t max_slots = 0;
-    for (int t0 = 0; t0 < n; t0 += chunk) {
-        Range r{t0, std::min(chunk, n - t0), plan.items.size(), 0, plan.slots.size(), 0};
-        plan_items(ctx, R.pair_of, t0, r.m, ch, mode, plan);
-        r.nitems = plan.items.size() - r.item0;
-        r.nslots = plan.slots.size() - r.slot0;
-        max_slots = std::max(max_slots, r.nslots);
-        ranges.push_back(r);
-    }
-    const size_t aff_bytes = align256((size_t)n * 48), items_at = aff_bytes,
-                 slots_at = items_at + align256(plan.items.size() * sizeof(Item)),
-                 in_bytes = slots_at + plan.slots.size() * sizeof(Slot);
-    const size_t hist_at = done_at + align256(max_slots * 4);
+    size_t max_slots, items_at, slots_at, in_bytes, hist_at;
     const bool own_hist = !(plain && R.dump);
-    const size_t work_bytes = hist_at + (own_hist ? max_slots * B2 * 4 : 0);
-    MI_CU(ctx->d_in.ensure(in_bytes), "allocating the call's inputs");
-    MI_CU(ctx->d_work.ensure(work_bytes), "allocating the workspace");
-    if (max_slots)
-        MI_CU(ctx->d_part.ensure(entropy_part_bytes((ctx->max_bins + 7) / 8, (int)max_slots)), "allocating partial sums");
+    auto make_plan = [&]() {
+        ranges.clear();
+        plan = HardPlan();
+        max_slots = 0;
+        for (int t0 = 0; t0 < n; t0 += chunk) {
+            Range r{t0, std::min(chunk, n - t0), plan.items.size(), 0, plan.slots.size(), 0};
+            plan_items(ctx, R.pair_of, t0, r.m, ch, mode, plan);
+            r.nitems = plan.items.size() - r.item0;
+            r.nslots = plan.slots.size() - r.slot0;
+            max_slots = std::max(max_slots, r.nslots);
+            ranges.push_back(r);
+        }
+        items_at = align256((size_t)n * 48);
+        slots_at = items_at + align256(plan.items.size() * sizeof(Item));
+        in_bytes = slots_at + plan.slots.size() * sizeof(Slot);
+        hist_at = done_at + align256(max_slots * 4);
+        return hist_at + (own_hist ? max_slots * B2 * 4 : 0);  // bytes of d_work
+    };
+    auto allocate = [&](size_t work_bytes) {
+        cudaError_t e = ctx->d_in.ensure(in_bytes);
+        if (e == cudaSuccess) e = ctx->d_work.ensure(work_bytes);
+        if (e == cudaSuccess && max_slots)
+            e = ctx->d_part.ensure(entropy_part_bytes((ctx->max_bins + 7) / 8, (int)max_slots));
+        return e;
+    };
+    size_t work_bytes = make_plan();
+    const bool split = mode == kPlanTail && max_slots > 0;
+    const bool refused = split && work_bytes >= ctx->no_room && work_bytes > ctx->d_work.cap;  // (by an earlier call)
+    cudaError_t room = refused ? cudaErrorMemoryAllocation : allocate(work_bytes);
+    if (room == cudaErrorMemoryAllocation && split) {
+        cudaGetLastError();
+        const size_t split_bytes = work_bytes;
+        mode = kPlanWhole;
+        work_bytes = make_plan();
+        room = allocate(work_bytes);
+        if (room == cudaSuccess) ctx->no_room = std::min(ctx->no_room, split_bytes);
+    }
+    MI_CU(room, "allocating the call's workspace");
     set_outputs();
     cudaStream_t s = ctx->stream;
     // A batched call is replayed as a CUDA graph, so its inputs go through pinned staging.  The plain path
