@@ -2086,19 +2086,24 @@ mi_status mi_last_kernel_ms(mi_ctx *ctx, float *ms, int *launches) {
     return MI_OK;
 }
 
-static const Choice *selected_choice(mi_ctx *ctx, int n) {
-    const int path = ctx->opt.path == MI_PATH_AUTO ? ((ctx->pairs.size() > 1 || n >= ctx->sms) ? MI_PATH_BATCHED : MI_PATH_PLAIN)
-                                                   : ctx->opt.path;
-    const int bucket = path == MI_PATH_BATCHED ? (n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0)) : plain_bucket(n);
-    auto it = ctx->tuned.find(std::make_tuple(path, path == MI_PATH_BATCHED ? -1 : 0, bucket));
-    return it == ctx->tuned.end() ? nullptr : &it->second;
+// The choice for calls of n transforms; variant -1 before a call that made it.  The plain path's follows from n
+// alone once one of its calls has been made, whatever that call's n.
+static Choice selected_choice(mi_ctx *ctx, int n) {
+    const bool batched = ctx->opt.path == MI_PATH_AUTO ? ctx->pairs.size() > 1 || n >= ctx->sms
+                                                       : ctx->opt.path == MI_PATH_BATCHED;
+    if (batched) {
+        auto it = ctx->tuned.find(std::make_tuple((int)MI_PATH_BATCHED, -1, n >= 4 * ctx->sms ? 2 : (n >= ctx->sms ? 1 : 0)));
+        return it == ctx->tuned.end() ? Choice() : it->second;
+    }
+    for (int bucket : {0, 1})
+        if (ctx->tuned.count(std::make_tuple((int)MI_PATH_PLAIN, 0, bucket))) return plain_choice(ctx, ctx->cands, n);
+    return Choice();
 }
 
 int mi_selected_variant(mi_ctx *ctx, int pair, int n) {
     if (!ctx) return -1;
     (void)pair;
-    const Choice *c = selected_choice(ctx, n);
-    return c ? c->variant : -1;
+    return selected_choice(ctx, n).variant;
 }
 
 void mi_autotune_cache(const char *path) {
@@ -2109,16 +2114,16 @@ void mi_autotune_cache(const char *path) {
 
 mi_status mi_selected_config(mi_ctx *ctx, int n, int out[5]) {
     if (!ctx || !out) return MI_EINVAL;
-    const Choice *c = selected_choice(ctx, n);
-    if (!c) {
+    const Choice c = selected_choice(ctx, n);
+    if (c.variant < 0) {
         for (int i = 0; i < 5; ++i) out[i] = -1;
         return MI_OK;
     }
-    out[0] = c->variant;
-    out[1] = c->threads;
-    out[2] = c->ctas;
-    out[3] = c->tile.lpr_log2 == 0 ? 32 : 32 >> c->tile.lpr_log2;
-    out[4] = c->tile.slabs;
+    out[0] = c.variant;
+    out[1] = c.threads;
+    out[2] = c.ctas;
+    out[3] = c.tile.lpr_log2 == 0 ? 32 : 32 >> c.tile.lpr_log2;
+    out[4] = c.tile.slabs;
     return MI_OK;
 }
 
