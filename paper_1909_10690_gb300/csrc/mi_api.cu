@@ -381,7 +381,7 @@ struct mi_ctx {
     int p_bmax = 0, p_nxmax = 0;
     // (p_in: affines, Jacobians and, for several pairs, pair indices and row offsets; p_out: overlap counts,
     // MI, gradients)
-    DevBuf p_in, p_out, p_hist, p_marg, p_ment, p_mterm, p_jsum, p_w, p_mom;
+    DevBuf p_in, p_out, p_hist, p_ment, p_mterm, p_jsum, p_w, p_mom;
     // autotune and graph caches
     std::map<std::tuple<int, int, int>, Choice> tuned;  // (path, pair-or--1, n bucket)
     std::map<std::string, std::unique_ptr<GraphEntry>> graphs;
@@ -1710,7 +1710,6 @@ mi_status parzen_core(mi_ctx *ctx, const std::vector<float> &prm, int n, const f
     const size_t mi_at = (size_t)n * 8, grad_at = mi_at + (size_t)n * nq * 8;
     MI_CU(ctx->p_out.ensure(grad_at + (size_t)n * nq * np * 8), "alloc");
     MI_CU(ctx->p_hist.ensure((size_t)n * BM2 * 8), "alloc");
-    MI_CU(ctx->p_marg.ensure((size_t)n * 2 * Bmax * 8), "alloc");
     MI_CU(ctx->p_ment.ensure((size_t)n * nq * 2 * 8), "alloc");
     MI_CU(ctx->p_mterm.ensure((size_t)n * nq * 2 * Bmax * 8), "alloc");
     MI_CU(ctx->p_jsum.ensure((size_t)n * nq * cblocks * 8), "alloc");
@@ -1725,7 +1724,7 @@ mi_status parzen_core(mi_ctx *ctx, const std::vector<float> &prm, int n, const f
     auto *hist = ctx->p_hist.as<unsigned long long>();
     MI_CU(cudaEventRecord(ctx->ev0, s), "event");
     MI_CU(launch_parzen_hist(L, d_aff, ctx->sms, hist, cnt, s), "Parzen histogram");
-    MI_CU(launch_parzen_weights(hist, cnt, L, Q, ctx->p_marg.as<double>(), ctx->p_ment.as<double>(),
+    MI_CU(launch_parzen_weights(hist, cnt, L, Q, ctx->p_ment.as<double>(),
                                 ctx->p_mterm.as<double>(), ctx->p_jsum.as<double>(), d_mi,
                                 ctx->p_w.as<float>(), s),
           "Parzen entropies");

@@ -633,19 +633,11 @@ __device__ typename HistOf<HV>::T make_hist(unsigned char *smem, const SmemLayou
 }
 
 // ---------------------------------------------------------------------------
-// Voxel loop: warps take batches of 32 fixed rows; lane l clips row rb + l,
-// then the warp walks the 32 clipped rows 32 voxels at a time.
+// Voxel loops: warps take batches of 32 fixed rows; lane l clips the l-th,
+// then the warp walks the clipped rows.  The row blocks first_block +
+// n * block_stride, n = 0, 1, ..., below n_end are visited.
 // ---------------------------------------------------------------------------
 
-// Row order: the CTA walks blocks of nwarps adjacent fixed rows (block blk
-// holds rows blk * nwarps + w) and warp w takes row w of each block, so at any
-// time the warps of a CTA sample neighbouring moving lines (row j's upper y
-// neighbours are row j + 1's samples).  Blocks are first_block + n *
-// block_stride, n = 0, 1, ...  A warp clips its next 32 rows at once (lane l
-// takes the warp's l-th upcoming row, exactly in 64 bits), then walks them one
-// by one, 32 voxels at a time, with each row's interval broadcast by shuffles.
-// Blocks first_block + n * block_stride, n = 0, 1, ..., below n_end are
-// visited (the batched kernel passes one slab of blocks at a time).
 // The interpolated moving value at a 16.16 index, through the variant's fetch path (PairT: uint16_t for an
 // 8-bit moving volume, uint32_t for a 16-bit one).
 template <int FM, typename PairT>
@@ -732,9 +724,16 @@ __device__ void accumulate_sampled(const PairDev &P, const int *q, const float2 
     }
 }
 
+// Row walk (x-pair fetches): the CTA walks blocks of nwarps adjacent fixed rows (block blk
+// holds rows blk * nwarps + w) and warp w takes row w of each block, so at any
+// time the warps of a CTA sample neighbouring moving lines (row j's upper y
+// neighbours are row j + 1's samples).  A warp clips its next 32 rows at once (lane l
+// takes the warp's l-th upcoming row, exactly in 64 bits), then walks them one
+// by one, 32 voxels at a time, with each row's interval broadcast by shuffles.
 template <typename PairT, int FM, class Hist>
-__device__ void accumulate_rows(const PairDev &P, const int *q, const float2 *zoff, long long first_block,
-                                long long block_stride, long long n_end, Hist &H) {
+__device__ void accumulate_rows(const PairDev &P, const int *q, long long first_block, long long block_stride,
+                                long long n_end, Hist &H) {
+    static_assert(FM == FM_LDG || FM == FM_TEX, "quads and gathers take the group and stream walks");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int nf0 = P.nf[0], nf1 = P.nf[1];
     const long long R = (long long)nf1 * P.nf[2];
@@ -773,10 +772,8 @@ __device__ void accumulate_rows(const PairDev &P, const int *q, const float2 *zo
                     int v;
                     if constexpr (FM == FM_TEX)
                         v = sample_hard_tex<PairT>(P.texp, (int)U0, (int)U1, (int)U2);
-                    else if constexpr (FM == FM_LDG)
-                        v = sample_hard_pair<PairT>(movp, sy, sz, n0, sz, (int)U0, (int)U1, (int)U2);
                     else
-                        v = sample_value<FM, PairT>(P, zoff, U0, U1, U2);
+                        v = sample_hard_pair<PairT>(movp, sy, sz, n0, sz, (int)U0, (int)U1, (int)U2);
                     bm = (v * bins) >> mdepth;
                     bf = (int)__ldg(frow + i);
                 }
@@ -972,9 +969,9 @@ __device__ __forceinline__ void walk_rows(const PairDev &P, const int *q, const 
             accumulate_stream<PairT, FM>(P, q, zoff, first_block, block_stride, n_end, H);
         else
             accumulate_groups<PairT, FM>(P, q, zoff, first_block, block_stride, n_end, lpr_log2, H);
-        return;
+    } else {
+        accumulate_rows<PairT, FM>(P, q, first_block, block_stride, n_end, H);
     }
-    accumulate_rows<PairT, FM>(P, q, zoff, first_block, block_stride, n_end, H);
 }
 
 // Copies the per-plane atlas offsets of pair P into shared memory (gather fetches only).
@@ -1563,7 +1560,7 @@ cudaError_t launch_f32_to_u16(const float *in, long long n, uint16_t *out, cudaS
 // Blocks of 256 threads for n elements, eight a thread, at most eight blocks an SM.
 static int eight_grid(long long n) {
     const long long g = (n + 2047) / 2048;
-    return (int)(g < 1 ? 1 : (g > 1216 ? 1216 : g));
+    return (int)(g < 1 ? 1 : (g > 8 * 152 ? 8 * 152 : g));
 }
 
 cudaError_t launch_copy_clamp(const void *in, int dtype, int depth, long long n, void *out, cudaStream_t s) {
@@ -1624,19 +1621,16 @@ cudaError_t launch_table(double *tab, float q, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Every variant as (public value, counter kind, fetch mode): those that read x-pairs (whose element
-// type follows the moving type) and those whose texels the texture unit unpacks (one instance each).
-#define MI_VARIANTS_PAIRED(X)                                                                       \
+// Every variant as (public value, counter kind, fetch mode).
+#define MI_VARIANTS(X)                                                                              \
     X(HV_U32, HV_U32, FM_LDG) X(HV_U32_MATCH, HV_U32_MATCH, FM_LDG) X(HV_U16, HV_U16, FM_LDG)        \
     X(HV_U16_MATCH, HV_U16_MATCH, FM_LDG) X(HV_TEX + HV_U32, HV_U32, FM_TEX)                        \
     X(HV_TEX + HV_U32_MATCH, HV_U32_MATCH, FM_TEX) X(HV_TEX + HV_U16, HV_U16, FM_TEX)                \
     X(HV_TEX + HV_U16_MATCH, HV_U16_MATCH, FM_TEX) X(HV_ROWS, HV_ROWS, FM_LDG)                      \
-    X(HV_ROWS_TEX, HV_ROWS, FM_TEX)
-#define MI_VARIANTS_TEXEL(X)                                                                        \
+    X(HV_ROWS_TEX, HV_ROWS, FM_TEX)                                                                 \
     X(HV_ROWS_QUAD, HV_ROWS, FM_QUAD) X(HV_U32_QUAD, HV_U32, FM_QUAD) X(HV_U16_QUAD, HV_U16, FM_QUAD) \
     X(HV_ROWS_GATHER, HV_ROWS, FM_GATHER) X(HV_U32_GATHER, HV_U32, FM_GATHER)                       \
     X(HV_U16_GATHER, HV_U16, FM_GATHER)
-#define MI_VARIANTS(X) MI_VARIANTS_PAIRED(X) MI_VARIANTS_TEXEL(X)
 
 cudaError_t launch_entropy_slots(const uint32_t *d_hist, long long hist_stride, const Slot *d_slots, int nslots,
                                  int parts, const QSet &Q, unsigned int *d_done, double *d_part, const Outputs &O,

@@ -202,8 +202,8 @@ int parzen_cell_blocks(int B);
 // One Parzen call over n transforms: the pairs as a device array, transform t evaluated on pair
 // d_pair_of[t] (NULL: every transform on pair 0) whose fixed rows start at d_row_start[t] in the
 // sequence of all transforms' rows (NULL: t R of pair 0; n + 1 entries).  Per-transform tables take
-// slots sized for the largest bin count Bmax (histograms and W: Bmax^2 per transform and q; marginals
-// 2 Bmax), the first B^2 used with row stride B.  nx_max: the longest fixed row of the pairs.
+// slots sized for the largest bin count Bmax (histograms and W: Bmax^2 per transform and q; marginal
+// factors 2 Bmax), the first B^2 used with row stride B.  nx_max: the longest fixed row of the pairs.
 struct ParzenLaunch {
     ParzenPair p0;  // pair 0 (single-pair calls pass it by value)
     const ParzenPair *d_pairs;
@@ -221,10 +221,9 @@ struct ParzenLaunch {
 cudaError_t launch_parzen_hist(const ParzenLaunch &L, const ParzenAffine *d_aff, int sms, unsigned long long *d_hist,
                                unsigned long long *d_count, cudaStream_t s);
 // MI per q (n x nq) and the weight tables W (n x nq x Bmax^2, FP32) from the soft histograms.
-// Scratch: marg (n x 2 Bmax), ment (n x nq x 2), mterm (n x nq x 2 Bmax), jpart (n x nq x
-// parzen_cell_blocks(Bmax)) FP64.
+// Scratch: ment (n x nq x 2), mterm (n x nq x 2 Bmax), jpart (n x nq x parzen_cell_blocks(Bmax)) FP64.
 cudaError_t launch_parzen_weights(const unsigned long long *d_hist, const unsigned long long *d_count,
-                                  const ParzenLaunch &L, const QSet &Q, double *marg, double *ment, double *mterm,
+                                  const ParzenLaunch &L, const QSet &Q, double *ment, double *mterm,
                                   double *jpart, double *d_mi, float *d_w, cudaStream_t s);
 // Gradient: per-CTA moments (scratch n x nq x ctas x 12 FP64) and dMI/dtheta (n x nq x np FP64);
 // d_jac: n x 12 x np (d[A|b]/dparam about the fixed centre), np = 9 or 12.

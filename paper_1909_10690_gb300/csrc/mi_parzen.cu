@@ -454,9 +454,9 @@ __device__ __forceinline__ int bins_of(const ParzenPair *pairs, const int *pair_
     return pairs[pair_of ? pair_of[t] : 0].B;
 }
 
-// One CTA per transform: marginals P_F (rows), P_M (cols), their entropies per q, and the row and
-// column factors of W per q (mterm: n x nq x 2B): ln P for q = 1, dS_q/dP = -q P^(q-1) / (q - 1)
-// otherwise.  marg: n x 2B (P_F then P_M); ment: n x nq x 2 (S_F, S_M).
+// One CTA per transform: the entropies of the marginals P_F (rows) and P_M (cols) per q (ment: n x nq x 2,
+// S_F, S_M), and the row and column factors of W per q (mterm: n x nq x 2B): ln P for q = 1,
+// dS_q/dP = -q P^(q-1) / (q - 1) otherwise.
 // Row sums by warps along the rows (coalesced), column sums by kMargSlices row slices per column,
 // added in shared memory (integer sums: any order).  Then every (q, marginal entry) is a task of its
 // own: one ln v serves the entropy term and the factor of W for that q.  With one thread per row
@@ -467,14 +467,13 @@ constexpr int kMargThreads = 512;
 __global__ void __launch_bounds__(kMargThreads)
     k_parzen_marg(const unsigned long long *__restrict__ ghist, const unsigned long long *__restrict__ gcount,
                   const ParzenPair *__restrict__ pairs, const int *__restrict__ pair_of, int Bmax, QSet Q,
-                  double *__restrict__ marg, double *__restrict__ ment, double *__restrict__ mterm) {
+                  double *__restrict__ ment, double *__restrict__ mterm) {
     __shared__ unsigned long long s_sum[2][128];  // row and column sums (B <= 128)
     __shared__ double s_ent[kMaxQ][2][128];       // entropy terms: q, marginal, entry
     const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = bins_of(pairs, pair_of, t);
     const double N = (double)gcount[t] * 4294967296.0;  // total weight: 2^32 per overlap voxel
     const unsigned long long *h = ghist + (size_t)t * Bmax * Bmax;
-    double *pf = marg + (size_t)t * 2 * Bmax;
     for (int c = tid; c < 256; c += kMargThreads) s_sum[c >> 7][c & 127] = 0;
     __syncthreads();
     for (int r = warp; r < B; r += kMargThreads / 32) {
@@ -492,10 +491,6 @@ __global__ void __launch_bounds__(kMargThreads)
         atomicAdd(&s_sum[1][c], sc);
     }
     __syncthreads();
-    for (int x = tid; x < 2 * B; x += kMargThreads) {
-        const int m = x / B, r = x % B;
-        pf[x] = N > 0 ? (double)s_sum[m][r] / N : 0.0;
-    }
     for (int x = tid; x < 2 * B * Q.nq; x += kMargThreads) {
         const int iq = x / (2 * B), y = x % (2 * B), m = y / B, r = y % B;
         const float qf = Q.q[iq];
@@ -1055,11 +1050,11 @@ cudaError_t launch_parzen_hist(const ParzenLaunch &L, const ParzenAffine *d_aff,
 }
 
 cudaError_t launch_parzen_weights(const unsigned long long *d_hist, const unsigned long long *d_count,
-                                  const ParzenLaunch &L, const QSet &Q, double *marg, double *ment, double *mterm,
+                                  const ParzenLaunch &L, const QSet &Q, double *ment, double *mterm,
                                   double *jpart, double *d_mi, float *d_w, cudaStream_t s) {
     cudaError_t e;
     const int n = L.n;
-    k_parzen_marg<<<n, kMargThreads, 0, s>>>(d_hist, d_count, L.d_pairs, L.d_pair_of, L.Bmax, Q, marg, ment, mterm);
+    k_parzen_marg<<<n, kMargThreads, 0, s>>>(d_hist, d_count, L.d_pairs, L.d_pair_of, L.Bmax, Q, ment, mterm);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int nb = parzen_cell_blocks(L.Bmax);
     dim3 grid(nb, n);
