@@ -82,53 +82,74 @@ def _wait_for(*args):
     """Waits for the torch work that produces device inputs (and last used the memory of outputs allocated
     beside them), on every device that holds one: a context works on a stream of its own, which nothing
     orders after torch's."""
-    for dev in dict.fromkeys(a.obj.device for a in args if a.on_gpu):
-        _torch().cuda.current_stream(dev).synchronize()
+    waited = []
+    for a in args:
+        if a.on_gpu and a.obj.device not in waited:
+            waited.append(a.obj.device)
+            _torch().cuda.current_stream(a.obj.device).synchronize()
 
 
-class _Order:
-    """How one call is ordered with torch's work on its device tensors.
+class _OwnStream:
+    """How a call on the context's own stream is ordered with torch's work on its device tensors: the host
+    waits for torch's current stream."""
 
-    On the context's own stream the host waits for torch's current stream (``wait``).  On a stream the
-    caller gave, the inputs are the caller's to order and nothing is waited for: conversions and outputs
-    are made on that stream, and an output is marked as used by the caller's current stream too, so that
-    its memory is not handed out again while work queued there still reads it.
-    """
-
-    def __init__(self, given, *inputs):
-        self._given = self._caller = self._ctx = None
-        gpu = [x for x in inputs if _is_torch(x) and x.is_cuda] if given is not None else []
-        if not gpu:
-            return
-        cuda, dev = _torch().cuda, gpu[0].device
-        if not hasattr(given, "cuda_stream"):  # a raw handle
-            given = cuda.ExternalStream(given, device=dev)
-        if all(x.device == given.device for x in gpu):
-            self._given, self._caller = given, cuda.current_stream(dev)
-            self._ctx = cuda.stream(given)
+    wait = staticmethod(_wait_for)
 
     def __enter__(self):
-        if self._ctx is not None:
-            self._ctx.__enter__()
         return self
 
     def __exit__(self, *exc):
-        if self._ctx is not None:
-            self._ctx.__exit__(*exc)
-
-    def wait(self, *args):
-        if self._given is None:
-            _wait_for(*args)
+        pass
 
     def out(self, shape, like, dtype):
         """An output beside the input ``like``: a tensor on its device, or a numpy array."""
         if not like.on_gpu:
             return np.empty(shape, dtype=dtype)
         torch = _torch()
-        t = torch.empty(shape, dtype=getattr(torch, np.dtype(dtype).name), device=like.obj.device)
-        if self._given is not None and self._caller.cuda_stream != self._given.cuda_stream:
+        return torch.empty(shape, dtype=getattr(torch, np.dtype(dtype).name), device=like.obj.device)
+
+
+class _GivenStream(_OwnStream):
+    """The same on a stream the caller gave: the inputs are the caller's to order and nothing is waited for.
+    Conversions and outputs are made on that stream, and an output is marked as used by the caller's current
+    stream too, so that its memory is not handed out again while work queued there still reads it."""
+
+    def __init__(self, stream, caller):
+        self._stream, self._caller, self._ctx = stream, caller, _torch().cuda.stream(stream)
+
+    def __enter__(self):
+        self._ctx.__enter__()
+        return self
+
+    def __exit__(self, *exc):
+        self._ctx.__exit__(*exc)
+
+    def wait(self, *args):
+        pass
+
+    def out(self, shape, like, dtype):
+        t = super().out(shape, like, dtype)
+        if like.on_gpu and self._caller.cuda_stream != self._stream.cuda_stream:
             t.record_stream(self._caller)
         return t
+
+
+_OWN = _OwnStream()
+
+
+def _order(given, *inputs):
+    """The ordering of one call of a context whose set_stream stream is ``given`` (None: its own)."""
+    if given is None:
+        return _OWN
+    gpu = [x for x in inputs if _is_torch(x) and x.is_cuda]
+    if not gpu:
+        return _OWN
+    cuda, dev = _torch().cuda, gpu[0].device
+    if not hasattr(given, "cuda_stream"):  # a raw handle
+        given = cuda.ExternalStream(given, device=dev)
+    if any(x.device != given.device for x in gpu):
+        return _OWN
+    return _GivenStream(given, cuda.current_stream(dev))
 
 
 def _np_dtype(x):
@@ -281,7 +302,7 @@ class Context:
         (for a Parzen context the entropies are None: only the counts)."""
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _Order(self._given, transforms) as order:
+        with _order(self._given, transforms) as order:
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
             mi = order.out((n, nq), T, np.float64)
@@ -295,7 +316,7 @@ class Context:
     def eval_q16(self, affines, q=(1.0,), with_entropies=False, allow_empty=True):
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _Order(self._given, affines) as order:
+        with _order(self._given, affines) as order:
             A = _Arg(affines, np.int32)
             n = int(np.prod(A.obj.shape) // 12)
             mi = order.out((n, nq), A, np.float64)
@@ -309,7 +330,7 @@ class Context:
     def batch_eval(self, pair_of_transform, transforms, q=(1.0,), with_entropies=False, allow_empty=True):
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _Order(self._given, pair_of_transform, transforms) as order:
+        with _order(self._given, pair_of_transform, transforms) as order:
             P = _Arg(pair_of_transform, np.int32)
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
@@ -325,7 +346,7 @@ class Context:
         """Parzen MI (n x nq) and dMI/dparam (n x nq x nparams)."""
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _Order(self._given, transforms) as order:
+        with _order(self._given, transforms) as order:
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
             mi = order.out((n, nq), T, np.float64)
@@ -340,7 +361,7 @@ class Context:
         context: transform t on pair pair_of_transform[t], one launch per kernel for all pairs."""
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _Order(self._given, pair_of_transform, transforms) as order:
+        with _order(self._given, pair_of_transform, transforms) as order:
             P = _Arg(pair_of_transform, np.int32)
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
@@ -356,7 +377,7 @@ class Context:
         if (transforms is None) == (affines is None):
             raise ValueError("give exactly one of transforms and affines")
         B = self.bins[pair]
-        with _Order(self._given, transforms, affines) as order:
+        with _order(self._given, transforms, affines) as order:
             src = _Arg(transforms, np.float32) if transforms is not None else _Arg(affines, np.int32)
             n = int(np.prod(src.obj.shape) // (self.nparams if transforms is not None else 12))
             out = np.empty((n, B, B), dtype=np.uint32)
