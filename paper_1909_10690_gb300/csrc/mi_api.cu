@@ -1154,7 +1154,10 @@ std::vector<Choice> candidates(mi_ctx *ctx, int bins, long long nvox_max) {
 // a step.  A few transforms wait for the moving volume's first use, where the gather atlas is half the
 // quads' bytes; from kPlainQuads on its reuse weighs more and the quads' fewer instructions win.  us, gather
 // and quads: 256 x 256 x 160 at 128 bins, one transform 65 and 66, two 93 and 96, four 162 and 159, eight 262
-// and 251, 81 1990 and 1804; 256^3 at 256 bins, one 96 and 98, two 145 and 127, four 276 and 263.
+// and 251, 81 1990 and 1804; 256^3 at 256 bins, one 96 and 98, two 145 and 127, four 276 and 263.  The line is the
+// 12-bit volumes'; of bytes, whose quads take no more memory than the atlas, the quads are as fast or faster from
+// one transform on: 256 x 256 x 160 at 128 bins, one 53 and 53, two 81 and 78, four 135 and 131, 81 1616 and 1539;
+// 256^3 at 64 bins, one 82 and 71, two 124 and 110; 64^3, one to four 29 to 30 and 29 to 30.
 constexpr int kPlainQuads = 3;
 
 Choice plain_choice(mi_ctx *ctx, const std::vector<Choice> &cands, int n) {
@@ -1197,7 +1200,9 @@ enum PlanMode {
 // CTAs' mean share of what is left: all but the last ~2 P of many equal transforms stay whole
 // (P = CTAs resident at once).  A part costs its CTA the clearing and flushing of a histogram, about
 // bins^2 / 8 + 2000 voxels' time, so parts stay eight times that; a call too small for such parts
-// (below 32 of them a CTA) is cut once into equal parts, one for every CTA.
+// (below 32 of them a CTA) is cut once into equal parts, at most one for every CTA.  A part takes whole row
+// blocks (warps x rows a step: 128 rows with 1024 threads and four rows), so a transform has at most as many
+// parts as blocks (64^3: 32) and its parts differ by up to a block.
 // Against whole transforms (batched) and equal CTA counts per transform (plain), kernel times: 81 transforms on
 // 256 x 256 x 160 at 128 bins 4320 -> 1945 us, 400 sampled ones 3875 -> 2710, 768 on twelve pairs of 96^3 to
 // 320 x 320 x 200 16490 -> 13400.
