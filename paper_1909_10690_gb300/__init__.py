@@ -109,13 +109,21 @@ class _OwnStream:
         return torch.empty(shape, dtype=getattr(torch, np.dtype(dtype).name), device=like.obj.device)
 
 
-class _GivenStream(_OwnStream):
-    """The same on a stream the caller gave: the inputs are the caller's to order and nothing is waited for.
-    Conversions and outputs are made on that stream, and an output is marked as used by the caller's current
-    stream too, so that its memory is not handed out again while work queued there still reads it."""
+class _NoWait(_OwnStream):
+    """On a stream the caller gave the inputs are the caller's to order and nothing is waited for.  Torch's
+    current stream is that stream, or has no work left that could still use the outputs' memory."""
 
-    def __init__(self, stream, caller):
-        self._stream, self._caller, self._ctx = stream, caller, _torch().cuda.stream(stream)
+    def wait(self, *args):
+        pass
+
+
+class _BesideWork(_NoWait):
+    """The same beside work queued on torch's current stream: conversions and outputs are made on the given
+    stream, and an output is marked as used by the current one too, so that its memory is not handed out
+    again while work queued there still reads it."""
+
+    def __init__(self, given, caller):
+        self._caller, self._ctx = caller, _torch().cuda.stream(given)
 
     def __enter__(self):
         self._ctx.__enter__()
@@ -124,32 +132,38 @@ class _GivenStream(_OwnStream):
     def __exit__(self, *exc):
         self._ctx.__exit__(*exc)
 
-    def wait(self, *args):
-        pass
-
     def out(self, shape, like, dtype):
         t = super().out(shape, like, dtype)
-        if like.on_gpu and self._caller.cuda_stream != self._stream.cuda_stream:
+        if like.on_gpu:
             t.record_stream(self._caller)
         return t
 
 
-_OWN = _OwnStream()
+_OWN, _NO_WAIT = _OwnStream(), _NoWait()
 
 
 def _order(given, *inputs):
-    """The ordering of one call of a context whose set_stream stream is ``given`` (None: its own)."""
+    """The ordering of one call of a context whose set_stream stream is ``given`` (None: its own); inputs:
+    (array or tensor, dtype it is read as)."""
     if given is None:
         return _OWN
-    gpu = [x for x in inputs if _is_torch(x) and x.is_cuda]
-    if not gpu:
+    dev, as_is = None, True
+    for x, dtype in inputs:
+        if _is_torch(x) and x.is_cuda:
+            dev = dev or x.device
+            as_is = as_is and x.device == dev and x.element_size() == 4 and x.is_contiguous() \
+                and x.dtype == getattr(_torch(), dtype)
+    if dev is None:
         return _OWN
-    cuda, dev = _torch().cuda, gpu[0].device
-    if not hasattr(given, "cuda_stream"):  # a raw handle
-        given = cuda.ExternalStream(given, device=dev)
-    if any(x.device != given.device for x in gpu):
+    cuda = _torch().cuda
+    caller, handle = cuda.current_stream(dev), getattr(given, "cuda_stream", given)
+    if as_is and (caller.cuda_stream == handle or caller.query()):
+        return _NO_WAIT
+    if any(x.device != getattr(given, "device", dev) for x, _ in inputs if _is_torch(x) and x.is_cuda):
         return _OWN
-    return _GivenStream(given, cuda.current_stream(dev))
+    if caller.cuda_stream == handle:
+        return _NO_WAIT
+    return _BesideWork(given if given is not handle else cuda.ExternalStream(handle, device=dev), caller)
 
 
 def _np_dtype(x):
@@ -302,7 +316,7 @@ class Context:
         (for a Parzen context the entropies are None: only the counts)."""
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _order(self._given, transforms) as order:
+        with _order(self._given, (transforms, "float32")) as order:
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
             mi = order.out((n, nq), T, np.float64)
@@ -316,7 +330,7 @@ class Context:
     def eval_q16(self, affines, q=(1.0,), with_entropies=False, allow_empty=True):
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _order(self._given, affines) as order:
+        with _order(self._given, (affines, "int32")) as order:
             A = _Arg(affines, np.int32)
             n = int(np.prod(A.obj.shape) // 12)
             mi = order.out((n, nq), A, np.float64)
@@ -330,7 +344,7 @@ class Context:
     def batch_eval(self, pair_of_transform, transforms, q=(1.0,), with_entropies=False, allow_empty=True):
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _order(self._given, pair_of_transform, transforms) as order:
+        with _order(self._given, (pair_of_transform, "int32"), (transforms, "float32")) as order:
             P = _Arg(pair_of_transform, np.int32)
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
@@ -346,7 +360,7 @@ class Context:
         """Parzen MI (n x nq) and dMI/dparam (n x nq x nparams)."""
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _order(self._given, transforms) as order:
+        with _order(self._given, (transforms, "float32")) as order:
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
             mi = order.out((n, nq), T, np.float64)
@@ -361,7 +375,7 @@ class Context:
         context: transform t on pair pair_of_transform[t], one launch per kernel for all pairs."""
         Q = _Arg(np.atleast_1d(np.asarray(q, dtype=np.float32)))
         nq = int(np.asarray(q).size)
-        with _order(self._given, pair_of_transform, transforms) as order:
+        with _order(self._given, (pair_of_transform, "int32"), (transforms, "float32")) as order:
             P = _Arg(pair_of_transform, np.int32)
             T = _Arg(transforms, np.float32)
             n = int(np.prod(T.obj.shape) // self.nparams)
@@ -377,7 +391,7 @@ class Context:
         if (transforms is None) == (affines is None):
             raise ValueError("give exactly one of transforms and affines")
         B = self.bins[pair]
-        with _order(self._given, transforms, affines) as order:
+        with _order(self._given, (transforms, "float32"), (affines, "int32")) as order:
             src = _Arg(transforms, np.float32) if transforms is not None else _Arg(affines, np.int32)
             n = int(np.prod(src.obj.shape) // (self.nparams if transforms is not None else 12))
             out = np.empty((n, B, B), dtype=np.uint32)
