@@ -45,10 +45,10 @@ DESIGN_OPS_PER_VOXT = 50
 # kernel source and the selected configuration are the ones measured: DRAM bytes of one full launch
 # (4096 transforms), and from a one-wave capture the issue and L1TEX utilisation and the
 # shared-memory wavefronts per shared atomic instruction.
-K_BATCHED_NCU = {"source_sha16": "3c94ed9a7ce37b1f", "config": [10, 4, 2],
-                 "dram_bytes_per_launch": 255594189568 + 10100736, "issue_active": 0.847,
-                 "l1tex_throughput": 0.844, "smem_wavefronts_per_atomic": 342238278 / 66419779,
-                 "smem_atomic_wavefronts_per_sm_cycle": 342238278 / 152 / 10787757.87,
+K_BATCHED_NCU = {"source_sha16": "51fe965b2279b42d", "config": [10, 4, 2],
+                 "dram_bytes_per_launch": 261380626688 + 10700032, "issue_active": 0.847,
+                 "l1tex_throughput": 0.844, "smem_wavefronts_per_atomic": 342236497 / 66419779,
+                 "smem_atomic_wavefronts_per_sm_cycle": 342236497 / 152 / 10701467.89,
                  "profile": "profiles/k_batched_rows_quad_256cubed_256bins.md"}
 # algorithmic FP32 operations per voxel x transform of the Parzen MI + gradient at 3 q values:
 # forward 31 (trilinear 14, bin coordinate 1, B-spline weights 12, 4 increments),
@@ -57,9 +57,9 @@ PARZEN_OPS_PER_VOXT = 120
 # Counters of the Parzen forward (k_parzen_hist) from one ncu capture of the 50-pose call (see profiles/),
 # reported while the kernel source is the one measured: shared-atomic instructions and wavefronts, SM
 # cycles elapsed per launch, and the DRAM bytes read and written by the forward and the adjoint
-K_PARZEN_NCU = {"source_sha16": "010ce02ddcf24dcd", "atom_inst": 52167744, "atom_wavefronts": 242416278,
-                "sm_cycles_elapsed": 2050648.05, "time_ms": 0.9954,
-                "dram_bytes_per_call": 416288512 + 4498944 + 26232320,
+K_PARZEN_NCU = {"source_sha16": "89720ea9f0f4a1e8", "atom_inst": 52167744, "atom_wavefronts": 242397249,
+                "sm_cycles_elapsed": 2048670.64, "time_ms": 0.9918,
+                "dram_bytes_per_call": 419462912 + 4554752 + 26234368,
                 "profile": "profiles/parzen_fwd_adj_192x192x128_64bins.md"}
 PARZEN_SHAPE = (128, 192, 192)
 PARZEN_SPACING = (1.0, 1.0, 1.2)
