@@ -1101,7 +1101,8 @@ __device__ void write_mi(uint32_t N, double S, const QSet &Q, long long t, const
 // and FP64 instructions issued with full warps: most cells hold small counts, which are only counted
 // (small[c] = number of cells that hold c < kSmallCounts, an integer atomic) and enter the sums as one
 // product per count; counts below the table's end are looked up on the way; the few beyond it are listed
-// and taken side by side at the end.  One addition per cell and q, in a pass
+// and taken side by side at the end, largest first: warps list them in whatever order they come by, and sums that
+// followed it differed from call to call.  One addition per cell and q, in a pass
 // per q, with every thread adding every warp's partial sums and log / pow beyond the table, was 4 % of the
 // batched kernel at 256 bins and four q (with the split tail, 4096 transforms of 256^3: 168.3 -> 163.6 ms a call).
 constexpr int kSmallCounts = 768;
@@ -1127,13 +1128,33 @@ struct CountTable {
         }
         if (v < kBig) return false;
         const uint32_t i = atomicAdd(nbig(), 1u);
-        if (i >= (uint32_t)kBigCounts) return false;
-        big()[i] = v;
+        if (i < (uint32_t)kBigCounts) big()[i] = v;
         return true;
     }
-    // The same answer for a pass after the first (which lists large counts if there is room for all).
+    // After the pass that took the counts: more large ones than the list holds.  Which of them it holds depends on
+    // the warps' order, so it is not used: the caller repeats the pass and adds every large count's terms.
+    __device__ __forceinline__ bool overflowed() const { return small && *nbig() > (uint32_t)kBigCounts; }
+    // Orders the list by value (the whole CTA; each entry counts those before it).
+    __device__ void sort() {
+        const int n = small ? (int)*nbig() : 0, tid = threadIdx.x;
+        if (n < 2) return;  // (the same for every thread)
+        uint32_t v = 0;
+        int rank = 0;
+        if (tid < n) {
+            v = big()[tid];
+#pragma unroll 4
+            for (int j = 0; j < n; ++j) {
+                const uint32_t w = big()[j];
+                rank += w > v || (w == v && j < tid);
+            }
+        }
+        __syncthreads();
+        if (tid < n) big()[rank] = v;
+        __syncthreads();
+    }
+    // take's answer for a pass after the first.
     __device__ __forceinline__ bool taken_before(uint32_t v) const {
-        return small && (v < (uint32_t)kSmallCounts || (v >= kBig && *nbig() <= (uint32_t)kBigCounts));
+        return small && (v < (uint32_t)kSmallCounts || (v >= kBig && !overflowed()));
     }
     // This thread's share of the table's terms of q0 .. q0 + 3.
     __device__ __forceinline__ void add_terms(double (&a)[4], int q0, const QSet &Q) const {
@@ -1150,8 +1171,7 @@ struct CountTable {
                 for (int k = 0; k < 4; ++k) a[k] = fma(dm, tv[k], a[k]);
             }
         }
-        // when the list overflowed, the passes after the first take every large count on the way
-        const int n = (int)*nbig() <= kBigCounts ? (int)*nbig() : (q0 == 0 ? kBigCounts : 0);
+        const int n = overflowed() ? 0 : (int)*nbig();
         for (int i = threadIdx.x; i < n; i += blockDim.x) add_count(a, big()[i], q0, Q);
     }
     __device__ __forceinline__ static void add_count(double (&a)[4], uint32_t v, int q0, const QSet &Q) {
@@ -1173,6 +1193,7 @@ __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *
     C.zero();
     __syncthreads();
     // four q per pass over the cells: the accumulators of more would spill
+    bool first = true;  // the pass that takes the counts
     for (int q0 = 0; q0 < nq; q0 += 4) {
         double aj[4] = {0.0, 0.0, 0.0, 0.0};
         for (int r = warp; r < B; r += nwarps) {
@@ -1181,7 +1202,7 @@ __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *
                 const uint32_t v = H.count(r, c);
                 if (v == 0) continue;
                 bool taken;
-                if (q0 == 0) {
+                if (first) {
                     rsum += v;
                     atomicAdd(&s_cols[c], v);
                     taken = C.take(v);
@@ -1190,12 +1211,20 @@ __device__ void reduce_entropies(const Hist &H, int B, const QSet &Q, uint32_t *
                 }
                 if (!taken) CountTable<16>::add_count(aj, v, q0, Q);
             }
-            if (q0 == 0) {
+            if (first) {
                 rsum = __reduce_add_sync(kFull, rsum);
                 if (lane == 0) s_rows[r] = rsum;
             }
         }
         __syncthreads();
+        if (first) {
+            first = false;
+            if (C.overflowed()) {  // the first four q again, large counts on the way
+                q0 -= 4;
+                continue;
+            }
+            C.sort();
+        }
         C.add_terms(aj, q0, Q);
         // joint sums: the upper 16 warps' into the lower 16; marginals: up to 64 entries a warp, warps
         // 0..3 the rows and 4..7 the columns; then warp 0 takes lane = 4 j + k for q0 + k
@@ -1286,9 +1315,10 @@ __global__ void __launch_bounds__(kEntThreads, 4)
     s_cols[tid] = 0;
     C.zero();
     __syncthreads();
+    bool first = true;  // the pass that takes the counts
     for (int q0 = 0; q0 < nq; q0 += 4) {
         double aj[4] = {0.0, 0.0, 0.0, 0.0};
-        if (q0 == 0 && parts > 1)  // the column share; with one part the row pass meets every column
+        if (first && parts > 1)  // the column share; with one part the row pass meets every column
             for (int x = tid; x < B * ncols; x += kEntThreads) {
                 const uint32_t v = __ldcg(h + (size_t)(x / ncols) * B + c0 + x % ncols);
                 if (v) atomicAdd(&s_cols[x % ncols], v);
@@ -1302,7 +1332,7 @@ __global__ void __launch_bounds__(kEntThreads, 4)
             for (int k = 0; k < 8; ++k) {
                 if (v[k] == 0) continue;
                 bool taken;
-                if (q0 == 0) {
+                if (first) {
                     rsum += v[k];
                     if (parts == 1) atomicAdd(&s_cols[lane + 32 * k], v[k]);
                     taken = C.take(v[k]);
@@ -1311,12 +1341,20 @@ __global__ void __launch_bounds__(kEntThreads, 4)
                 }
                 if (!taken) CountTable<TB>::add_count(aj, v[k], q0, Q);
             }
-            if (q0 == 0) {
+            if (first) {
                 rsum = __reduce_add_sync(kFull, rsum);
                 if (lane == 0) s_rows[i] = rsum;
             }
         }
         __syncthreads();
+        if (first) {
+            first = false;
+            if (C.overflowed()) {  // the first four q again, large counts on the way
+                q0 -= 4;
+                continue;
+            }
+            C.sort();
+        }
         // marginal entries: warps 0..3 the rows, 4..7 the columns
         const uint32_t *line = warp < 4 ? s_rows : s_cols;
         const int nline = warp < 4 ? nrows : ncols;
