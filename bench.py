@@ -45,10 +45,10 @@ DESIGN_OPS_PER_VOXT = 50
 # kernel source and the selected configuration are the ones measured: DRAM bytes of one full launch
 # (4096 transforms), and from a one-wave capture the issue and L1TEX utilisation and the
 # shared-memory wavefronts per shared atomic instruction.
-K_BATCHED_NCU = {"source_sha16": "51fe965b2279b42d", "config": [10, 4, 2],
-                 "dram_bytes_per_launch": 261380626688 + 10700032, "issue_active": 0.847,
-                 "l1tex_throughput": 0.844, "smem_wavefronts_per_atomic": 342236497 / 66419779,
-                 "smem_atomic_wavefronts_per_sm_cycle": 342236497 / 152 / 10701467.89,
+K_BATCHED_NCU = {"source_sha16": "31d4f6fd6ae9c7af", "config": [10, 4, 2],
+                 "dram_bytes_per_launch": 251704813312 + 13494272, "issue_active": 0.843,
+                 "l1tex_throughput": 0.846, "smem_wavefronts_per_atomic": 342080054 / 66419779,
+                 "smem_atomic_wavefronts_per_sm_cycle": 342080054 / 152 / 10778931.51,
                  "profile": "profiles/k_batched_rows_quad_256cubed_256bins.md"}
 # algorithmic FP32 operations per voxel x transform of the Parzen MI + gradient at 3 q values:
 # forward 31 (trilinear 14, bin coordinate 1, B-spline weights 12, 4 increments),
